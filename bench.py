@@ -560,20 +560,12 @@ def run_gpu(args):
         wev[k][1].record(stream)
         flush_l2(stream)                                # between steps, outside the steps' events
     # ... then K joins as the four calls, with events between the kernels (the per-kernel split),
-    # each followed (after an L2 flush) by the probe of the same table as one call, whose kernel
-    # computes S's signatures and probes in one pass (the whole join's pass over S), and by the
-    # build without given signatures, whose kernel computes R's signatures and inserts them (the
-    # whole join's pass over R, the table clear included)
-    fev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
+    # each followed (after an L2 flush) by the build without given signatures, whose kernel computes
+    # R's signatures and inserts them (the whole join's pass over R, the table clear included)
     bev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
-    fcount = torch.zeros(1, dtype=torch.int64, device="cuda")
     table_cap = 0
     for k in range(args.steps):
-        t_k = step(ev[k])
-        flush_l2(stream)
-        fev[k][0].record(stream)
-        ag.join_probe(t_k, dS, pairs, fcount, sigS_out=sigS, sync=False, stream=stream)
-        fev[k][1].record(stream)
+        step(ev[k])
         flush_l2(stream)
         bev[k][0].record(stream)
         table_cap = int(ag.join_build(dR, ws[:tb], lf, stream=stream).cap)
@@ -827,22 +819,17 @@ def run_gpu(args):
                    + total_pairs * (16 + 4 + 8)                        # offR pair, idR, output pair
                    + 2 * verified_bytes),                              # R and S key bytes compared
     }
-    fused = n >= FUSED_PROBE_FROM                       # the whole join's S pass is one kernel
     # the whole join's R pass: signatures and inserts in one kernel, after the table clear
     phase_ms["sig_build_R"] = [a.elapsed_time(b) for a, b in bev]
     alg["sig_build_R"] = wl.R.nbytes + 8 * (m + 1) + 8 * m + 16 * m + 16 * table_cap
     phases = PH + ("sig_build_R",)
-    if fused:                                          # its time from the probe calls after the split steps
-        phase_ms["sig_probe_S"] = [a.elapsed_time(b) for a, b in fev]
-        alg["sig_probe_S"] = alg["sig_S"] + alg["verify"]
-        phases = phases + ("sig_probe_S",)
     kernels = {}
     for ph in phases:
         avg = statistics.mean(phase_ms[ph])
         kernels[ph] = {"ms": avg, "algorithmic_bytes": alg[ph], "gbps": alg[ph] / (avg * 1e-3) / 1e9,
                        "frac_hbm": alg[ph] / (avg * 1e-3) / 1e9 / hbm}
-    # the dominant kernel of the timed step: the fused S pass, or the larger of the S signatures and the probe
-    dom = "sig_probe_S" if fused else max(("sig_S", "verify"), key=lambda ph: kernels[ph]["ms"])
+    # the dominant kernel of the timed step: the larger of the S signatures and the probe
+    dom = max(("sig_S", "verify"), key=lambda ph: kernels[ph]["ms"])
     traffic = None
     tp = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(tp):
@@ -850,7 +837,7 @@ def run_gpu(args):
             d = json.load(f)
         ent = d.get(KERNEL_NAMES[dom], {})
         if ent.get("kernel_rev") == KERNEL_REVS[KERNEL_NAMES[dom]] and ent.get("per_byte_of_keys"):
-            keyb = wl.S.nbytes if dom in ("sig_S", "sig_probe_S") else 2 * verified_bytes
+            keyb = wl.S.nbytes if dom == "sig_S" else 2 * verified_bytes
             traffic = ent["per_byte_of_keys"] * keyb
 
     extra = {}
@@ -896,7 +883,7 @@ def run_gpu(args):
                 "h2d_pinned_gbs": h2d_gbs,
                 "copy_bound_ms": (h2d + d2h) / (h2d_gbs * 1e9) * 1e3,
                 "path": "stream.HostStreamJoin: pinned host R and S, S copied in chunks under the kernels"},
-        "gpu_launches": (2 if fused else 3) * args.steps,
+        "gpu_launches": 3 * args.steps,
         "roofline": {"bound": "hbm", "kernel": KERNEL_NAMES[dom], "achieved": kernels[dom]["gbps"], "peak": hbm,
                      "peak_kind": f"{peak_kind} (copy bandwidth, burst)", "unit": "GB/s",
                      "frac": kernels[dom]["frac_hbm"], "traffic": traffic,
@@ -925,11 +912,9 @@ def run_gpu(args):
 
 
 # revision of each kernel's code; profiles/traffic.json holds counters per revision
-KERNEL_REVS = {"sig_key_kernel": "v4", "build_kernel": "v8", "verify_kernel": "v17", "sig_key_kernel+probe": "v2",
-               "sig_key_kernel+build": "v1"}
+KERNEL_REVS = {"sig_key_kernel": "v5", "build_kernel": "v8", "verify_kernel": "v17", "sig_key_kernel+build": "v2"}
 KERNEL_NAMES = {"sig_R": "sig_key_kernel", "sig_S": "sig_key_kernel", "build": "build_kernel",
-                "verify": "verify_kernel", "sig_probe_S": "sig_key_kernel+probe", "sig_build_R": "sig_key_kernel+build"}
-FUSED_PROBE_FROM = 1 << 19    # S keys from which the library's probe computes signatures and probes in one kernel
+                "verify": "verify_kernel", "sig_build_R": "sig_key_kernel+build"}
 
 
 def main():

@@ -44,7 +44,7 @@
  * Streams: every call is asynchronous on the given stream (a cudaStream_t
  * passed as void*, NULL = legacy default stream) unless it is given a host
  * pointer to return a count, in which case it synchronises that stream.
- * as_join (below 2^19 S keys), as_join_batch_run and as_baseline_join run
+ * as_join, as_join_batch_run and as_baseline_join run
  * S's signatures (or hashes) on a side stream of the library (four per
  * device, created with the tables) forked from the given stream and joined
  * back into it before the probe, so that they overlap R's signatures and the
@@ -233,9 +233,7 @@ size_t as_join_probe_ws_bytes(uint64_t n);
  * S's signatures are computed first (as by as_sig_compute); then every S key
  * walks its bucket sequence until an empty slot; a slot is a candidate when
  * its signature and key length equal the S key's, and a candidate is emitted
- * only if the R key's bytes equal the S key's bytes.  From 2^19 S keys the
- * two steps run as one kernel (each group of 32 keys is probed and verified
- * right after its signatures), with the same result.
+ * only if the R key's bytes equal the S key's bytes.
  *   t              : table from as_join_build (host struct)
  *   d_arenaS, d_offS, d_idS, n : relation S
  *   d_sigS_out     : uint64[n] device buffer to receive S's signatures, or NULL
@@ -332,10 +330,8 @@ size_t as_join_ws_bytes(uint64_t m, uint64_t n, float load_factor);
  * Arguments as for as_join_build and as_join_probe; d_ws must hold
  * as_join_ws_bytes(m, load_factor) bytes.  d_count may be NULL (the counter
  * then lives in the workspace).  R's signatures and the build are one kernel.
- * From 2^19 S keys it is as_join_build then as_join_probe (whose signatures
- * and probe then run as one kernel too: one pass over each relation's keys);
- * below that, S's signatures overlap R's pass on a side stream.  The result is
- * the same either way.
+ * S's signatures run on a side stream, beside R's pass where that leaves SMs
+ * idle.
  */
 as_status as_join(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_t* d_idR, uint64_t m,
                   const uint8_t* d_arenaS, const uint64_t* d_offS, const uint32_t* d_idS, uint64_t n,

@@ -181,7 +181,7 @@ namespace algsig {
 // device decides whether the tables can be addressed at the fixed 0x400).
 __device__ uint32_t g_dyn_smem_base;
 __global__ void dyn_smem_base_kernel() {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   if (threadIdx.x == 0) g_dyn_smem_base = (uint32_t)__cvta_generic_to_shared(smem);
 }
 
@@ -251,16 +251,13 @@ __global__ void build_kernel(Slot* __restrict__ slots, uint64_t mask, const uint
 // lane inserts its key.  The probe runs in a later kernel, so it never sees a
 // slot whose signature word is not yet written.
 struct BuildPost {
-  static constexpr size_t kScratch = 0;
   Slot* slots;
   uint64_t mask;
   const uint64_t* offR;
   uint32_t* flags;
-  __device__ __forceinline__ void init(uint8_t*, const uint4*) {}
   __device__ __forceinline__ void group(uint64_t kq, uint64_t sig, bool valid) {
     if (valid) table_insert(slots, mask, sig, __ldg(offR + kq + 1) - __ldg(offR + kq), kq, flags);
   }
-  __device__ __forceinline__ void finish() {}
 };
 
 // ----------------------------------------------------------------------------
@@ -400,9 +397,6 @@ __device__ __forceinline__ void realign_r(const uint4& ra, const uint4& rb, uint
 // so a key of up to 1 KB costs one memory round trip.  Only aligned chunks
 // that hold a key byte are read; only the steps that hold the key's first or
 // last byte apply byte masks.
-// (emask[kMS * e] holds the mask of e bytes: kMS = 2 reads the first halves of
-// the signature kernel's 32-byte block masks)
-template <int kMS = 1>
 __device__ __forceinline__ bool warp_equal(const uint8_t* __restrict__ pR, const uint8_t* __restrict__ pS,
                                            uint32_t len, const uint4* __restrict__ emask) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -435,7 +429,7 @@ __device__ __forceinline__ bool warp_equal(const uint8_t* __restrict__ pR, const
       if ((hb == 0u && sa != 0u) || hb + 512u > kend) {   // warp-uniform: the key's first or last byte
         const uint32_t lo = off < sa ? sa - off : 0u;
         const uint32_t hi = off < kend ? (kend - off < 16u ? kend - off : 16u) : 0u;
-        const uint4 mh = emask[kMS * hi], ml = emask[kMS * lo];
+        const uint4 mh = emask[hi], ml = emask[lo];
         x0 &= mh.x & ~ml.x; x1 &= mh.y & ~ml.y; x2 &= mh.z & ~ml.z; x3 &= mh.w & ~ml.w;
       }
       diff |= x0 | x1 | x2 | x3;
@@ -638,107 +632,6 @@ __global__ void __launch_bounds__(kVThreads, 4) verify_kernel(VerifyParams P) {
   }
 }
 
-// The probe of the whole join fused into the signature kernel over S (plain
-// inner join of one table): after a group of 32 keys has its signatures, the
-// warp walks the table for each key and verifies the candidates as
-// verify_kernel does, while the key bytes it has just streamed may still sit
-// in L2.  Pairs are staged per warp in the kernel's shared scratch.
-struct ProbePost {
-  static constexpr size_t kScratch = sizeof(Stage);
-  VerifyParams P;
-  Stage* st;
-  const uint4* mt;                                   // 32-byte block masks: row e keeps bytes [0, e)
-  uint32_t np;
-  __device__ __forceinline__ void init(uint8_t* scratch, const uint4* masks) {
-    st = reinterpret_cast<Stage*>(scratch);
-    mt = masks;
-    np = 0;
-  }
-  __device__ __forceinline__ void group(uint64_t kq, uint64_t sig, bool valid) {
-    const int lane = threadIdx.x & 31;
-    bool live = valid;
-    uint64_t start = 0, len = 0, b = 0, steps = 0;
-    uint32_t l32 = 0;
-    if (live) {
-      start = __ldg(P.offS + kq);
-      len = __ldg(P.offS + kq + 1) - start;
-      b = sig_hash(sig, len) & P.mask;
-      l32 = len32(len);
-    }
-    while (__any_sync(kFull, live)) {
-      bool cand = false;
-      uint32_t row = 0;
-      if (live) {
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(P.slots + b));
-        if (v.y == kEmpty) {
-          live = false;
-        } else {
-          if (v.x == sig && (uint32_t)(v.y >> 32) == l32) {
-            cand = true;
-            row = (uint32_t)v.y;
-          }
-          b = (b + 1) & P.mask;
-          if (++steps > P.mask) live = false;
-          if (!cand && live && (b & 1u)) {         // the other slot of the 32-byte sector
-            const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2*>(P.slots + b));
-            if (v2.y == kEmpty) {
-              live = false;
-            } else {
-              if (v2.x == sig && (uint32_t)(v2.y >> 32) == l32) {
-                cand = true;
-                row = (uint32_t)v2.y;
-              }
-              b = (b + 1) & P.mask;
-              if (++steps > P.mask) live = false;
-            }
-          }
-        }
-      }
-      uint32_t cm = __ballot_sync(kFull, cand);
-      while (cm) {                                   // candidates one by one, whole warp
-        const int j = __ffs(cm) - 1;
-        cm &= cm - 1;
-        const uint32_t rj = __shfl_sync(kFull, row, j);
-        const uint32_t lj = __shfl_sync(kFull, l32, j);
-        const uint64_t stj = __shfl_sync(kFull, start, j);
-        if (cm) {                                    // the next candidate's S bytes and R offset, ahead
-          const int j2 = __ffs(cm) - 1;
-          const uint64_t st2 = __shfl_sync(kFull, start, j2);
-          const uint32_t l2 = __shfl_sync(kFull, l32, j2);
-          const uint32_t r2 = __shfl_sync(kFull, row, j2);
-          const uint64_t o = 32u * (uint64_t)lane;
-          if (o < (uint64_t)l2) asm volatile("prefetch.global.L1 [%0];" ::"l"(P.arenaS + st2 + o));
-          if (lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(P.offR + r2));
-        }
-        const uint64_t rs = __ldg(P.offR + rj);
-        bool eq;
-        if (lj < kNarrowLen) {
-          eq = warp_equal<2>(P.arenaR + rs, P.arenaS + stj, lj, mt);
-        } else {
-          const uint64_t ls = __shfl_sync(kFull, len, j);
-          const uint64_t lr = __ldg(P.offR + rj + 1) - rs;
-          eq = lr == ls && warp_equal_wide(P.arenaR, rs, P.arenaS, stj, ls);
-        }
-        if (eq) {
-          const uint64_t srow = __shfl_sync(kFull, kq, j);
-          if (lane == 0) {
-            st->r[np] = rj;
-            st->s[np] = srow;
-          }
-          __syncwarp();
-          if (++np == (uint32_t)kVStage) {
-            flush_stage(*st, np, P);
-            np = 0;
-          }
-        }
-      }
-    }
-  }
-  __device__ __forceinline__ void finish() {
-    if (np) flush_stage(*st, np, P);
-  }
-};
-
 // The R-side output modes' rows: one (r_id, AS_NO_ROW) per R row whose bit in
 // `matched` is `want` (1: semi-join rows, 0: anti-join / outer-join rows),
 // appended to the pairs after those of the probe.  One warp per 32 rows: a
@@ -783,7 +676,7 @@ constexpr size_t kSmemBHash = (size_t)kWarpsPerBlock * 2 * kBBufBytes;
 __global__ void __launch_bounds__(kThreads, 1) bl_hash_kernel(const uint8_t* __restrict__ arena,
                                                               const uint64_t* __restrict__ off, uint64_t n,
                                                               uint64_t* __restrict__ hash_out) {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   uint8_t* bufs = smem + (size_t)wib * 2 * kBBufBytes;
@@ -985,11 +878,11 @@ static cudaError_t key_kernel_attrs() {
   return e;
 }
 template <bool AT400, int NCOMP, int SHAPE, bool BATCH>
-static void key_kernel_launch(int sms, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
+static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
                               const BatchJoin* J, int nj, int s_side, cudaStream_t s) {
   constexpr LKShape k = kLKShapes[SHAPE];
-  const uint64_t want = (n + 32ull * k.warps - 1) / (32ull * k.warps);
-  const unsigned blocks = (unsigned)(want < (uint64_t)sms ? (want < 1 ? 1 : want) : (uint64_t)sms);
+  const uint64_t want = (n + 31) / 32;               // a group of 32 keys per block, until every SM has one
+  const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
   sig_key_kernel<AT400, NCOMP, k.warps, k.depth, BATCH>
       <<<blocks, 32 * k.warps, lk_smem_bytes(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side);
 }
@@ -1063,6 +956,19 @@ static as_status ensure_device(DeviceState** out) {
       }
     }
     if ((e = cudaMemcpyToSymbol(g_const, h_const, sizeof(h_const))) != cudaSuccess) return cuda_fail(e, "table setup");
+    {  // the signature kernel's constant-multiply tables (quotient.cuh)
+      static uint16_t h_inv[2 * kInvEntries];
+      for (int t = 0; t < 2 * kInvTables; t++) {
+        const int k = t % kInvTables / 2 + 1, h = t % 2;
+        const int ex = 8 * k * h - (t < kInvTables ? kQExp : kXExp)[k - 1];
+        const uint32_t C = h_alog[((int)kOrder + ex) % (int)kOrder];
+        for (uint32_t b = 0; b < 256; b++) {
+          h_inv[t * 512 + b] = (uint16_t)mul(b, C);
+          h_inv[t * 512 + 256 + b] = (uint16_t)mul(mul(b, h_alog[8]), C);
+        }
+      }
+      if ((e = cudaMemcpyToSymbol(g_inv, h_inv, sizeof(h_inv))) != cudaSuccess) return cuda_fail(e, "table setup");
+    }
     {  // the reduction tables' shared-memory image: row b, word l: T16[b] (l < 32), T24[b] (l >= 32)
       static uint32_t h_red[kRedWords];
       for (uint32_t b = 0; b < 256; b++) {
@@ -1099,20 +1005,13 @@ static as_status ensure_device(DeviceState** out) {
         return cuda_fail(e, "kernel attribute");
       {
         constexpr LKShape k = kLKShapes[0];
-        const int smem = (int)lk_smem_bytes(k.warps, k.depth, ProbePost::kScratch);
-        const int smem_b = (int)lk_smem_bytes(k.warps, k.depth, BuildPost::kScratch);
+        const int smem = (int)lk_smem_bytes(k.warps, k.depth);
         if ((e = cudaFuncSetAttribute(
-                 reinterpret_cast<const void*>(sig_key_kernel<true, 4, k.warps, k.depth, false, ProbePost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(
-                 reinterpret_cast<const void*>(sig_key_kernel<false, 4, k.warps, k.depth, false, ProbePost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(
                  reinterpret_cast<const void*>(sig_key_kernel<true, 4, k.warps, k.depth, false, BuildPost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem_b)) != cudaSuccess ||
+                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(
                  reinterpret_cast<const void*>(sig_key_kernel<false, 4, k.warps, k.depth, false, BuildPost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem_b)) != cudaSuccess)
+                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
           return cuda_fail(e, "kernel attribute");
       }
     }
@@ -1195,18 +1094,19 @@ static bool table_geometry(uint64_t m, float lf, uint64_t* cap, uint32_t* log2ca
 }
 
 static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out, cudaStream_t s,
-                            int ncomp = 4, int shape = 0) {
+                            int ncomp = 4, int shape = 0, int max_blocks = 0) {
   DeviceState* d = nullptr;
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
+  if (max_blocks <= 0) max_blocks = d->sms;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
   if (ncomp == 2) {
-    if (d->tables_at400) key_kernel_launch_shape<true, 2, false>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
-    else key_kernel_launch_shape<false, 2, false>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
+    else key_kernel_launch_shape<false, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
   } else {
-    if (d->tables_at400) key_kernel_launch_shape<true, 4, false>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
-    else key_kernel_launch_shape<false, 4, false>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
+    else key_kernel_launch_shape<false, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
@@ -1226,60 +1126,11 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
   return AS_OK;
 }
 
-// S relations from this many keys take the fused pass in as_join_probe and as_join
-// (measured: 1.5-4 % faster at 1M to 10M keys; for 100k keys as_join's side-stream
-// overlap wins)
-constexpr uint64_t kFusedProbeFrom = 1ull << 19;
-
-// The whole join's pass over S: the signature kernel (shape 0) with the probe
-// of table t fused in (ProbePost; plain inner join).
-static as_status launch_sig_probe(const DeviceState* d, const as_table* t, const uint8_t* arenaS,
-                                  const uint64_t* offS, const uint32_t* idS, uint64_t n, uint64_t* sigS,
-                                  uint32_t* pairs, uint64_t cap_pairs, uint64_t* count, cudaStream_t s) {
-  if (n == 0) return AS_OK;
-  ProbePost post;
-  VerifyParams& P = post.P;
-  P.slots = reinterpret_cast<const Slot*>(t->slots);
-  P.mask = t->cap - 1;
-  P.arenaR = t->arenaR;
-  P.offR = t->offR;
-  P.idR = t->idR;
-  P.arenaS = arenaS;
-  P.offS = offS;
-  P.idS = idS;
-  P.sigS = sigS;
-  P.n = n;
-  P.pairs = pairs;
-  P.cap = cap_pairs;
-  P.count = reinterpret_cast<unsigned long long*>(count);
-  P.mode = AS_JOIN_INNER;
-  P.matched = nullptr;
-  P.J = nullptr;
-  P.nj = 0;
-  P.counts = nullptr;
-  P.cap_len = ~0ull;
-  post.st = nullptr;
-  post.mt = nullptr;
-  post.np = 0;
-  constexpr LKShape k = kLKShapes[0];
-  const uint64_t want = (n + 32ull * k.warps - 1) / (32ull * k.warps);
-  const unsigned blocks = (unsigned)(want < (uint64_t)d->sms ? (want < 1 ? 1 : want) : (uint64_t)d->sms);
-  const size_t smem = lk_smem_bytes(k.warps, k.depth, ProbePost::kScratch);
-  if (d->tables_at400)
-    sig_key_kernel<true, 4, k.warps, k.depth, false, ProbePost>
-        <<<blocks, 32 * k.warps, smem, s>>>(arenaS, offS, n, sigS, nullptr, 0, 0, post);
-  else
-    sig_key_kernel<false, 4, k.warps, k.depth, false, ProbePost>
-        <<<blocks, 32 * k.warps, smem, s>>>(arenaS, offS, n, sigS, nullptr, 0, 0, post);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "signature and probe kernel launch");
-  return AS_OK;
-}
-
 // R's signatures with the build fused in (BuildPost): the signature kernel
 // (shape 0) inserts each group of keys into the cleared table slots[0..mask].
 static as_status launch_sig_build(const DeviceState* d, const uint8_t* arenaR, const uint64_t* offR, uint64_t m,
-                                  uint64_t* sigR, Slot* slots, uint64_t mask, uint32_t* flags, cudaStream_t s) {
+                                  uint64_t* sigR, Slot* slots, uint64_t mask, uint32_t* flags, cudaStream_t s,
+                                  int max_blocks) {
   if (m == 0) return AS_OK;
   BuildPost post;
   post.slots = slots;
@@ -1287,9 +1138,9 @@ static as_status launch_sig_build(const DeviceState* d, const uint8_t* arenaR, c
   post.offR = offR;
   post.flags = flags;
   constexpr LKShape k = kLKShapes[0];
-  const uint64_t want = (m + 32ull * k.warps - 1) / (32ull * k.warps);
-  const unsigned blocks = (unsigned)(want < (uint64_t)d->sms ? (want < 1 ? 1 : want) : (uint64_t)d->sms);
-  const size_t smem = lk_smem_bytes(k.warps, k.depth, BuildPost::kScratch);
+  const uint64_t want = (m + 31) / 32;
+  const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
+  const size_t smem = lk_smem_bytes(k.warps, k.depth);
   if (d->tables_at400)
     sig_key_kernel<true, 4, k.warps, k.depth, false, BuildPost>
         <<<blocks, 32 * k.warps, smem, s>>>(arenaR, offR, m, sigR, nullptr, 0, 0, post);
@@ -1299,6 +1150,26 @@ static as_status launch_sig_build(const DeviceState* d, const uint8_t* arenaR, c
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature and build kernel launch");
   return AS_OK;
+}
+
+// Blocks of the passes over R (m keys) and S (n keys) of a join whose two passes
+// run at the same time.  A block of the signature kernel takes a whole SM, so
+// where a pass has at most four groups of 32 keys per warp of the device the
+// SMs are divided and both run beside each other.  R's pass, which goes on to
+// insert its keys, gets a warp for every group if that takes no more than a
+// quarter of the SMs (10k x 100k keys of 64-256 bytes: 23 us on 14 SMs, 12 us
+// on 20), else its share by key count.  Larger passes take all SMs one after
+// the other, which needs no guess about the keys' lengths.
+static void split_sms(int sms, uint64_t m, uint64_t n, int* blocks_r, int* blocks_s) {
+  const int warps = kLKShapes[0].warps;
+  const uint64_t groups = (m + 31) / 32 + (n + 31) / 32;
+  *blocks_r = *blocks_s = sms;
+  if (m == 0 || n == 0 || sms < 4 || groups > 4ull * sms * warps) return;
+  const int all = (int)(((m + 31) / 32 + warps - 1) / warps);   // a warp per group of R
+  const int share = (int)((double)sms * (double)m / (double)(m + n) + 0.5);
+  const int r = all <= sms / 4 ? all : share;
+  *blocks_r = r < 1 ? 1 : (r > sms - 1 ? sms - 1 : r);
+  *blocks_s = sms - *blocks_r;
 }
 
 // Work that may overlap the caller's stream s: fork() makes a side stream
@@ -1496,10 +1367,12 @@ size_t as_join_ws_bytes(uint64_t m, uint64_t n, float load_factor) {
   return t ? t + 256 + as_join_probe_ws_bytes(n) : 0;
 }
 
-as_status as_join_build(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
-                        const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
-                        as_stream stream) {
-  NvtxRange nvtx_range("as_join_build");
+}  // extern "C"
+
+// as_join_build's work; max_blocks: blocks of the pass over R (0: one per SM)
+static as_status build_impl(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
+                            const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
+                            as_stream stream, int max_blocks) {
   if (!out) return fail(AS_ERR_INVALID, "as_join_build: null table");
   uint64_t cap;
   uint32_t l2;
@@ -1524,7 +1397,7 @@ as_status as_join_build(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, co
   if ((e = cudaMemsetAsync(flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
   const uint64_t* sigR = d_sigR;
   if (!sigR && m > 0) {                              // R's signatures with the build in the same kernel
-    st = launch_sig_build(d, d_arenaR, d_offR, m, sig_ws, slots, cap - 1, flags, s);
+    st = launch_sig_build(d, d_arenaR, d_offR, m, sig_ws, slots, cap - 1, flags, s, max_blocks > 0 ? max_blocks : d->sms);
     if (st != AS_OK) return st;
     sigR = sig_ws;
   } else if (m > 0) {
@@ -1546,6 +1419,15 @@ as_status as_join_build(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, co
   out->reserved = 0;
   out->matched = reinterpret_cast<uint32_t*>(ws + round256(cap * 16) + round256(m * 8) + 256);
   return AS_OK;
+}
+
+extern "C" {
+
+as_status as_join_build(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
+                        const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
+                        as_stream stream) {
+  NvtxRange nvtx_range("as_join_build");
+  return build_impl(d_ws, ws_bytes, d_arenaR, d_offR, d_idR, m, d_sigR, load_factor, out, stream, 0);
 }
 
 size_t as_join_probe_ws_bytes(uint64_t n) { return (size_t)(round256(n * 8) + 256); }
@@ -1640,10 +1522,7 @@ static as_status probe_impl(const char* fn, const as_table* t, const uint8_t* d_
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e;
   if ((e = cudaMemsetAsync(d_count, 0, 8, s)) != cudaSuccess) return cuda_fail(e, "counter clear");
-  if (n >= kFusedProbeFrom) {                      // signatures and probe in one kernel
-    st = launch_sig_probe(d, t, d_arenaS, d_offS, d_idS, n, sigS, d_pairs, cap_pairs, d_count, s);
-    if (st != AS_OK) return st;
-  } else if (n > 0) {
+  if (n > 0) {
     st = launch_sig(d_arenaS, d_offS, n, sigS, s);
     if (st != AS_OK) return st;
     st = launch_verify(d, t, d_arenaS, d_offS, d_idS, n, sigS, d_pairs, cap_pairs, d_count, s);
@@ -1736,25 +1615,19 @@ as_status as_join(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_
   uint64_t* cnt = d_count ? d_count : (uint64_t*)rest;
   cudaStream_t s = (cudaStream_t)stream;
   as_table t;
-  if (n >= kFusedProbeFrom) {
-    // R's signatures and the build, then S's signatures with the probe fused in (the verification
-    // reads the S keys while they may still sit in L2)
-    if ((st = as_join_build(d_ws, tb, d_arenaR, d_offR, d_idR, m, nullptr, load_factor, &t, stream)) != AS_OK)
-      return st;
-    return probe_impl("as_join", &t, d_arenaS, d_offS, d_idS, n, sigS, nullptr, 0, d_pairs, cap_pairs, cnt, h_count,
-                      stream);
-  }
-  // smaller S: its signatures on a side stream, concurrently with R's signatures and the build
-  // (kernels of small relations leave SMs idle), then the probe
+  // S's signatures on a side stream, concurrently with R's signatures and the build (kernels of small
+  // relations leave SMs idle), then the probe
   SideStream side;
+  int blocks_r, blocks_s;
+  split_sms(d->sms, m, n, &blocks_r, &blocks_s);
   if (n > 0) {
     if ((st = side.fork(d, s)) != AS_OK) return st;
-    if ((st = launch_sig(d_arenaS, d_offS, n, sigS, side.side)) != AS_OK) {
+    if ((st = launch_sig(d_arenaS, d_offS, n, sigS, side.side, 4, 0, blocks_s)) != AS_OK) {
       side.join();
       return st;
     }
   }
-  st = as_join_build(d_ws, tb, d_arenaR, d_offR, d_idR, m, nullptr, load_factor, &t, stream);
+  st = build_impl(d_ws, tb, d_arenaR, d_offR, d_idR, m, nullptr, load_factor, &t, stream, blocks_r);
   const as_status js = side.join();
   if (st != AS_OK) return st;
   if (js != AS_OK) return js;

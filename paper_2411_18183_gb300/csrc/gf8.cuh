@@ -83,7 +83,7 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int j) {
 __global__ void __launch_bounds__(kG8Threads) sig8_kernel(const uint8_t* __restrict__ arena,
                                                           const uint64_t* __restrict__ off, uint64_t n,
                                                           uint64_t* __restrict__ sig_out) {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   init_red8_tables(red, red + kRedWords);           // ends with __syncthreads()
   const RedCursor rc = red_cursor(red);

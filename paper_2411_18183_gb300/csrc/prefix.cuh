@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __rest
                                                            uint32_t block_bytes,
                                                            const uint64_t* __restrict__ pref_off,
                                                            uint64_t* __restrict__ out) {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* ptab = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);
@@ -318,7 +318,7 @@ constexpr int kCapThreads = 1024;       // threads per block of capsig_kernel (3
 __global__ void __launch_bounds__(kCapThreads) capsig_kernel(const uint8_t* __restrict__ arena,
                                                            const uint64_t* __restrict__ off, uint64_t n,
                                                            uint64_t cap_len, uint64_t* __restrict__ out) {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* inv32 = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kCapThreads) prefix_thread_kernel(const uint8_
                                                                     uint32_t block_bytes,
                                                                     const uint64_t* __restrict__ pref_off,
                                                                     uint64_t* __restrict__ out) {
-  extern __shared__ __align__(16) uint8_t smem[];
+  extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* inv32 = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);

@@ -25,50 +25,68 @@
 // conjugate of x^3 (so D_b(x^6) is a fixed GF(2)-linear image of D_b(theta)),
 // kept in a basis of GF(2^16) where its Horner step is 13 logic operations per
 // 16 bytes; xs3_net.h (written by gen_xs3.py) holds that step and the map back
-// to polynomial coordinates.
+// to polynomial coordinates.  Groups whose keys have at most kLKShort blocks are
+// computed this way; longer ones by the same evaluations in quotient form
+// (quotient.cuh), 32 instead of 50 logic operations per block and about 70 more
+// per key.
 //
 // Scheduling.  Each warp owns a range of keys with an equal share of the work
-// (key bytes + a fixed cost per key) and walks it in windows of kLKWin keys.  A window's keys are sorted by length, and the warp
-// computes them in groups of 32 consecutive sorted keys, one key per lane, so
-// the lanes of a group have (nearly) the same amount of work.  A lane streams
-// its key from global memory in 32-byte blocks (one 256-bit load per block,
-// read-only path, no L1 allocation: every DRAM sector is fetched once), from
-// the key's last block to its first, kLKDepth blocks ahead of the arithmetic
-// in registers.  Lanes of a group whose keys are shorter start later, so all
-// lanes reach their first block in the group's last iteration and finish the
-// signatures together.  (Staging the keys through shared memory was measured
-// slower: per-lane 16-byte copies fetch each 32-byte sector twice, and a TMA
-// bulk copy per lane is serialised because its operands are warp-uniform.)
+// (key bytes + a fixed cost per key) and walks it in windows of kLKWin keys.  A
+// window's keys are sorted by length, and the warp computes them in groups of
+// 32 consecutive sorted keys, one key per lane, so the lanes of a group have
+// (nearly) the same amount of work.  Keys are taken in 32-byte blocks from the
+// last to the first; the lanes of a group whose keys are shorter start later,
+// so all lanes reach their first block in the group's last step and finish the
+// signatures together.
+//
+// Loads.  A step is 4 blocks (128 bytes) of each of the group's keys.  The warp
+// copies them into its shared-memory rows (one row per key) by 16-byte
+// asynchronous copies, eight consecutive lanes to a key, so that a request
+// covers up to a whole 128-byte line; then each lane reads its own row.  With
+// every lane loading its own key's 32-byte blocks into registers instead, a
+// warp load is 32 requests of one sector each, and keys of 256-1024 bytes stop
+// at 4.2 TB/s whatever the arithmetic, the order of the keys or the bytes in
+// flight (fixed-length keys, 5.1 TB/s); the copies alone reach 5.8 TB/s in the
+// same order.  Steps are two or three ahead of the arithmetic, and the next
+// group's first steps are requested before a group's signatures are finished.
+// Copies are of the 16-byte chunks of a key's 32-byte blocks up to its last
+// byte; nothing outside the arena's readable range is touched, and the rest of
+// a row is zero-filled.
+// Measured (signatures of 2M keys of 256-1024 bytes, 1.28 GB: 346 us with the
+// register loads and the remainder form, 265 us now, 4.8 TB/s; 300k keys of
+// 2048-8192 bytes, two components: 375 and 277 us; 4M keys of 32-128 bytes: 204
+// and 193 us, bound by the arithmetic per key).
 // In a batch the keys are the joins' row ranges back to back ("virtual
 // rows"): the warps split them by work across the joins, and a window
 // ends with its join's rows so that its keys are consecutive in the relation.
 #pragma once
 #include <cstdint>
 
+#include "quotient.cuh"
 #include "xs3_net.h"
 
 namespace algsig {
 
-#ifndef ALGSIG_LK_FINISH
-#define ALGSIG_LK_FINISH __forceinline__
-#endif
-#ifndef ALGSIG_LK_LDQUAL
-#define ALGSIG_LK_LDQUAL volatile
-#endif
-// Kernel shapes: warps per block (one block per SM) and 32-byte blocks in
-// flight per key.  More warps hide more latency, more blocks in flight per key
-// need more registers; the batch autotuner picks one per batch.  Shape 0 is
-// the default of single relations.
+// image of the shared-memory constant-multiply tables (quotient.cuh): those of
+// the quotient form, then those of the remainder form; set up once per device
+__device__ uint4 g_inv[4 * kInvEntries / 16];
+
+// Kernel shapes: warps per block (one block per SM) and 32-byte blocks of each
+// key in flight (a multiple of 4, one step).  The batch autotuner picks one per
+// batch.  Shape 0 is the default of single relations.
 struct LKShape {
   int warps, depth;
 };
-constexpr LKShape kLKShapes[] = {{24, 2}, {16, 2}, {32, 1}};
+constexpr LKShape kLKShapes[] = {{16, 8}, {10, 12}, {8, 16}};
 constexpr int kLKShapeCount = sizeof(kLKShapes) / sizeof(kLKShapes[0]);
-#ifndef ALGSIG_LK_WIN
-#define ALGSIG_LK_WIN 256
-#endif
-constexpr int kLKWin = ALGSIG_LK_WIN;                 // keys per sorting window (a power of two)
-constexpr uint32_t kLKNoKey = 0xFFFFFFFFu;            // empty sorting entry
+constexpr int kLKWin = 256;                           // most keys of a sorting window
+// Keys of at least kLKNarrowFrom bytes on average are sorted in windows of
+// kLKNarrowWin: neighbouring keys share a 128-byte line of DRAM, and with the
+// larger window the line is often gone from L2 when the second key is read
+// (2M keys of 256-1024 bytes: 1.47 GB read for 1.28 GB of keys, 283 against
+// 271 us); for keys of 32-128 bytes the sort's share counts (197 against 205 us).
+constexpr int kLKNarrowWin = 128;
+constexpr uint64_t kLKNarrowFrom = 256;
 // relations of this many keys and more are split over the warps by work (a
 // search in the offsets); smaller ones by key count, which saves the search's
 // dependent loads where they would be a large share of the kernel's time
@@ -79,61 +97,93 @@ constexpr uint64_t kLKSearchFrom = 1ull << 19;
 // warps' shares are cut on it, so that a relation (or batch) that mixes short
 // and long keys leaves no warp with far more keys than the others.
 constexpr uint64_t kLKKeyCost = 140;
-constexpr int kLKIdxBits = kLKWin == 256 ? 8 : (kLKWin == 128 ? 7 : (kLKWin == 64 ? 6 : 10));
-static_assert((1 << kLKIdxBits) == kLKWin, "window sizes 64, 128, 256");
-constexpr uint32_t kLKNbCap = (1u << (31 - kLKIdxBits)) - 1u;   // block counts above sort together
 
 struct LKWarp {
   uint64_t woff[kLKWin + 2];       // offsets of the window's keys (woff[i] = off[wb + i]), i <= wn
-  uint32_t order[kLKWin];          // window entries by block count: (block count << 8 | index)
-  uint32_t hist[256];              // the counting sort's bins (block counts, 255 and up in the last)
+  uint8_t order[kLKWin];           // window entries by block count
 };
-static_assert(kLKWin >= 64 && kLKWin <= 256, "the window sort: up to 8 entries and 8 bins per lane");
-constexpr size_t kSmemLKMasks = 1056;                 // 33 rows of 32 bytes
-// (the blocks in flight of a shape live in registers: its depth takes no shared memory)
-constexpr size_t lk_smem_bytes(int warps, int /*depth*/, size_t scratch_per_warp = 0) {
-  return (size_t)kRedBytes + 1024 + kSmemLKMasks + (size_t)warps * (sizeof(LKWarp) + scratch_per_warp);
+static_assert(kLKWin == 256, "the window sort: 8 entries and 8 bins per lane, entries in a byte");
+constexpr int kLKStep = 4;                            // blocks per step
+constexpr int kLKRow = 32 * kLKStep;                  // bytes of a key's row
+constexpr int kLKPitch = 2 * kLKRow;                  // rows of two stages, or of a stage and a table, side by side
+constexpr int kLKState = 40;                          // state registers of a key: 16 + 16 or 16 + 24
+// groups of at most this many blocks take lk_short_blocks (at most one step; 4M keys of 32-128 bytes:
+// 201, 199, 193 and 197 us with 0, 2, 3 and 4)
+constexpr int kLKShort = 3;
+
+// Shared memory: 256-byte lines of two halves.  The lower halves of the first
+// 256 lines hold the reduction tables (16 copies of each entry).  A warp's
+// stages are 32 rows each in one column of halves, one after the other: the
+// upper halves beside the tables serve the first 8 / stages warps, the lines
+// after them two warps side by side.  Then the constant-multiply tables, the
+// byte masks and the warps' windows.
+constexpr size_t kSmemLKInv = 4 * kInvEntries;
+constexpr size_t kSmemLKMasks = 17 * 16;
+constexpr uint32_t kLKStageBytes = 32 * kLKPitch;     // from one stage of a warp to the next
+__host__ __device__ constexpr size_t lk_line_bytes(int warps, int depth) {
+  const int stages = depth / kLKStep, beside = 8 / stages;
+  return (size_t)256 * kLKPitch + (size_t)((warps > beside ? warps - beside : 0) + 1) / 2 * stages * kLKStageBytes;
 }
-static_assert(lk_smem_bytes(32, 1) <= 232448, "lane-per-key signature kernel: shared memory");
+__host__ __device__ constexpr size_t lk_smem_bytes(int warps, int depth) {
+  return lk_line_bytes(warps, depth) + kSmemLKInv + kSmemLKMasks + (size_t)warps * sizeof(LKWarp);
+}
+static_assert(lk_smem_bytes(16, 8) <= 232448 && lk_smem_bytes(10, 12) <= 232448 && lk_smem_bytes(8, 16) <= 232448,
+              "the shapes' shared memory");
+// byte offset of a warp's first stage
+template <int kStages>
+__device__ __forceinline__ uint32_t lk_stage_base(uint32_t w) {
+  constexpr uint32_t kBeside = 8 / kStages;
+  if (w < kBeside) return w * kStages * kLKStageBytes + kLKRow;
+  const uint32_t j = w - kBeside;
+  return 256u * kLKPitch + (j >> 1) * kStages * kLKStageBytes + (j & 1u) * kLKRow;
+}
 
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem_src) : "memory");
 }
+// chunk c of a key of n chunks, at src + s * kStep, to shared memory; zeros (nothing read) past the key
+__device__ __forceinline__ void cp_async16_below(uint32_t smem_dst, const uint8_t* src, uint32_t s, uint32_t step,
+                                                 uint32_t c, uint32_t n) {
+  asm volatile(
+      "{\n.reg .pred p;\n.reg .u64 a;\n"
+      "setp.ge.u32 p, %4, %5;\n"
+      "mad.wide.u32 a, %2, %3, %1;\n"
+      "cp.async.cg.shared.global [%0], [a], 16, p;\n}\n" ::"r"(smem_dst), "l"(src), "r"(s), "r"(step), "r"(c), "r"(n)
+      : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait_but() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint4& v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
 
-// One 32-byte block of key bytes.
-struct Blk {
-  uint32_t w[8];
+// Table cursors of the half-line tables (red32 and red24 of gf16.cuh): 16
+// copies of each entry, lanes l and l + 16 share one.  Lookups take two bank
+// cycles instead of one, 26 lookups of a pair per 32 keys, and the tables half
+// the shared memory and half the time to copy.
+template <bool AT400>
+struct LKCursor {
+  uint32_t tab, off16, off24;
+  __device__ __forceinline__ explicit LKCursor(const uint8_t* smem) {
+    tab = (uint32_t)__cvta_generic_to_shared(smem);
+    off16 = 4u * (threadIdx.x & 15u);
+    off24 = off16 + 64u;
+  }
+  __device__ __forceinline__ uint32_t load(uint32_t idx) const {
+    if constexpr (!AT400) return lds32(tab + idx);
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1+1024];" : "=r"(v) : "r"(idx));
+    return v;
+  }
 };
-
-// 32 bytes at the 32-byte aligned address p, read-only path without L1
-// allocation.
-__device__ __forceinline__ Blk ld_blk(const uint8_t* p) {
-  Blk b;
-  asm ALGSIG_LK_LDQUAL("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                       : "=r"(b.w[0]), "=r"(b.w[1]), "=r"(b.w[2]), "=r"(b.w[3]), "=r"(b.w[4]), "=r"(b.w[5]),
-                         "=r"(b.w[6]), "=r"(b.w[7])
-                       : "l"(p));
-  return b;
-}
-// The same with bytes outside [lim_lo, lim_hi) (the arena's readable range)
-// not read and returned as zero; they never hold key bytes.  Only keys in the
-// arena's first or last 32 bytes need it (lk_edge_key).
-__device__ __forceinline__ Blk ld_blk_checked(const uint8_t* p, const uint8_t* lim_lo, const uint8_t* lim_hi) {
-  if (p >= lim_lo && p + 32 <= lim_hi) return ld_blk(p);
-  Blk b;
-#pragma unroll
-  for (int i = 0; i < 8; i++) b.w[i] = 0;
-  if (p >= lim_lo && p + 16 <= lim_hi) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-    b.w[0] = v.x; b.w[1] = v.y; b.w[2] = v.z; b.w[3] = v.w;
-  }
-  if (p + 16 >= lim_lo && p + 32 <= lim_hi) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p + 16));
-    b.w[4] = v.x; b.w[5] = v.y; b.w[6] = v.z; b.w[7] = v.w;
-  }
-  return b;
-}
 
 // Bit-sliced Horner step over one 16-byte chunk (words v0..v3, v3 last in the
 // key): S <- S x^4 + v3 x^3 + v2 x^2 + v1 x + v0, with x^16 = x^12 + x^3 + x + 1.
@@ -154,21 +204,6 @@ __device__ __forceinline__ void xs_chunk(uint32_t (&c)[16], uint32_t v0, uint32_
   c[6] = n6; c[5] = n5; c[4] = n4; c[3] = n3; c[2] = n2; c[1] = n1; c[0] = n0;
 }
 
-// Component K (1, 2 or 4) from the bit-sliced state:
-//   sum_m x^(2 K m) (lo16(c_m) + x^K hi16(c_m)) mod P,
-// by Horner over m with a 32-bit accumulator reduced every 8/K steps.
-template <int K, class Cursor>
-__device__ __forceinline__ uint32_t xs_component(const uint32_t (&c)[16], const Cursor& rc) {
-  constexpr int kEvery = 8 / K;
-  uint32_t acc = 0;
-#pragma unroll
-  for (int m = 15; m >= 0; --m) {
-    acc = (acc << (2 * K)) ^ (c[m] & 0xFFFFu) ^ ((c[m] >> 16) << K);
-    if ((16 - m) % kEvery == 0) acc = red32(acc, rc);
-  }
-  return acc;
-}
-
 // Component 3 from its bit-sliced state: with p_i = the poly coordinate i of
 // every D_b(x^6) (bit b), sum_i x^i (lo16(p_i) + x^3 hi16(p_i)) mod P, by
 // Horner over i with a 32-bit accumulator reduced once on the way.
@@ -179,34 +214,21 @@ __device__ __forceinline__ uint32_t xs3_component(const uint32_t (&c3)[16], cons
   uint32_t acc = 0;
 #pragma unroll
   for (int i = 15; i >= 0; --i) {
-    acc = (acc << 1) ^ (p[i] & 0xFFFFu) ^ ((p[i] >> 16) << 3);   // degree <= 18 + (15 - i)
+    acc = (acc * c_pow2[1]) ^ (p[i] & 0xFFFFu) ^ ((p[i] >> 16) * c_pow2[3]);   // degree <= 18 + (15 - i)
     if (i == 3) acc = red32(acc, rc);
   }
   return red32(acc, rc);
-}
-
-// x^-m * v in GF(2^16) for 0 <= m <= 60; inv32: the multiply table of x^-32
-template <class Cursor>
-__device__ __forceinline__ uint32_t mul_xinv(const uint16_t* inv32, uint32_t v, uint32_t m, const Cursor& rc) {
-  if (m >= 32) {
-    v = mulc(inv32, v);
-    m -= 32;
-  }
-  const uint32_t d = mulc(inv32, v);                     // v x^-32
-  const uint64_t E = (uint64_t)d << (32 - m);            // v x^-32 x^(32-m), < 2^48
-  const uint32_t r1 = red32((uint32_t)(E >> 16), rc);
-  return red32(((uint32_t)E & 0xFFFFu) ^ (r1 << 16), rc);
 }
 
 // A lane's key in the current group.
 struct LKKey {
   uint64_t kq;          // key index
   const uint8_t* base;  // 32-byte aligned address of the key's first block
-  uint32_t nb;          // realigned 32-byte blocks (0: empty key)
+  uint32_t nb;          // 32-byte blocks (0: empty key)
   uint32_t a;           // offset of the key's first byte in its first block (0..31)
-  uint32_t tail;        // bytes of the last aligned block that belong to the key, counted from its start
+  uint32_t c1;          // 16-byte chunks from base up to the key's last byte
+  uint32_t te;          // key bytes of the last of them (0: all 16)
   bool valid;
-  bool edge;            // a block of the key reaches outside the arena's readable range
 };
 
 // prefetch the offsets of the window starting at key wb (cp.async, one group)
@@ -215,48 +237,50 @@ __device__ __forceinline__ void lk_prefetch_window(LKWarp& W, const uint64_t* __
   const uint32_t lane = threadIdx.x & 31u;
   if (wb < k_hi) {
     const uint64_t left = k_hi - wb;
-    const uint32_t wn = left < (uint64_t)kLKWin ? (uint32_t)left : (uint32_t)kLKWin;
+    const uint32_t wn = left < (uint64_t)kLKWin ? (uint32_t)left : (uint32_t)kLKWin;   // (a window at most)
     for (uint32_t e = lane; e <= wn; e += 32) cp_async8(&W.woff[e], off + wb + e);
   }
   cp_async_commit();
 }
 
-// realigned 32-byte blocks of the key at absolute address abs
+// aligned 32-byte blocks that hold the key at absolute address abs
 __device__ __forceinline__ uint32_t lk_blocks(uintptr_t abs, uint64_t len) {
   if (len == 0) return 0u;
-  const uint64_t lo = (abs & 31u) & ~1ull;
-  const uint64_t nb = (lo + len + 31) >> 5;
+  const uint64_t nb = ((abs & 31u) + len + 31) >> 5;
   return nb < 0xFFFFFFFFull ? (uint32_t)nb : 0xFFFFFFFFu;
 }
 
 // order the window's entries by block count: a counting sort over the block
 // counts (255 and more share the last bin; the order within a bin is
 // arbitrary), so that each group of 32 consecutive entries has keys of
-// nearly equal length
-__device__ __forceinline__ void lk_sort_window(LKWarp& W, uint32_t wn, uintptr_t arena) {
+// nearly equal length.  rows: an empty stage, the first 8 rows of which hold
+// the bins' counts.
+__device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_t wn, uintptr_t arena) {
   const uint32_t lane = threadIdx.x & 31u;
   if (wn <= 32) {                                    // one group: nothing to balance
-    for (uint32_t i = lane; i < (uint32_t)kLKWin; i += 32) W.order[i] = i < wn ? i : kLKNoKey;
+    W.order[lane] = (uint8_t)lane;
     __syncwarp();
     return;
   }
+  auto count = [&](uint32_t b) -> uint32_t& {
+    return reinterpret_cast<uint32_t*>(rows + (b >> 5) * kLKPitch)[b & 31u];
+  };
+  uint32_t* mine = &count(8 * lane);                  // the lane's 8 consecutive bins
 #pragma unroll
-  for (int t = 0; t < 8; ++t) W.hist[8 * lane + t] = 0u;
+  for (int t = 0; t < 8; ++t) mine[t] = 0u;
   __syncwarp();
   constexpr int kPer = kLKWin / 32;                   // entries per lane
-  uint32_t e[kPer], bin[kPer], rank[kPer];
+  uint32_t bin[kPer], rank[kPer];
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const uint32_t i = lane + 32u * (uint32_t)j;
-    e[j] = kLKNoKey;
     bin[j] = 0;
     rank[j] = 0;
     if (i < wn) {
       const uint64_t ks = W.woff[i], len = W.woff[i + 1] - ks;
       const uint32_t nb = lk_blocks(arena + ks, len);
-      e[j] = ((nb < kLKNbCap ? nb : kLKNbCap) << kLKIdxBits) | i;
       bin[j] = nb < 255u ? nb : 255u;
-      rank[j] = atomicAdd(&W.hist[bin[j]], 1u);
+      rank[j] = atomicAdd(&count(bin[j]), 1u);
     }
   }
   __syncwarp();
@@ -264,7 +288,7 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint32_t wn, uintptr_t
   uint32_t h[8], sum = 0;
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
-    h[t] = W.hist[8 * lane + t];
+    h[t] = mine[t];
     sum += h[t];
   }
   uint32_t incl = sum;
@@ -277,87 +301,131 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint32_t wn, uintptr_t
   __syncwarp();
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
-    W.hist[8 * lane + t] = base;
+    mine[t] = base;
     base += h[t];
   }
   __syncwarp();
 #pragma unroll
-  for (int j = 0; j < kPer; ++j)
-    if (e[j] != kLKNoKey) W.order[W.hist[bin[j]] + rank[j]] = e[j];
-  for (uint32_t i = wn + lane; i < (uint32_t)kLKWin; i += 32) W.order[i] = kLKNoKey;
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t i = lane + 32u * (uint32_t)j;
+    if (i < wn) W.order[count(bin[j]) + rank[j]] = (uint8_t)i;
+  }
   __syncwarp();
 }
 
 // group g of the window (wb: its first key) into the lanes; returns the
-// group's iteration count (its longest key's blocks, at least 1)
-__device__ __forceinline__ uint32_t lk_load_group(LKKey& k, const LKWarp& W, uint64_t wb, uint32_t g,
-                                                  const uint8_t* arena, const uint8_t* lim_lo,
-                                                  const uint8_t* lim_hi) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t e = W.order[32 * g + lane];
-  k.valid = e != kLKNoKey;
-  k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.tail = 0; k.edge = false;
+// group's block count (its longest key's, at least 1)
+__device__ __forceinline__ uint32_t lk_load_group(LKKey& k, const LKWarp& W, uint64_t wb, uint32_t wn, uint32_t g,
+                                                  const uint8_t* arena) {
+  const uint32_t r = 32u * g + (threadIdx.x & 31u);
+  k.valid = r < wn;
+  k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.c1 = 0; k.te = 0;
   if (k.valid) {
-    const uint32_t i = e & (kLKWin - 1);
+    const uint32_t i = W.order[r];
     const uint64_t ks = W.woff[i], len = W.woff[i + 1] - ks;
     const uintptr_t abs = reinterpret_cast<uintptr_t>(arena) + ks;
     k.kq = wb + i;
+    // blocks start on a 32-byte boundary (a DRAM sector each), but at the arena's first chunk where
+    // that lies on an odd 16-byte boundary
     k.base = reinterpret_cast<const uint8_t*>(abs & ~(uintptr_t)31);
-    k.a = (uint32_t)(abs & 31u);
-    k.nb = lk_blocks(abs, len);
-    if (k.nb) k.tail = (uint32_t)((uint64_t)k.a + len - 32ull * (k.nb - 1));
-    k.edge = k.nb && (k.base < lim_lo || k.base + 32ull * k.nb > lim_hi);
+    if (k.base < arena) k.base += 16;
+    k.a = (uint32_t)(abs - reinterpret_cast<uintptr_t>(k.base));
+    k.nb = len ? (uint32_t)min((uint64_t)0xFFFFFFFFu, (k.a + len + 31) >> 5) : 0u;
+    if (k.nb) {
+      k.c1 = (uint32_t)((k.a + len + 15) >> 4);
+      k.te = (uint32_t)(k.a + len) & 15u;
+    }
   }
-  // an edge key is computed apart (lk_edge_key); the group's loop skips it
-  const uint32_t G = __reduce_max_sync(kFull, k.edge ? 0u : k.nb);
+  const uint32_t G = __reduce_max_sync(kFull, k.nb);
   return G < 1u ? 1u : G;
 }
 
-// an empty slot (no key) for a lane
-__device__ __forceinline__ uint32_t lk_no_group(LKKey& k, const uint8_t* arena) {
-  k.valid = false;
-  k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.tail = 0; k.edge = false;
-  return 1u;
-}
-
-// Byte masks of a 32-byte block in shared memory: row e (0..32) keeps bytes
-// [0, e).  Masking a block is two 16-byte loads and eight logic operations.
-constexpr int kLKMaskRows = 33;
+// mask of the first e bytes of a chunk, e = 0..16
 __device__ __forceinline__ void lk_fill_masks(uint4* mt) {
-  for (int i = threadIdx.x; i < kLKMaskRows * 2; i += blockDim.x) {
-    const int e = i >> 1, h = i & 1;
+  for (int e = threadIdx.x; e <= 16; e += blockDim.x) {
     uint32_t m[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      const int r = e - 16 * h - 4 * j;
+      const int r = e - 4 * j;
       m[j] = r <= 0 ? 0u : (r >= 4 ? ~0u : ((1u << (8 * r)) - 1u));
     }
-    mt[i] = make_uint4(m[0], m[1], m[2], m[3]);
+    mt[e] = make_uint4(m[0], m[1], m[2], m[3]);
   }
 }
-// keep bytes [0, e) of a block (e >= 32 keeps all)
-__device__ __forceinline__ void blk_keep_below(Blk& b, uint32_t e, const uint4* mt) {
-  const uint32_t r = e < 32u ? e : 32u;
-  const uint4 m0 = mt[2 * r], m1 = mt[2 * r + 1];
-  b.w[0] &= m0.x; b.w[1] &= m0.y; b.w[2] &= m0.z; b.w[3] &= m0.w;
-  b.w[4] &= m1.x; b.w[5] &= m1.y; b.w[6] &= m1.z; b.w[7] &= m1.w;
+
+// The copies of a group's steps: lane l copies chunk l % 8 of the rows of keys
+// l / 8, l / 8 + 4, ..., whose addresses and chunk counts it holds here.
+struct LKCopy {
+  const uint8_t* src[8];   // base + 16 (l % 8) of the key
+  uint32_t c1[8];          // the key's chunk count from base
+};
+
+// chunk c of the lane's row at shared address row (the lane's swizzle folded in)
+__device__ __forceinline__ uint32_t lk_chunk(uint32_t row, uint32_t c) { return row ^ (c << 4); }
+
+// the group's keys to the lanes that copy them, through the empty stage at shared address st
+__device__ __forceinline__ void lk_copy_setup(LKCopy& y, const LKKey& k, uint32_t st) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t b = reinterpret_cast<uint64_t>(k.base);
+  __syncwarp();
+  sts128(st + kLKPitch * lane, make_uint4((uint32_t)b, (uint32_t)(b >> 32), k.c1, 0u));
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 v = lds128(st + kLKPitch * (4 * i + (lane >> 3)));
+    y.src[i] = reinterpret_cast<const uint8_t*>((uint64_t)v.x | ((uint64_t)v.y << 32)) + 16 * (lane & 7u);
+    y.c1[i] = v.z;
+  }
+  __syncwarp();
 }
-// zero bytes [0, a) of a block (a < 32)
-__device__ __forceinline__ void blk_zero_below(Blk& b, uint32_t a, const uint4* mt) {
-  const uint4 m0 = mt[2 * a], m1 = mt[2 * a + 1];
-  b.w[0] &= ~m0.x; b.w[1] &= ~m0.y; b.w[2] &= ~m0.z; b.w[3] &= ~m0.w;
-  b.w[4] &= ~m1.x; b.w[5] &= ~m1.y; b.w[6] &= ~m1.z; b.w[7] &= ~m1.w;
+
+// request step s of the group's keys into the stage at shared address st
+__device__ __forceinline__ void lk_copy_step(const LKCopy& y, uint32_t st, uint32_t s) {
+  const uint32_t lane = threadIdx.x & 31u, q = lane & 7u, r = lane >> 3;
+  const uint32_t c = 8u * s + q;
+  // row 4 i + r, chunk q: its place is q ^ (row % 8), and row % 8 = 4 (i % 2) + r
+  const uint32_t d0 = st + r * kLKPitch + ((q ^ r) << 4), d1 = st + r * kLKPitch + ((q ^ (r + 4u)) << 4);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    cp_async16_below((i & 1 ? d1 : d0) + 4 * i * kLKPitch, y.src[i], s, kLKRow, c, y.c1[i]);
+}
+
+// zero what is not the key's in the rows that hold its ends: the bytes after
+// its last (in the step that holds it) and before its first (in step 0)
+__device__ __forceinline__ void lk_trim(const LKKey& k, uint32_t row, uint32_t s, const uint4* mt) {
+  if (k.te && (k.c1 - 1) >> 3 == s) {
+    const uint32_t p = lk_chunk(row, (k.c1 - 1) & 7u);
+    uint4 v = lds128(p);
+    const uint4 m = mt[k.te];
+    v.x &= m.x; v.y &= m.y; v.z &= m.z; v.w &= m.w;
+    sts128(p, v);
+  }
+  if (s == 0) {
+    const uint32_t p = lk_chunk(row, k.a >> 4);
+    uint4 v = lds128(p);
+    const uint4 m = mt[k.a & 15u];
+    v.x &= ~m.x; v.y &= ~m.y; v.z &= ~m.z; v.w &= ~m.w;
+    sts128(p, v);
+    if (k.a >= 16u) sts128(lk_chunk(row, 0), make_uint4(0, 0, 0, 0));
+  }
+}
+
+// block b (0..3) of the lane's row
+__device__ __forceinline__ void lk_read(uint32_t (&w)[8], uint32_t row, int b) {
+  const uint4 u = lds128(lk_chunk(row, 2 * b)), v = lds128(lk_chunk(row, 2 * b + 1));
+  w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
+  w[4] = v.x; w[5] = v.y; w[6] = v.z; w[7] = v.w;
 }
 
 // the Horner steps of one 32-byte block (its two chunks, the upper one first)
-template <int NCOMP, class Cursor>
-__device__ __forceinline__ void lk_block(const Blk& w, uint32_t sh, uint32_t& nxt0, uint32_t (&c)[16],
-                                         uint32_t (&c3)[16], const Cursor& rc) {
+template <int NCOMP>
+__device__ __forceinline__ void lk_block(const uint32_t (&w)[8], uint32_t sh, uint32_t& nxt0, uint32_t (&c)[16],
+                                         uint32_t (&c3)[16]) {
   uint32_t v[8];
 #pragma unroll
-  for (int i = 0; i < 7; i++) v[i] = __funnelshift_r(w.w[i], w.w[i + 1], sh);
-  v[7] = __funnelshift_r(w.w[7], nxt0, sh);
-  nxt0 = w.w[0];
+  for (int i = 0; i < 7; i++) v[i] = __funnelshift_r(w[i], w[i + 1], sh);
+  v[7] = __funnelshift_r(w[7], nxt0, sh);
+  nxt0 = w[0];
   xs_chunk(c, v[4], v[5], v[6], v[7]);
   xs_chunk(c, v[0], v[1], v[2], v[3]);
   if constexpr (NCOMP == 4) {
@@ -367,134 +435,101 @@ __device__ __forceinline__ void lk_block(const Blk& w, uint32_t sh, uint32_t& nx
 }
 
 // A key's signature from the Horner state of its blocks (values counted from
-// the first block's start; the key starts s = (a & ~1) / 2 symbols later).
+// the first block's start; the key starts floor(a / 2) symbols later).
 template <int NCOMP, class Cursor>
-__device__ ALGSIG_LK_FINISH uint64_t lk_finish(const uint32_t (&c)[16], const uint32_t (&c3)[16], uint32_t a,
-                                              const uint16_t* inv32, const Cursor& rc) {
-  const uint32_t v1 = xs_component<1>(c, rc);
-  const uint32_t v2 = xs_component<2>(c, rc);
-  const uint32_t s = (a & ~1u) >> 1;
-  uint64_t sig = (uint64_t)mul_xinv(inv32, v1, s, rc) | ((uint64_t)mul_xinv(inv32, v2, 2 * s, rc) << 16);
-  if constexpr (NCOMP == 4) {
-    const uint32_t v3 = xs3_component(c3, rc);
-    const uint32_t v4 = xs_component<4>(c, rc);
-    sig |= ((uint64_t)mul_xinv(inv32, v3, 3 * s, rc) << 32) | ((uint64_t)mul_xinv(inv32, v4, 4 * s, rc) << 48);
+__device__ __forceinline__ uint64_t lk_finish(const uint32_t (&st)[kLKState], uint32_t a, const uint16_t* inv,
+                                              const Cursor& rc) {
+  uint32_t c[16], c3[16], v[4];
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    c[i] = st[i];
+    c3[i] = st[16 + i];
   }
-  return sig;
+  components_124<NCOMP>(c, v, rc);
+  if constexpr (NCOMP == 4) v[2] = xs3_component(c3, rc);
+  return place_components<NCOMP>(v, a, inv, rc);
 }
 
-// The signature of a key with a block outside the arena's readable range
-// (its first 32 bytes or its last): the blocks one by one with checked loads.
-// At most a few keys per relation take this path.
-// (one copy per kernel instantiation: ptxas fails on a non-inlined function
-// shared by kernels of different shapes)
-template <int NCOMP, int kLKWarps, int kLKDepth, bool BATCH, class Unique, class Cursor>
-__device__ __noinline__ uint64_t lk_edge_key(const LKKey& k, const uint8_t* lim_lo, const uint8_t* lim_hi,
-                                             const uint16_t* inv32, const uint4* mt, const Cursor& rc) {
+// The state after a group of keys of at most kLKShort blocks, all of them in
+// the row, by the Horner step on the remainders (lk_block): components 1, 2
+// and 4's 16 registers, then component 3's.
+template <int NCOMP>
+__device__ __forceinline__ void lk_short_blocks(uint32_t (&st)[kLKState], const LKKey& k, uint32_t G, uint32_t row) {
   const uint32_t sh = 8u * (k.a & 1u);
   uint32_t nxt0 = 0;
-  if (k.tail > 32u) nxt0 = __ldg(reinterpret_cast<const uint32_t*>(k.base + 32ull * k.nb));
-  uint32_t c[16];
+  uint32_t c[16], c3[16];
 #pragma unroll
-  for (int i = 0; i < 16; i++) c[i] = 0;
-  uint32_t c3[16];                                    // component 3's state (unused with 2 components)
+  for (int i = 0; i < 16; i++) c[i] = c3[i] = 0;
 #pragma unroll
-  for (int i = 0; i < 16; i++) c3[i] = 0;
-  for (uint32_t vb = k.nb; vb-- > 0;) {
-    Blk w = ld_blk_checked(k.base + 32ull * vb, lim_lo, lim_hi);
-    if (vb + 1 == k.nb) blk_keep_below(w, k.tail, mt);
-    if (vb == 0) blk_zero_below(w, k.a, mt);
-    lk_block<NCOMP>(w, sh, nxt0, c, c3, rc);
+  for (int vb = kLKShort - 1; vb >= 0; --vb) {
+    if ((uint32_t)vb < G) {                           // warp-uniform
+      uint32_t w[8];
+      lk_read(w, row, vb);
+      lk_block<NCOMP>(w, sh, nxt0, c, c3);
+    }
   }
-  return lk_finish<NCOMP>(c, c3, k.a, inv32, rc);
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    st[i] = c[i];
+    st[16 + i] = c3[i];
+  }
 }
 
-// The signatures of one group of keys: in iteration it of the group's G
-// iterations the lane takes block vb = G - 1 - it of its key (its own blocks
-// are vb < nb), so the lanes of shorter keys start later and every key reaches
-// its block 0 in the group's last iteration.  An odd key whose last aligned
-// block ends with a key byte needs the next block's first byte.  Keys with a
-// block outside the arena's readable range are computed apart (lk_edge_key).
-template <int NCOMP, int kLKWarps, int kLKDepth, bool BATCH, class Unique, class Cursor>
-__device__ __forceinline__ uint64_t lk_group(const LKKey& k, uint32_t G, const uint8_t* lim_lo, const uint8_t* lim_hi,
-                                         const uint16_t* inv32, const uint4* mt, uint64_t* __restrict__ sig_out,
-                                         const Cursor& rc) {
-  const uint32_t nb = k.edge ? 0u : k.nb;
-  const uint32_t sh = 8u * (k.a & 1u);
-  uint32_t nxt0 = 0;
-  if (nb && k.tail > 32u) nxt0 = __ldg(reinterpret_cast<const uint32_t*>(k.base + 32ull * nb));
-  // kLKDepth blocks in flight: iteration it takes its block out of ring slot it % kLKDepth and
-  // refills the slot with block it + kLKDepth before computing (a ring of kLKDepth + 1 slots
-  // written in place, and loads that run on into the next group, measured slower)
-  Blk ring[kLKDepth];
+// The state after a group of longer keys, by division in quotient form
+// (quotient.cuh): the digit rings, in st.  A stage is refilled with the step
+// kStages further down once it is computed.  The loop is unrolled over three
+// steps (12 blocks), after which the digit rings are at their first registers
+// again.  base: shared address of the warp's first stage, row: of the lane's
+// row in it; step s waits in stage s % kStages.
+template <class Net, int kStages>
+__device__ __forceinline__ void lk_long_blocks(uint32_t (&st)[kLKState], const LKKey& k, uint32_t G, const LKCopy& copy,
+                                               uint32_t base, uint32_t row, const uint4* mt) {
+  constexpr int P = Net::kPhases, U = 3;
+  static_assert(U * kLKStep % P == 0, "the rings close over the unrolled steps");
+  const uint32_t S = (G + kLKStep - 1) / kLKStep;
+  Net net;
+  net.clear();
+  for (uint32_t s0 = (S - 1) / U * U;; s0 -= U) {
 #pragma unroll
-  for (int u = 0; u < kLKDepth; ++u) {
+    for (int j = U - 1; j >= 0; --j) {
+      const uint32_t s = s0 + (uint32_t)j;
+      if (s < S) {                                    // warp-uniform
+        const uint32_t at = (kStages == U ? (uint32_t)j : s % kStages) * kLKStageBytes;
+        cp_async_wait_but<kStages - 1>();
+        __syncwarp();
+        lk_trim(k, row + at, s, mt);
+        uint32_t w[2][8];                             // a block is read while the one above is computed
+        lk_read(w[(kLKStep - 1) & 1], row + at, kLKStep - 1);
 #pragma unroll
-    for (int i = 0; i < 8; i++) ring[u].w[i] = 0;
-    const int vb = (int)G - 1 - u;
-    if (vb >= 0 && (uint32_t)vb < nb) ring[u] = ld_blk(k.base + 32ull * (uint32_t)vb);
-  }
-  uint32_t c[16];
-#pragma unroll
-  for (int i = 0; i < 16; i++) c[i] = 0;
-  uint32_t c3[16];                                    // component 3's state (unused with 2 components)
-#pragma unroll
-  for (int i = 0; i < 16; i++) c3[i] = 0;
-  // all iterations but the last (block 0, the bytes before the key's start masked)
-  const uint32_t M = G - 1;
-  for (uint32_t it0 = 0; it0 < M; it0 += kLKDepth) {
-#pragma unroll
-    for (int u = 0; u < kLKDepth; ++u) {
-      const uint32_t it = it0 + (uint32_t)u;
-      if (it >= M) break;
-      const uint32_t vb = G - 1 - it;
-      Blk w = ring[u];
-      if (it + kLKDepth < G) {
-        const uint32_t vb2 = vb - kLKDepth;
-        if (vb2 < nb) ring[u] = ld_blk(k.base + 32ull * vb2);
-      }
-      if (vb < nb) {
-        if (vb + 1 == nb) blk_keep_below(w, k.tail, mt);   // bytes after the key's end
-        lk_block<NCOMP>(w, sh, nxt0, c, c3, rc);
+        for (int b = kLKStep - 1; b >= 0; --b) {
+          if (b) lk_read(w[(b - 1) & 1], row + at, b - 1);
+          // (warp-uniform: false only for the blocks above the longest key's last, in the group's first step)
+          if (kLKStep * s + b < G) net.step((kLKStep * j + b) % P, w[b & 1]);
+        }
+        __syncwarp();
+        if (s >= (uint32_t)kStages) lk_copy_step(copy, base + at, s - kStages);
+        cp_async_commit();
       }
     }
+    if (s0 == 0) break;
   }
-  {                                                   // the last iteration: block 0 of every key
-    static_assert(kLKDepth == 1 || kLKDepth == 2, "the last iteration's ring slot: depths 1 and 2");
-    Blk w = ring[0];
-    if constexpr (kLKDepth == 2) {
-      if (M & 1u) w = ring[kLKDepth - 1];
-    }
-    if (nb) {
-      if (nb == 1) blk_keep_below(w, k.tail, mt);
-      blk_zero_below(w, k.a, mt);
-      lk_block<NCOMP>(w, sh, nxt0, c, c3, rc);
-    }
-  }
-  uint64_t sig = 0;
-  if (k.valid && !k.edge) sig_out[k.kq] = sig = lk_finish<NCOMP>(c, c3, k.a, inv32, rc);
-  if (__any_sync(kFull, k.edge))
-    if (k.edge) sig_out[k.kq] = sig = lk_edge_key<NCOMP, kLKWarps, kLKDepth, BATCH, Unique>(k, lim_lo, lim_hi, inv32, mt, rc);
-  return sig;
+  net.put(st);
 }
 
 // What a kernel does with each group's signatures besides writing them out:
-// nothing (LKNoPost), or a probe of a hash table (the whole join's fused
-// pass).  kScratch: shared-memory bytes a warp needs for it.
+// nothing (LKNoPost), or the insertion into a hash table (the build's pass
+// over R).
 struct LKNoPost {
-  static constexpr size_t kScratch = 0;
-  __device__ __forceinline__ void init(uint8_t*, const uint4*) {}
   __device__ __forceinline__ void group(uint64_t, uint64_t, bool) {}
-  __device__ __forceinline__ void finish() {}
 };
 
-// The window of keys starting at key wb (keys below k_hi): returns its key
+// The window of at most win keys starting at key wb (keys below k_hi): returns its key
 // count and sets *wa to its first row in the relation.  In a batch the keys are
 // virtual rows (the joins' row ranges back to back) and a window ends with its
 // join's rows, so that its keys are consecutive rows of the relation.
 template <bool BATCH>
 __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, int nj, int s_side, uint64_t wb,
-                                              uint64_t k_hi, uint64_t* wa) {
+                                              uint64_t k_hi, uint32_t win, uint64_t* wa) {
   uint64_t lim = k_hi;
   *wa = wb;
   if constexpr (BATCH) {
@@ -506,24 +541,59 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
     if (v0 + (e - b) < lim) lim = v0 + (e - b);
   }
   const uint64_t left = lim - wb;
-  return left < (uint64_t)kLKWin ? (uint32_t)left : (uint32_t)kLKWin;
+  return left < win ? (uint32_t)left : win;
 }
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
 // relation): equal counts below kLKSearchFrom keys, else equal shares of the
 // work, key bytes + kLKKeyCost per key (in a batch, over the joins' keys back
 // to back).  Whole warp.
-template <bool BATCH>
+template <bool BATCH, int kWarps>
 __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, int nj, int s_side,
                                               const uint64_t* __restrict__ off, uint64_t n, uint64_t warp,
                                               uint64_t nwarps, uint64_t* lo, uint64_t* hi) {
+  if (n <= 32 * nwarps) {                            // at most one group per warp
+    const uint64_t u = (warp % kWarps) * gridDim.x + warp / kWarps;   // neighbouring groups on different SMs
+    *lo = 32 * u < n ? 32 * u : n;
+    *hi = 32 * u + 32 < n ? 32 * u + 32 : n;
+    return;
+  }
   if (n < kLKSearchFrom) {
     *lo = (uint64_t)((unsigned __int128)n * warp / nwarps);
     *hi = (uint64_t)((unsigned __int128)n * (warp + 1) / nwarps);
     return;
   }
   if constexpr (!BATCH) {
-    warp_key_range(off, n, warp, nwarps, lo, hi, kLKKeyCost);
+    // lanes 0 and 1 look for the two cuts by secant steps from the cut by count: where key lengths are
+    // alike all along the relation two or three loads in sequence find a key whose start is off by less
+    // than a 64th of a share, against five of the search's for each cut.  (A cut depends on its number
+    // alone, so neighbouring warps agree on it.)
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t base = __ldg(off), total = __ldg(off + n) - base + kLKKeyCost * n;
+    const uint64_t w = warp + (lane & 1u);
+    const uint64_t t = (uint64_t)((unsigned __int128)total * w / nwarps);
+    const double per = (double)total / (double)n;     // work per key, > 0
+    uint64_t cut = (uint64_t)((unsigned __int128)n * w / nwarps);
+    bool found = cut == 0 || cut >= n;
+    for (int it = 0; it < 3 && !__all_sync(kFull, found); ++it) {
+      if (!found) {
+        const double d = (double)t - (double)(__ldg(off + cut) - base + kLKKeyCost * cut);
+        if (fabs(d) * 64.0 * (double)nwarps <= (double)total) {
+          found = true;
+        } else {
+          const double c = (double)cut + rint(d / per);
+          cut = c <= 0.0 ? 0 : (c >= (double)n ? n : (uint64_t)c);
+          if (cut == 0 || cut == n) cut = cut ? n - 1 : 1;   // (n is large here)
+        }
+      }
+    }
+    const uint64_t c0 = __shfl_sync(kFull, cut, 0), c1 = __shfl_sync(kFull, cut, 1);
+    const bool f0 = __shfl_sync(kFull, (int)found, 0), f1 = __shfl_sync(kFull, (int)found, 1);
+    auto search = [&](uint64_t v) -> uint64_t {
+      return warp_lower_bound(off, n, base + (uint64_t)((unsigned __int128)total * v / nwarps), kLKKeyCost);
+    };
+    *lo = f0 ? c0 : search(warp);
+    *hi = warp + 1 >= nwarps ? n : (f1 ? c1 : search(warp + 1));
   } else {
     const uint64_t total = s_side ? vcost_of_join<true>(J, nj, kLKKeyCost) : vcost_of_join<false>(J, nj, kLKKeyCost);
     auto cut = [&](uint64_t w) -> uint64_t {
@@ -548,62 +618,103 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
                                                                 uint64_t* __restrict__ sig_out,
                                                                 const BatchJoin* __restrict__ J, int nj, int s_side,
                                                                 Post post = Post()) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t* red = reinterpret_cast<uint32_t*>(smem);
-  uint16_t* inv32 = reinterpret_cast<uint16_t*>(smem + kRedBytes);
-  uint4* mt = reinterpret_cast<uint4*>(smem + kRedBytes + 1024);
-  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kRedBytes + 1024 + kSmemLKMasks);
-  post.init(smem + kRedBytes + 1024 + kSmemLKMasks + kLKWarps * sizeof(LKWarp) + (threadIdx.x >> 5) * Post::kScratch,
-            reinterpret_cast<const uint4*>(smem + kRedBytes + 1024));
-  lk_fill_masks(mt);
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)   // the x^-32 multiply table (512 entries)
-    reinterpret_cast<uint32_t*>(inv32)[i] = reinterpret_cast<const uint32_t*>(g_const + 16 * 512)[i];
+  extern __shared__ __align__(128) uint8_t smem[];
+  constexpr int kStages = kLKDepth / kLKStep;
+  static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
+  constexpr size_t kLines = lk_line_bytes(kLKWarps, kLKDepth);
+  uint16_t* inv = reinterpret_cast<uint16_t*>(smem + kLines);
+  uint4* mt = reinterpret_cast<uint4*>(smem + kLines + kSmemLKInv);
+  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kLines + kSmemLKInv + kSmemLKMasks);
   const int wib = threadIdx.x >> 5;
+  const uint32_t lane = threadIdx.x & 31u;
   LKWarp& W = warps[wib];
   // the warp's keys and its first window's offsets first, so that their loads overlap the tables' copy
   const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
   const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
   uint64_t k_lo, k_hi;
-  lk_warp_range<BATCH>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
-  uint64_t wa = 0;                                  // the current window: first row and key count
-  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, &wa) : 0u;
+  lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
+  uint64_t bytes;                                   // the relation's (or batch side's) key bytes
+  if constexpr (BATCH) bytes = s_side ? __ldg(&J[nj].vbs) : __ldg(&J[nj].vbr);
+  else bytes = __ldg(off + n) - __ldg(off);
+  const uint32_t win = bytes >= kLKNarrowFrom * n ? kLKNarrowWin : kLKWin;
+  uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
+  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, win, &wa) : 0u;
   if (wn) lk_prefetch_window(W, off, wa, wa + wn);
-  // readable bytes of the arena: from its start to the 16-byte boundary after the relation's last key byte
-  uint64_t rows_all = n;
-  if constexpr (BATCH) rows_all = s_side ? __ldg(&J[nj].s_end) : __ldg(&J[nj].r_end);
-  const uint8_t* lim_lo = arena;
-  const uint8_t* lim_hi = arena + ((__ldg(off + rows_all) + 15) & ~15ull);
-  for (int i = threadIdx.x; i < kRedWords / 4; i += blockDim.x)   // the reduction tables, from their image
-    reinterpret_cast<uint4*>(red)[i] = g_red_img[i];
+  lk_fill_masks(mt);
+  for (int i = threadIdx.x; i < (int)(kSmemLKInv / 16); i += blockDim.x)
+    reinterpret_cast<uint4*>(inv)[i] = g_inv[i];
+  // the reduction tables: line b is 16 copies of T16[b], then 16 of T24[b]
+  for (int i = threadIdx.x; i < 256 * 8; i += blockDim.x)
+    *reinterpret_cast<uint4*>(smem + (i >> 3) * kLKPitch + (i & 7) * 16) = g_red_img[(i >> 3) * 16 + (i & 4) * 2 + (i & 3)];
   __syncthreads();
   if (k_lo >= k_hi) return;
-  using Cursor = typename std::conditional<AT400, RedCursorAt400, RedCursor>::type;
-  Cursor rc;
-  if constexpr (AT400) rc = red_cursor_at400(); else rc = red_cursor(red);
+  const LKCursor<AT400> rc(smem);
 
-  for (uint64_t wb = k_lo; wb < k_hi;) {
-    wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, &wa);   // as prefetched
-    cp_async_wait_all();                            // the window's offsets
-    __syncwarp();
-    lk_sort_window(W, wn, reinterpret_cast<uintptr_t>(arena));
-    const uint32_t ng = (wn + 31) / 32;
-    for (uint32_t g = 0; g < ng; ++g) {
-      LKKey k;
-      const uint32_t G = lk_load_group(k, W, wb, g, arena, lim_lo, lim_hi);
-      if (g + 1 == ng) {                            // the window's offsets are free: fetch the next ones
-        __syncwarp();
-        if (wb + wn < k_hi) {
-          uint64_t na;
-          const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, &na);
-          lk_prefetch_window(W, off, na, na + nn);
-        }
+  uint8_t* stages = smem + lk_stage_base<kStages>((uint32_t)wib);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(stages);
+  const uint32_t row = base + lane * kLKPitch + ((lane & 7u) << 4);
+  uint32_t g = 0, ng = 0;
+  LKKey k, k2;
+  LKCopy copy;
+  // The warp's next group into k2, its first steps requested; returns its block count, 0 when there is
+  // none.  The stages are empty and serve as scratch before they are filled.
+  auto next_group = [&]() -> uint32_t {
+    if (g == ng) {                                    // the next window, as prefetched
+      if (ng) {
+        wb += wn;
+        if (wb >= k_hi) return 0u;
+        wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, win, &wa);
       }
-      const uint64_t sig = lk_group<NCOMP, kLKWarps, kLKDepth, BATCH, Post>(k, G, lim_lo, lim_hi, inv32, mt, sig_out, rc);
-      post.group(k.kq, sig, k.valid);
+      g = 0;
+      ng = (wn + 31) / 32;
+      cp_async_wait_all();
+      __syncwarp();
+      lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena));
     }
-    wb += wn;
+    const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena);
+    if (++g == ng) {                                  // the window's offsets are free: fetch the next ones
+      __syncwarp();
+      if (wb + wn < k_hi) {
+        uint64_t na;
+        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, win, &na);
+        lk_prefetch_window(W, off, na, na + nn);
+      }
+    }
+    lk_copy_setup(copy, k2, base);
+    const uint32_t S = (G2 + kLKStep - 1) / kLKStep;
+#pragma unroll
+    for (uint32_t u = 0; u < (uint32_t)kStages; ++u) {
+      if (u < S) lk_copy_step(copy, base + (S - 1 - u) % kStages * kLKStageBytes, S - 1 - u);
+      cp_async_commit();
+    }
+    return G2;
+  };
+  for (uint32_t G2 = next_group(); G2;) {
+    const uint32_t G = G2;
+    k = k2;
+    uint32_t st[kLKState];
+    if (G <= (uint32_t)kLKShort) {
+      cp_async_wait_but<0>();
+      __syncwarp();
+      lk_trim(k, row, 0, mt);
+      lk_short_blocks<NCOMP>(st, k, G, row);
+      __syncwarp();
+    } else {
+      lk_long_blocks<QNet<NCOMP>, kStages>(st, k, G, copy, base, row, mt);
+    }
+    // the next group's first steps are in flight while this one's signatures are finished
+    G2 = next_group();
+    uint64_t sig;
+    if (G <= (uint32_t)kLKShort) {
+      sig = lk_finish<NCOMP>(st, k.a, inv + kInvEntries, rc);
+    } else {
+      QNet<NCOMP> net;
+      net.get(st);
+      sig = net.finish(k.a, inv, rc);
+    }
+    if (k.valid) sig_out[k.kq] = sig;
+    post.group(k.kq, sig, k.valid);
   }
-  post.finish();
   cp_async_wait_all();
 }
 

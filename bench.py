@@ -560,8 +560,8 @@ def run_gpu(args):
         wev[k][1].record(stream)
         flush_l2(stream)                                # between steps, outside the steps' events
     # ... then K joins as the four calls, with events between the kernels (the per-kernel split),
-    # each followed (after an L2 flush) by the build without given signatures, whose kernel computes
-    # R's signatures and inserts them (the whole join's pass over R, the table clear included)
+    # each followed (after an L2 flush) by the build without given signatures (the whole join's work on
+    # R: table clear, signatures, inserts)
     bev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     table_cap = 0
     for k in range(args.steps):
@@ -819,7 +819,7 @@ def run_gpu(args):
                    + total_pairs * (16 + 4 + 8)                        # offR pair, idR, output pair
                    + 2 * verified_bytes),                              # R and S key bytes compared
     }
-    # the whole join's R pass: signatures and inserts in one kernel, after the table clear
+    # the whole join's work on R: signatures and inserts, after the table clear
     phase_ms["sig_build_R"] = [a.elapsed_time(b) for a, b in bev]
     alg["sig_build_R"] = wl.R.nbytes + 8 * (m + 1) + 8 * m + 16 * m + 16 * table_cap
     phases = PH + ("sig_build_R",)
@@ -883,7 +883,7 @@ def run_gpu(args):
                 "h2d_pinned_gbs": h2d_gbs,
                 "copy_bound_ms": (h2d + d2h) / (h2d_gbs * 1e9) * 1e3,
                 "path": "stream.HostStreamJoin: pinned host R and S, S copied in chunks under the kernels"},
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": 4 * args.steps,
         "roofline": {"bound": "hbm", "kernel": KERNEL_NAMES[dom], "achieved": kernels[dom]["gbps"], "peak": hbm,
                      "peak_kind": f"{peak_kind} (copy bandwidth, burst)", "unit": "GB/s",
                      "frac": kernels[dom]["frac_hbm"], "traffic": traffic,
@@ -912,7 +912,7 @@ def run_gpu(args):
 
 
 # revision of each kernel's code; profiles/traffic.json holds counters per revision
-KERNEL_REVS = {"sig_key_kernel": "v5", "build_kernel": "v8", "verify_kernel": "v17", "sig_key_kernel+build": "v2"}
+KERNEL_REVS = {"sig_key_kernel": "v5", "build_kernel": "v8", "verify_kernel": "v17", "sig_key_kernel+build": "v3"}
 KERNEL_NAMES = {"sig_R": "sig_key_kernel", "sig_S": "sig_key_kernel", "build": "build_kernel",
                 "verify": "verify_kernel", "sig_build_R": "sig_key_kernel+build"}
 

@@ -246,20 +246,6 @@ __global__ void build_kernel(Slot* __restrict__ slots, uint64_t mask, const uint
   }
 }
 
-// The build fused into the signature kernel over R (as_join_build without
-// given signatures): after each group of 32 keys has its signatures, every
-// lane inserts its key.  The probe runs in a later kernel, so it never sees a
-// slot whose signature word is not yet written.
-struct BuildPost {
-  Slot* slots;
-  uint64_t mask;
-  const uint64_t* offR;
-  uint32_t* flags;
-  __device__ __forceinline__ void group(uint64_t kq, uint64_t sig, bool valid) {
-    if (valid) table_insert(slots, mask, sig, __ldg(offR + kq + 1) - __ldg(offR + kq), kq, flags);
-  }
-};
-
 // ----------------------------------------------------------------------------
 // Probe: table walk + byte-exact verification + output compaction.  The S
 // signatures come from sig_kernel; this kernel needs no large shared memory,
@@ -1003,17 +989,6 @@ static as_status ensure_device(DeviceState** out) {
           (e = key_kernel_attrs<true, 4, true>()) != cudaSuccess ||
           (e = key_kernel_attrs<false, 4, true>()) != cudaSuccess)
         return cuda_fail(e, "kernel attribute");
-      {
-        constexpr LKShape k = kLKShapes[0];
-        const int smem = (int)lk_smem_bytes(k.warps, k.depth);
-        if ((e = cudaFuncSetAttribute(
-                 reinterpret_cast<const void*>(sig_key_kernel<true, 4, k.warps, k.depth, false, BuildPost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(
-                 reinterpret_cast<const void*>(sig_key_kernel<false, 4, k.warps, k.depth, false, BuildPost>),
-                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-          return cuda_fail(e, "kernel attribute");
-      }
     }
     // where dynamic shared memory starts (the tables are its first bytes)
     if ((e = cudaFuncSetAttribute(dyn_smem_base_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemSig)) !=
@@ -1126,39 +1101,12 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
   return AS_OK;
 }
 
-// R's signatures with the build fused in (BuildPost): the signature kernel
-// (shape 0) inserts each group of keys into the cleared table slots[0..mask].
-static as_status launch_sig_build(const DeviceState* d, const uint8_t* arenaR, const uint64_t* offR, uint64_t m,
-                                  uint64_t* sigR, Slot* slots, uint64_t mask, uint32_t* flags, cudaStream_t s,
-                                  int max_blocks) {
-  if (m == 0) return AS_OK;
-  BuildPost post;
-  post.slots = slots;
-  post.mask = mask;
-  post.offR = offR;
-  post.flags = flags;
-  constexpr LKShape k = kLKShapes[0];
-  const uint64_t want = (m + 31) / 32;
-  const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
-  const size_t smem = lk_smem_bytes(k.warps, k.depth);
-  if (d->tables_at400)
-    sig_key_kernel<true, 4, k.warps, k.depth, false, BuildPost>
-        <<<blocks, 32 * k.warps, smem, s>>>(arenaR, offR, m, sigR, nullptr, 0, 0, post);
-  else
-    sig_key_kernel<false, 4, k.warps, k.depth, false, BuildPost>
-        <<<blocks, 32 * k.warps, smem, s>>>(arenaR, offR, m, sigR, nullptr, 0, 0, post);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "signature and build kernel launch");
-  return AS_OK;
-}
-
 // Blocks of the passes over R (m keys) and S (n keys) of a join whose two passes
 // run at the same time.  A block of the signature kernel takes a whole SM, so
 // where a pass has at most four groups of 32 keys per warp of the device the
-// SMs are divided and both run beside each other.  R's pass, which goes on to
-// insert its keys, gets a warp for every group if that takes no more than a
-// quarter of the SMs (10k x 100k keys of 64-256 bytes: 23 us on 14 SMs, 12 us
-// on 20), else its share by key count.  Larger passes take all SMs one after
+// SMs are divided and both run beside each other.  R's pass, which the build
+// waits for, gets a warp for every group if that takes no more than a quarter
+// of the SMs, else its share by key count.  Larger passes take all SMs one after
 // the other, which needs no guess about the keys' lengths.
 static void split_sms(int sms, uint64_t m, uint64_t n, int* blocks_r, int* blocks_s) {
   const int warps = kLKShapes[0].warps;
@@ -1369,7 +1317,10 @@ size_t as_join_ws_bytes(uint64_t m, uint64_t n, float load_factor) {
 
 }  // extern "C"
 
-// as_join_build's work; max_blocks: blocks of the pass over R (0: one per SM)
+// as_join_build's work; max_blocks: most blocks of the signature kernel over R (0: one per SM).  R's
+// signatures and the insertions are two kernels: inserting each group right after its signatures makes
+// the signature kernel's 16 warps per SM wait for the table (1M keys of 256-1024 bytes: 326 us against
+// 160 + 55 us apart).
 static as_status build_impl(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
                             const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
                             as_stream stream, int max_blocks) {
@@ -1396,11 +1347,12 @@ static as_status build_impl(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR
   if ((e = cudaMemsetAsync(slots, 0xFF, cap * 16, s)) != cudaSuccess) return cuda_fail(e, "table clear");
   if ((e = cudaMemsetAsync(flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
   const uint64_t* sigR = d_sigR;
-  if (!sigR && m > 0) {                              // R's signatures with the build in the same kernel
-    st = launch_sig_build(d, d_arenaR, d_offR, m, sig_ws, slots, cap - 1, flags, s, max_blocks > 0 ? max_blocks : d->sms);
+  if (!sigR && m > 0) {
+    st = launch_sig(d_arenaR, d_offR, m, sig_ws, s, 4, 0, max_blocks);
     if (st != AS_OK) return st;
     sigR = sig_ws;
-  } else if (m > 0) {
+  }
+  if (m > 0) {
     uint64_t blocks = (m + 255) / 256;
     const uint64_t lim = (uint64_t)d->sms * 16;
     if (blocks > lim) blocks = lim;

@@ -516,13 +516,6 @@ __device__ __forceinline__ void lk_long_blocks(uint32_t (&st)[kLKState], const L
   net.put(st);
 }
 
-// What a kernel does with each group's signatures besides writing them out:
-// nothing (LKNoPost), or the insertion into a hash table (the build's pass
-// over R).
-struct LKNoPost {
-  __device__ __forceinline__ void group(uint64_t, uint64_t, bool) {}
-};
-
 // The window of at most win keys starting at key wb (keys below k_hi): returns its key
 // count and sets *wa to its first row in the relation.  In a batch the keys are
 // virtual rows (the joins' row ranges back to back) and a window ends with its
@@ -612,12 +605,11 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
 // The signatures of n keys: the rows of a relation (BATCH false), or the
 // virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
 // describe the joins, and sig_out is indexed by virtual row).
-template <bool AT400, int NCOMP, int kLKWarps, int kLKDepth, bool BATCH, class Post = LKNoPost>
+template <bool AT400, int NCOMP, int kLKWarps, int kLKDepth, bool BATCH>
 __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t* __restrict__ arena,
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
-                                                                const BatchJoin* __restrict__ J, int nj, int s_side,
-                                                                Post post = Post()) {
+                                                                const BatchJoin* __restrict__ J, int nj, int s_side) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int kStages = kLKDepth / kLKStep;
   static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
@@ -713,7 +705,6 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       sig = net.finish(k.a, inv, rc);
     }
     if (k.valid) sig_out[k.kq] = sig;
-    post.group(k.kq, sig, k.valid);
   }
   cp_async_wait_all();
 }

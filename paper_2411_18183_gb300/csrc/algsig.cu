@@ -255,6 +255,7 @@ __global__ void build_kernel(Slot* __restrict__ slots, uint64_t mask, const uint
 
 constexpr int kVThreads = 256;
 constexpr int kVWarps = kVThreads / 32;
+constexpr int kVBlocks = 4;     // blocks per SM of the probe kernels
 constexpr int kVStage = 64;     // verified pairs staged per warp before one atomic append
 
 struct VerifyParams {
@@ -453,168 +454,321 @@ __device__ __forceinline__ void flush_stage(const Stage& st, uint32_t np, const 
   __syncwarp();
 }
 
-// flush for join j of a batch: its counter, region and capacity
-__device__ __forceinline__ void flush_stage_join(const Stage& st, uint32_t np, const VerifyParams& P, int j) {
-  const int lane = threadIdx.x & 31;
-  unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(P.counts + j, (unsigned long long)np);
-  base = __shfl_sync(kFull, base, 0);
-  const uint64_t off = __ldg(&P.J[j].pair_off), cap = __ldg(&P.J[j].pair_cap);
-  const uint64_t rb = __ldg(&P.J[j].r_begin), sb = __ldg(&P.J[j].s_begin);
-  for (uint32_t i = (uint32_t)lane; i < np; i += 32) {
-    const unsigned long long idx = base + i;
-    if (idx < cap) reinterpret_cast<uint64_t*>(P.pairs)[off + idx] = pair_ids(st.r[i], st.s[i], P.idR, P.idS, rb, sb);
+// Candidates of a warp's S rows wait in a queue in shared memory and are
+// verified 32 at a time: their R offsets and ids are loaded by 32 lanes at
+// once, and four candidates are compared at a time, eight lanes to each (long
+// keys: one, by the whole warp).  (With each candidate verified by the warp as
+// it was found, its R offset and its bytes were two waits in sequence, and the
+// set-up was repeated per candidate: 1.72 ms for the 5M candidates of 256-1024
+// bytes of the large join, 1.3 ms now; with the queue drained while lanes were
+// still on their way through the table, the live registers spilled and cost
+// that gain.)
+struct Cand {
+  uint4 a;                   // S start (64 bits), S row (64 bits); while verified: the aligned bases of S and R
+  uint4 b;                   // R row, length (32 bits), join of a batch, lane; while verified: end, alignment, row, join or lane
+};
+constexpr uint32_t kVDrain = 32;             // candidates verified at a time
+constexpr uint32_t kVQueue = 80;             // a probe step (32 new ones at most) runs while 48 or fewer wait
+struct CandQueue {
+  Cand q[kVQueue];
+  uint64_t ids[kVDrain];     // the ids of the candidates being verified
+};
+// Chunks of each lane in flight: with 4 blocks of 64 registers two fit without spills (large join, blocks x
+// chunks: 4 x 2 2.83 ms, 3 x 4 2.85, 3 x 3 2.96, 4 x 3 3.02, 4 x 1 3.11)
+constexpr int kVAhead = 2;
+// Longest key compared by eight lanes: the whole warp's 512 bytes in a row take fewer requests (400k
+// candidates of 2-8 KB: 821 us with eight lanes, 750 us with the warp, when the line was drawn; 679 us now),
+// eight lanes fewer instructions and waits per candidate (5M of 256-1024 bytes: 1.3 against 1.7 ms)
+constexpr uint32_t kVFourMax = 2048;
+
+// the candidates of a probe step (lanes with `cand`) to the end of the queue
+__device__ __forceinline__ void queue_push(Cand* q, uint32_t& cnt, bool cand, uint64_t start, uint64_t srow,
+                                           uint32_t row, uint32_t l32, uint32_t jn) {
+  const uint32_t m = __ballot_sync(kFull, cand);
+  if (cand) {
+    Cand& e = q[cnt + (uint32_t)__popc(m & lanemask_lt())];
+    e.a = make_uint4((uint32_t)start, (uint32_t)(start >> 32), (uint32_t)srow, (uint32_t)(srow >> 32));
+    e.b = make_uint4(row, l32, jn, threadIdx.x & 31u);
   }
+  cnt += (uint32_t)__popc(m);
   __syncwarp();
+}
+
+__device__ __forceinline__ uint4 ld16_stream(const uint8_t* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ const uint8_t* ptr_of(uint32_t lo, uint32_t hi) {
+  return reinterpret_cast<const uint8_t*>((uint64_t)lo | ((uint64_t)hi << 32));
+}
+
+// the bits in which 16 S bytes differ from the 16 R bytes that start d bytes into the 32 at ra, rb
+__device__ __forceinline__ uint4 chunk_diff(const uint4& sv, const uint4& ra, const uint4& rb, uint32_t d) {
+  const bool w2 = d & 8u, w1 = d & 4u;                 // the word part of d, by selects (it differs between lanes)
+  const uint32_t sh = 8u * (d & 3u);
+  const uint32_t t0 = w2 ? ra.z : ra.x, t1 = w2 ? ra.w : ra.y, t2 = w2 ? rb.x : ra.z, t3 = w2 ? rb.y : ra.w;
+  const uint32_t t4 = w2 ? rb.z : rb.x, t5 = w2 ? rb.w : rb.y;
+  const uint32_t u0 = w1 ? t1 : t0, u1 = w1 ? t2 : t1, u2 = w1 ? t3 : t2, u3 = w1 ? t4 : t3, u4 = w1 ? t5 : t4;
+  return make_uint4(__funnelshift_r(u0, u1, sh) ^ sv.x, __funnelshift_r(u1, u2, sh) ^ sv.y,
+                    __funnelshift_r(u2, u3, sh) ^ sv.z, __funnelshift_r(u3, u4, sh) ^ sv.w);
+}
+
+// Compare the keys of the candidates from r on at q that are in `todo`, 2^lg
+// lanes to a candidate; returns a bit per candidate whose keys differ.  Lane i
+// of a candidate's lanes takes the 16-byte S chunks i, i + 2^lg, ... and the two
+// aligned R chunks under each, kVAhead at a time; the last chunk, where it is
+// partial, is compared apart.  Only aligned chunks that hold a key byte are read.
+template <uint32_t lg>
+__device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint32_t todo,
+                                                 const uint4* __restrict__ emask) {
+  const uint32_t lane = threadIdx.x & 31u, li = lane & ((1u << lg) - 1u), c = r + (lane >> lg);
+  const uint4 a = q[c].a;
+  const uint2 b = *reinterpret_cast<const uint2*>(&q[c].b);
+  const uint32_t kend = (todo >> (c & 31u)) & 1u ? b.x : 0u, sa = b.y & 15u, d = (b.y >> 8) & 15u;
+  const uint32_t nfull = kend >> 4, rem = kend & 15u;  // whole chunks from S's aligned base on, and the rest
+  const uint8_t* pS = ptr_of(a.x, a.y) + 16u * li;
+  const uint8_t* pR = ptr_of(a.z, a.w) + 16u * li;
+  uint32_t diff = 0;
+  uint4 ts = make_uint4(0, 0, 0, 0), ta = ts, tb = ts;  // the partial chunk
+  const bool tail = rem != 0u && ((nfull ^ li) & ((1u << lg) - 1u)) == 0u;
+  if (tail) {
+    const uint32_t off = (nfull - li) << 4;
+    ts = ld16_stream(pS + off);
+    if ((nfull << 4) + 16u > sa + d) ta = ld16(pR + off);
+    if (16u < rem + d) tb = ld16(pR + off + 16);
+  }
+  const uint32_t nmax = __reduce_max_sync(kFull, nfull);
+  for (uint32_t c0 = 0; c0 < nmax; c0 += (uint32_t)kVAhead << lg) {   // warp-uniform
+    uint4 sv[kVAhead], ra[kVAhead], rb[kVAhead];
+#pragma unroll
+    for (int u = 0; u < kVAhead; ++u) {
+      const uint32_t ci = c0 + ((uint32_t)u << lg) + li;
+      sv[u] = ra[u] = rb[u] = make_uint4(0, 0, 0, 0);
+      if (ci < nfull) {
+        sv[u] = ld16_stream(pS);
+        if (ci > 0u || sa + d < 16u) ra[u] = ld16(pR);
+        if (ci + 1u < nfull || rem + d > 0u) rb[u] = ld16(pR + 16);
+      }
+      pS += 16u << lg;
+      pR += 16u << lg;
+    }
+#pragma unroll
+    for (int u = 0; u < kVAhead; ++u) {
+      uint4 x = chunk_diff(sv[u], ra[u], rb[u], d);
+      if (u == 0 && c0 == 0u) {                        // the first chunk: bytes before the key
+        const uint4 m = emask[li == 0u ? sa : 0u];
+        x.x &= ~m.x; x.y &= ~m.y; x.z &= ~m.z; x.w &= ~m.w;
+      }
+      diff |= (x.x | x.y) | (x.z | x.w);
+    }
+  }
+  if (__any_sync(kFull, tail)) {
+    const uint4 x = chunk_diff(ts, ta, tb, d);
+    const uint4 mh = emask[tail ? rem : 0u], ml = emask[nfull == 0u ? sa : 0u];
+    diff |= (x.x & mh.x & ~ml.x) | (x.y & mh.y & ~ml.y) | (x.z & mh.z & ~ml.z) | (x.w & mh.w & ~ml.w);
+  }
+  if (!__any_sync(kFull, diff != 0u)) return 0u;
+  return __reduce_or_sync(kFull, diff != 0u ? 1u << c : 0u);
+}
+
+// Verify the nc (at most 32) candidates at q and put out what the mode asks for
+// each verified one; returns a bit per lane that queued a verified candidate.
+// Between its parts the candidates' fields are in shared memory, not in
+// registers: the comparison needs those for the bytes in flight.
+template <bool BATCH, bool INNER>
+__device__ __forceinline__ uint32_t queue_verify(Cand* q, uint64_t* ids, uint32_t nc, const VerifyParams& P,
+                                                 const uint4* emask) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const int mode = BATCH || INNER ? (int)AS_JOIN_INNER : P.mode;
+  const bool pairs = mode == AS_JOIN_INNER || mode == AS_JOIN_OUTER_S || mode == AS_JOIN_OUTER_R ||
+                     mode == AS_JOIN_SIG_ONLY;
+  const bool bytes = BATCH || mode != AS_JOIN_SIG_ONLY;   // signature-only: no byte comparison
+  uint32_t todo, bad = 0, lg = 3u;
+  {
+    const bool have = lane < nc;
+    uint64_t start = 0, srow = 0, rs = 0;
+    uint32_t row = 0, l32 = 0, tag = 0;
+    if (have) {
+      const uint4 a = q[lane].a, b = q[lane].b;
+      start = (uint64_t)a.x | ((uint64_t)a.y << 32);
+      srow = (uint64_t)a.z | ((uint64_t)a.w << 32);
+      row = b.x;
+      l32 = b.y;
+      tag = BATCH ? b.z : b.w;
+      rs = __ldg(P.offR + row);
+      if (pairs) {
+        uint64_t rb = 0, sb = 0;
+        if (BATCH) {
+          rb = __ldg(&P.J[tag].r_begin);
+          sb = __ldg(&P.J[tag].s_begin);
+        }
+        ids[lane] = pair_ids(row, srow, P.idR, P.idS, rb, sb);
+      }
+    }
+    const bool wide = have && l32 >= kNarrowLen;       // lengths that the slot's 32-bit field saturates
+    todo = __ballot_sync(kFull, have && !wide && bytes && l32 > 0u);
+    if (__any_sync(kFull, have && l32 > kVFourMax)) lg = 5u;
+    for (uint32_t wm = __ballot_sync(kFull, wide); wm; wm &= wm - 1u) {   // one by one, in 64-bit offsets
+      const int c = __ffs((int)wm) - 1;
+      const uint64_t rsc = __shfl_sync(kFull, rs, c), ssc = __shfl_sync(kFull, start, c);
+      const uint64_t sr = __shfl_sync(kFull, srow, c);
+      const uint32_t rr = __shfl_sync(kFull, row, c);
+      uint64_t ls = __ldg(P.offS + sr + 1) - ssc, lr = __ldg(P.offR + rr + 1) - rsc;
+      if (ls > P.cap_len) ls = P.cap_len;
+      if (lr > P.cap_len) lr = P.cap_len;
+      if (lr != ls || (bytes && !warp_equal_wide(P.arenaR, rsc, P.arenaS, ssc, ls))) bad |= 1u << c;
+    }
+    __syncwarp();
+    if (have) {
+      const uint8_t *pS = P.arenaS + start, *pR = P.arenaR + rs;
+      const uint32_t sa = (uint32_t)reinterpret_cast<uintptr_t>(pS) & 15u;
+      const uint32_t d = (uint32_t)(reinterpret_cast<uintptr_t>(pR) - sa) & 15u;
+      const uint64_t bS = reinterpret_cast<uint64_t>(pS - sa), bR = reinterpret_cast<uint64_t>(pR - sa - d);
+      q[lane].a = make_uint4((uint32_t)bS, (uint32_t)(bS >> 32), (uint32_t)bR, (uint32_t)(bR >> 32));
+      q[lane].b = make_uint4(sa + l32, sa | (d << 8), row, tag);
+    }
+    __syncwarp();
+  }
+  if (lg == 3u)
+    for (uint32_t r = 0; r < nc; r += 4u) bad |= compare_some<3>(q, r, todo, emask);
+  else
+    for (uint32_t r = 0; r < nc; ++r) bad |= compare_some<5>(q, r, todo, emask);
+  const bool eq = lane < nc && !((bad >> lane) & 1u);
+  const uint32_t row = q[lane].b.z, tag = q[lane].b.w;   // (defined where eq)
+  if (!BATCH && !INNER && eq && mode >= AS_JOIN_OUTER_R) atomicOr(P.matched + (row >> 5), 1u << (row & 31u));
+  if (pairs) {
+    uint32_t em = __ballot_sync(kFull, eq);
+    if (!BATCH) {
+      unsigned long long base = 0;
+      if (lane == 0 && em) base = atomicAdd(P.count, (unsigned long long)__popc(em));
+      base = __shfl_sync(kFull, base, 0) + (unsigned long long)__popc(em & lanemask_lt());
+      if (eq && base < P.cap) reinterpret_cast<uint64_t*>(P.pairs)[base] = ids[lane];
+    } else {
+      while (em) {                                    // one join's pairs at a time (nearly always all of them)
+        const uint32_t j = __shfl_sync(kFull, tag, __ffs((int)em) - 1);
+        const uint32_t mine = __ballot_sync(kFull, eq && tag == j);
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(P.counts + j, (unsigned long long)__popc(mine));
+        base = __shfl_sync(kFull, base, 0) + (unsigned long long)__popc(mine & lanemask_lt());
+        if (((mine >> lane) & 1u) && base < __ldg(&P.J[j].pair_cap))
+          reinterpret_cast<uint64_t*>(P.pairs)[__ldg(&P.J[j].pair_off) + base] = ids[lane];
+        em &= ~mine;
+      }
+    }
+  }
+  const uint32_t m = INNER || BATCH ? 0u : __reduce_or_sync(kFull, eq ? 1u << (tag & 31u) : 0u);
+  __syncwarp();
+  return m;
 }
 
 // BATCH: the S rows of a batch's joins; INNER: the plain inner join of one
 // table (no output mode to test per pair)
 template <bool BATCH, bool INNER = false>
-__global__ void __launch_bounds__(kVThreads, 4) verify_kernel(VerifyParams P) {
-  __shared__ Stage stage_all[kVWarps];
+__global__ void __launch_bounds__(kVThreads, kVBlocks) verify_kernel(const __grid_constant__ VerifyParams P) {
+  __shared__ CandQueue queue_all[kVWarps];
   __shared__ uint4 emask[17];
   fill_emask(emask);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  Stage& stage = stage_all[threadIdx.x >> 5];
-  uint32_t np = 0;                                   // staged pairs (warp-uniform)
-  int sj = -1;                                       // batch: join of the staged pairs
-  constexpr bool batch = BATCH;
-  const int mode = INNER ? (int)AS_JOIN_INNER : P.mode;
+  const uint32_t lane = threadIdx.x & 31u;
+  CandQueue& Q = queue_all[threadIdx.x >> 5];
+  uint32_t cnt = 0;                                  // candidates waiting
+  uint32_t matched = 0;                              // a bit per lane whose S row has a verified match
   const uint64_t ngroups = (P.n + 31) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * kVWarps;
-  for (uint64_t grp = (uint64_t)blockIdx.x * kVWarps + (threadIdx.x >> 5); grp < ngroups; grp += nwarps) {
+  constexpr bool kRows = !BATCH && !INNER;           // a group's rows may have to know their matches
+  bool resume = false;                               // a group was left with lanes on their way, for a full queue
+  volatile uint64_t saved[3];                        // then: the lane's place in its bucket sequence, and whether it goes on
+  for (uint64_t grp = (uint64_t)blockIdx.x * kVWarps + (threadIdx.x >> 5); grp < ngroups;) {
     const uint64_t vi = grp * 32 + (uint64_t)lane;   // virtual S row (= actual row for one join)
-    bool live = vi < P.n;
-    const Slot* slots = P.slots;
-    uint64_t mask = P.mask;
-    uint64_t i = vi;
-    int jn = 0;                                      // batch: join of the lane's S row
-    if (batch && live) {
-      jn = join_of_virtual<true>(P.J, P.nj, vi);
-      i = __ldg(&P.J[jn].s_begin) + (vi - __ldg(&P.J[jn].vs));
-      slots = P.slots + __ldg(&P.J[jn].slot_off);
-      mask = __ldg(&P.J[jn].mask);
-    }
-    uint64_t sig = 0, start = 0, len = 0, b = 0, steps = 0;
-    uint32_t l32 = 0;
-    bool matched = false;                            // the lane's S row has a verified match
-    const bool row_live = live;
-    if (live) {
-      sig = __ldg(P.sigS + vi);
-      start = __ldg(P.offS + i);
-      len = __ldg(P.offS + i + 1) - start;
-      if (len > P.cap_len) len = P.cap_len;
-      b = sig_hash(sig, len) & mask;
-      l32 = len32(len);
-    }
-    while (__any_sync(kFull, live)) {
-      bool cand = false;
-      uint32_t row = 0;
+    {
+      bool live = vi < P.n;
+      const Slot* slots = P.slots;
+      uint64_t mask = P.mask;
+      uint64_t i = vi;
+      uint32_t jn = 0;                               // batch: join of the lane's S row
+      if (BATCH && live) {
+        jn = (uint32_t)join_of_virtual<true>(P.J, P.nj, vi);
+        i = __ldg(&P.J[jn].s_begin) + (vi - __ldg(&P.J[jn].vs));
+        slots = P.slots + __ldg(&P.J[jn].slot_off);
+        mask = __ldg(&P.J[jn].mask);
+      }
+      uint64_t sig = 0, start = 0, b = 0, steps = 0;
+      uint32_t l32 = 0;
       if (live) {
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(slots + b));
-        if (v.y == kEmpty) {
-          live = false;
-        } else {
-          if (v.x == sig && (uint32_t)(v.y >> 32) == l32) {
-            cand = true;
-            row = (uint32_t)v.y;
-          }
-          b = (b + 1) & mask;
-          if (++steps > mask) live = false;
-          // a slot at an even index shares its 32-byte sector with the next one: look at that one
-          // too in this step (an L1 hit), unless this one was already a candidate
-          if (!cand && live && (b & 1u)) {
-            const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2*>(slots + b));
-            if (v2.y == kEmpty) {
-              live = false;
-            } else {
-              if (v2.x == sig && (uint32_t)(v2.y >> 32) == l32) {
-                cand = true;
-                row = (uint32_t)v2.y;
+        sig = __ldg(P.sigS + vi);
+        start = __ldg(P.offS + i);
+        uint64_t len = __ldg(P.offS + i + 1) - start;
+        if (len > P.cap_len) len = P.cap_len;
+        b = sig_hash(sig, len) & mask;
+        l32 = len32(len);
+      }
+      if (resume) {
+        b = saved[0];
+        steps = saved[1];
+        live = saved[2] != 0u;
+      }
+      do {
+        bool cand = false;
+        uint32_t row = 0;
+        if (live) {
+          const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(slots + b));
+          if (v.y == kEmpty) {
+            live = false;
+          } else {
+            if (v.x == sig && (uint32_t)(v.y >> 32) == l32) {
+              cand = true;
+              row = (uint32_t)v.y;
+            }
+            b = (b + 1) & mask;
+            if (++steps > mask) live = false;
+            // a slot at an even index shares its 32-byte sector with the next one: look at that one
+            // too in this step (an L1 hit), unless this one was already a candidate
+            if (!cand && live && (b & 1u)) {
+              const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2*>(slots + b));
+              if (v2.y == kEmpty) {
+                live = false;
+              } else {
+                if (v2.x == sig && (uint32_t)(v2.y >> 32) == l32) {
+                  cand = true;
+                  row = (uint32_t)v2.y;
+                }
+                b = (b + 1) & mask;
+                if (++steps > mask) live = false;
               }
-              b = (b + 1) & mask;
-              if (++steps > mask) live = false;
             }
           }
         }
-      }
-      uint32_t cm = __ballot_sync(kFull, cand);
-      while (cm) {                                   // verify candidates one by one, whole warp
-        const int j = __ffs(cm) - 1;
-        cm &= cm - 1;
-        const uint32_t rj = __shfl_sync(kFull, row, j);
-        const uint32_t lj = __shfl_sync(kFull, l32, j);   // the slot holds the same length
-        const uint64_t stj = __shfl_sync(kFull, start, j);
-        if (cm) {                                    // the next candidate's S bytes and R offset, ahead
-          const int j2 = __ffs(cm) - 1;
-          const uint64_t st2 = __shfl_sync(kFull, start, j2);
-          const uint32_t l2 = __shfl_sync(kFull, l32, j2);
-          const uint32_t r2 = __shfl_sync(kFull, row, j2);
-          const uint64_t o = 32u * (uint64_t)lane;   // one 32-byte sector per lane, the first 1 KB
-          if (o < (uint64_t)l2)                     // addresses inside the key only
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(P.arenaS + st2 + o));
-          if (lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(P.offR + r2));
-        }
-        const uint64_t rs = __ldg(P.offR + rj);
-        const bool verify = batch || mode != AS_JOIN_SIG_ONLY;   // signature-only: no byte comparison
-        bool eq;
-        if (lj < kNarrowLen) {
-          eq = !verify || warp_equal(P.arenaR + rs, P.arenaS + stj, lj, emask);
-        } else {                                      // lengths that the slot's 32-bit field saturates
-          const uint64_t ls = __shfl_sync(kFull, len, j);
-          uint64_t lr = __ldg(P.offR + rj + 1) - rs;
-          if (lr > P.cap_len) lr = P.cap_len;
-          eq = lr == ls && (!verify || warp_equal_wide(P.arenaR, rs, P.arenaS, stj, ls));
-        }
-        if (eq) {
-          const uint64_t srow = __shfl_sync(kFull, i, j);
-          if (lane == j) matched = true;
-          if (!batch && mode >= AS_JOIN_OUTER_R) {  // R-side modes: mark the R row
-            if (lane == 0) atomicOr(P.matched + (rj >> 5), 1u << (rj & 31u));
-            if (mode != AS_JOIN_OUTER_R) continue;   // rows, not pairs
-          }
-          if (!batch && (mode == AS_JOIN_SEMI || mode == AS_JOIN_ANTI)) continue;   // rows, not pairs
-          const int jj = __shfl_sync(kFull, jn, j);
-          if (batch && np && jj != sj) {              // the stage holds one join's pairs
-            flush_stage_join(stage, np, P, sj);
-            np = 0;
-          }
-          sj = jj;
-          if (lane == 0) {
-            stage.r[np] = rj;
-            stage.s[np] = srow;
-          }
-          __syncwarp();
-          if (++np == (uint32_t)kVStage) {
-            if (batch) flush_stage_join(stage, np, P, sj); else flush_stage(stage, np, P);
-            np = 0;
-          }
-        }
+        queue_push(Q.q, cnt, cand, start, i, row, l32, jn);
+        resume = __any_sync(kFull, live);
+      } while (resume && cnt <= kVQueue - kVDrain);
+      if (resume) {
+        saved[0] = b;
+        saved[1] = steps;
+        saved[2] = live ? 1u : 0u;
       }
     }
-    if (!batch && (mode == AS_JOIN_SEMI || mode == AS_JOIN_ANTI || mode == AS_JOIN_OUTER_S)) {
+    const bool flush = resume || kRows || grp + nwarps >= ngroups;
+    while (cnt >= kVDrain || (flush && cnt)) {
+      const uint32_t nc = cnt < kVDrain ? cnt : kVDrain;
+      cnt -= nc;
+      matched |= queue_verify<BATCH, INNER>(Q.q + cnt, Q.ids, nc, P, emask);
+    }
+    if (resume) continue;                            // the same group's next steps
+    if (kRows && (P.mode == AS_JOIN_SEMI || P.mode == AS_JOIN_ANTI || P.mode == AS_JOIN_OUTER_S)) {
       // one (AS_NO_ROW, s_id) per selected S row
-      const bool emit = row_live && (mode == AS_JOIN_SEMI ? matched : !matched);
+      const bool emit = vi < P.n && (((matched >> lane) & 1u) != 0u) == (P.mode == AS_JOIN_SEMI);
       const uint32_t em = __ballot_sync(kFull, emit);
-      if (em) {
-        if (np + (uint32_t)__popc(em) > (uint32_t)kVStage) {
-          flush_stage(stage, np, P);
-          np = 0;
-        }
-        if (emit) {
-          const uint32_t pos = np + __popc(em & lanemask_lt());
-          stage.r[pos] = AS_NO_ROW;
-          stage.s[pos] = i;
-        }
-        np += (uint32_t)__popc(em);
-        __syncwarp();
-      }
+      unsigned long long base = 0;
+      if (lane == 0 && em) base = atomicAdd(P.count, (unsigned long long)__popc(em));
+      base = __shfl_sync(kFull, base, 0) + (unsigned long long)__popc(em & lanemask_lt());
+      if (emit && base < P.cap)
+        reinterpret_cast<uint64_t*>(P.pairs)[base] = pair_ids(AS_NO_ROW, vi, P.idR, P.idS, 0, 0);
     }
-  }
-  if (np) {
-    if (batch) flush_stage_join(stage, np, P, sj); else flush_stage(stage, np, P);
+    matched = 0;
+    grp += nwarps;
   }
 }
 

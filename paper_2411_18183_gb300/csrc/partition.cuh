@@ -192,85 +192,78 @@ struct PartProbeParams {
 };
 
 // S entries in partition order: each lane walks its entry's bucket sequence in
-// its partition's table; candidates (signature and length equal) are compared
-// byte for byte by the whole warp; verified pairs are staged per warp.
-__global__ void __launch_bounds__(kVThreads, 4) part_probe_kernel(PartProbeParams Q) {
-  __shared__ Stage stage_all[kVWarps];
+// its partition's table; candidates (signature and length equal) are queued and
+// verified as in verify_kernel.
+__global__ void __launch_bounds__(kVThreads, kVBlocks) part_probe_kernel(const __grid_constant__ PartProbeParams Q) {
+  __shared__ CandQueue queue_all[kVWarps];
   __shared__ uint4 emask[17];
   fill_emask(emask);
   __syncthreads();
   const VerifyParams& P = Q.V;
-  const int lane = threadIdx.x & 31;
-  Stage& stage = stage_all[threadIdx.x >> 5];
-  uint32_t np = 0;
+  const uint32_t lane = threadIdx.x & 31u;
+  CandQueue& W = queue_all[threadIdx.x >> 5];
+  uint32_t cnt = 0;
   const uint64_t ngroups = (Q.n + 31) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * kVWarps;
-  for (uint64_t grp = (uint64_t)blockIdx.x * kVWarps + (threadIdx.x >> 5); grp < ngroups; grp += nwarps) {
-    const uint64_t v = grp * 32 + (uint64_t)lane;
-    bool live = v < Q.n;
-    uint64_t sig = 0, start = 0, len = 0, b = 0, msk = 0, steps = 0;
-    uint32_t l32 = 0, srow = 0;
-    const Slot* tab = Q.slots;
-    if (live) {
-      const PartEntry e = Q.entS[v];
-      sig = e.sig;
-      l32 = (uint32_t)(e.key >> 32);
-      srow = (uint32_t)e.key;
-      start = __ldg(P.offS + srow);
-      len = __ldg(P.offS + srow + 1) - start;
-      const uint64_t h = sig_hash(sig, l32);
-      const uint32_t p = part_of(h, Q.pbits);
-      tab = Q.slots + Q.slot_off[p];
-      msk = Q.slot_off[p + 1] - Q.slot_off[p] - 1;
-      b = h & msk;
-    }
-    while (__any_sync(kFull, live)) {
-      bool cand = false;
-      uint32_t row = 0;
+  bool resume = false;
+  volatile uint64_t saved[3];
+  for (uint64_t grp = (uint64_t)blockIdx.x * kVWarps + (threadIdx.x >> 5); grp < ngroups;) {
+    {
+      const uint64_t v = grp * 32 + (uint64_t)lane;
+      bool live = v < Q.n;
+      uint64_t sig = 0, start = 0, b = 0, msk = 0, steps = 0;
+      uint32_t l32 = 0, srow = 0;
+      const Slot* tab = Q.slots;
       if (live) {
-        const ulonglong2 s = __ldg(reinterpret_cast<const ulonglong2*>(tab + b));
-        if (s.y == kEmpty) {
-          live = false;
-        } else {
-          if (s.x == sig && (uint32_t)(s.y >> 32) == l32) {
-            cand = true;
-            row = (uint32_t)s.y;
-          }
-          b = (b + 1) & msk;
-          if (++steps > msk) live = false;
-        }
+        const PartEntry e = Q.entS[v];
+        sig = e.sig;
+        l32 = (uint32_t)(e.key >> 32);
+        srow = (uint32_t)e.key;
+        start = __ldg(P.offS + srow);
+        const uint64_t h = sig_hash(sig, l32);
+        const uint32_t p = part_of(h, Q.pbits);
+        tab = Q.slots + Q.slot_off[p];
+        msk = Q.slot_off[p + 1] - Q.slot_off[p] - 1;
+        b = h & msk;
       }
-      uint32_t cm = __ballot_sync(kFull, cand);
-      while (cm) {
-        const int j = __ffs(cm) - 1;
-        cm &= cm - 1;
-        const uint32_t rj = __shfl_sync(kFull, row, j);
-        const uint32_t lj = __shfl_sync(kFull, l32, j);
-        const uint64_t stj = __shfl_sync(kFull, start, j);
-        const uint64_t rs = __ldg(P.offR + rj);
-        bool eq;
-        if (lj < kNarrowLen) {
-          eq = warp_equal(P.arenaR + rs, P.arenaS + stj, lj, emask);
-        } else {
-          const uint64_t ls = __shfl_sync(kFull, len, j);
-          eq = __ldg(P.offR + rj + 1) - rs == ls && warp_equal_wide(P.arenaR, rs, P.arenaS, stj, ls);
-        }
-        if (eq) {
-          const uint32_t sj = __shfl_sync(kFull, srow, j);
-          if (lane == 0) {
-            stage.r[np] = rj;
-            stage.s[np] = sj;
-          }
-          __syncwarp();
-          if (++np == (uint32_t)kVStage) {
-            flush_stage(stage, np, P);
-            np = 0;
+      if (resume) {
+        b = saved[0];
+        steps = saved[1];
+        live = saved[2] != 0u;
+      }
+      do {
+        bool cand = false;
+        uint32_t row = 0;
+        if (live) {
+          const ulonglong2 s = __ldg(reinterpret_cast<const ulonglong2*>(tab + b));
+          if (s.y == kEmpty) {
+            live = false;
+          } else {
+            if (s.x == sig && (uint32_t)(s.y >> 32) == l32) {
+              cand = true;
+              row = (uint32_t)s.y;
+            }
+            b = (b + 1) & msk;
+            if (++steps > msk) live = false;
           }
         }
+        queue_push(W.q, cnt, cand, start, srow, row, l32, 0u);
+        resume = __any_sync(kFull, live);
+      } while (resume && cnt <= kVQueue - kVDrain);
+      if (resume) {
+        saved[0] = b;
+        saved[1] = steps;
+        saved[2] = live ? 1u : 0u;
       }
     }
+    const bool flush = resume || grp + nwarps >= ngroups;
+    while (cnt >= kVDrain || (flush && cnt)) {
+      const uint32_t nc = cnt < kVDrain ? cnt : kVDrain;
+      cnt -= nc;
+      queue_verify<false, true>(W.q + cnt, W.ids, nc, P, emask);
+    }
+    if (!resume) grp += nwarps;
   }
-  if (np) flush_stage(stage, np, P);
 }
 
 }  // namespace algsig

@@ -1019,20 +1019,21 @@ static cudaError_t key_kernel_attrs() {
 }
 template <bool AT400, int NCOMP, int SHAPE, bool BATCH>
 static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
-                              const BatchJoin* J, int nj, int s_side, cudaStream_t s) {
+                              const BatchJoin* J, int nj, int s_side, uint64_t cap_len, cudaStream_t s) {
   constexpr LKShape k = kLKShapes[SHAPE];
   const uint64_t want = (n + 31) / 32;               // a group of 32 keys per block, until every SM has one
   const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
   sig_key_kernel<AT400, NCOMP, k.warps, k.depth, BATCH>
-      <<<blocks, 32 * k.warps, lk_smem_bytes(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side);
+      <<<blocks, 32 * k.warps, lk_smem_bytes(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len);
 }
 template <bool AT400, int NCOMP, bool BATCH>
 static void key_kernel_launch_shape(int shape, int sms, const uint8_t* arena, const uint64_t* off, uint64_t n,
-                                    uint64_t* out, const BatchJoin* J, int nj, int s_side, cudaStream_t s) {
+                                    uint64_t* out, const BatchJoin* J, int nj, int s_side, uint64_t cap_len,
+                                    cudaStream_t s) {
   switch (shape) {
-    case 1: key_kernel_launch<AT400, NCOMP, 1, BATCH>(sms, arena, off, n, out, J, nj, s_side, s); break;
-    case 2: key_kernel_launch<AT400, NCOMP, 2, BATCH>(sms, arena, off, n, out, J, nj, s_side, s); break;
-    default: key_kernel_launch<AT400, NCOMP, 0, BATCH>(sms, arena, off, n, out, J, nj, s_side, s); break;
+    case 1: key_kernel_launch<AT400, NCOMP, 1, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    case 2: key_kernel_launch<AT400, NCOMP, 2, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    default: key_kernel_launch<AT400, NCOMP, 0, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
   }
 }
 
@@ -1042,7 +1043,6 @@ struct DeviceState {
   int sms = 0;
   int verify_blocks_per_sm = 1;
   int prefix_blocks_per_sm = 1;
-  int capsig_blocks_per_sm = 1;
   int prefix_thread_blocks_per_sm = 1;
   bool tables_at400 = false;   // dynamic shared memory starts at shared address 0x400
   cudaStream_t side[kSideStreams] = {};   // side streams (SideStream), created with the state
@@ -1164,13 +1164,6 @@ static as_status ensure_device(DeviceState** out) {
                                                            kSmemPrefix)) != cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.prefix_blocks_per_sm < 1) d.prefix_blocks_per_sm = 1;
-    if ((e = cudaFuncSetAttribute(capsig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCapSig)) !=
-        cudaSuccess)
-      return cuda_fail(e, "kernel attribute");
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.capsig_blocks_per_sm, capsig_kernel, kCapThreads,
-                                                           kSmemCapSig)) != cudaSuccess)
-      return cuda_fail(e, "occupancy query");
-    if (d.capsig_blocks_per_sm < 1) d.capsig_blocks_per_sm = 1;
     if ((e = cudaFuncSetAttribute(prefix_thread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kSmemCapSig)) != cudaSuccess)
       return cuda_fail(e, "kernel attribute");
@@ -1223,7 +1216,7 @@ static bool table_geometry(uint64_t m, float lf, uint64_t* cap, uint32_t* log2ca
 }
 
 static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out, cudaStream_t s,
-                            int ncomp = 4, int shape = 0, int max_blocks = 0) {
+                            int ncomp = 4, int shape = 0, int max_blocks = 0, uint64_t cap_len = ~0ull) {
   DeviceState* d = nullptr;
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
@@ -1231,11 +1224,11 @@ static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t 
   if (max_blocks <= 0) max_blocks = d->sms;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
   if (ncomp == 2) {
-    if (d->tables_at400) key_kernel_launch_shape<true, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
-    else key_kernel_launch_shape<false, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    else key_kernel_launch_shape<false, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
   } else {
-    if (d->tables_at400) key_kernel_launch_shape<true, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
-    else key_kernel_launch_shape<false, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    else key_kernel_launch_shape<false, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
@@ -1248,8 +1241,8 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
                                   uint64_t* out, const BatchJoin* J, int nj, int s_side, int shape, cudaStream_t s) {
   if (n == 0) return AS_OK;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
-  if (d->tables_at400) key_kernel_launch_shape<true, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, s);
-  else key_kernel_launch_shape<false, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, s);
+  if (d->tables_at400) key_kernel_launch_shape<true, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
+  else key_kernel_launch_shape<false, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "batch signature kernel launch");
   return AS_OK;
@@ -1751,18 +1744,6 @@ size_t as_join_prefix_ws_bytes(uint64_t m, uint64_t n, float load_factor) {
   return (size_t)(round256(cap * 16) + round256(m * 8) + round256(n * 8) + 512);
 }
 
-// signatures of the first min(len, L) bytes of every key (one thread per key)
-static as_status launch_capped_sigs(DeviceState* d, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t L,
-                                    uint64_t* out, cudaStream_t s) {
-  if (n == 0) return AS_OK;
-  const uint64_t want = (n + kCapThreads - 1) / kCapThreads;
-  const uint64_t lim = (uint64_t)d->sms * (uint64_t)d->capsig_blocks_per_sm;
-  const unsigned blocks = (unsigned)(want < lim ? want : lim);
-  capsig_kernel<<<blocks, kCapThreads, kSmemCapSig, s>>>(arena, off, n, L, out);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? AS_OK : cuda_fail(e, "prefix signature launch");
-}
-
 as_status as_join_prefix(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_t* d_idR, uint64_t m,
                          const uint8_t* d_arenaS, const uint64_t* d_offS, const uint32_t* d_idS, uint64_t n,
                          uint64_t prefix_len, float load_factor, void* d_ws, size_t ws_bytes, uint32_t* d_pairs,
@@ -1799,14 +1780,14 @@ as_status as_join_prefix(const uint8_t* d_arenaR, const uint64_t* d_offR, const 
   if ((e = cudaMemsetAsync(slots, 0xFF, cap * 16, s)) != cudaSuccess) return cuda_fail(e, "table clear");
   if ((e = cudaMemsetAsync(flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
   if ((e = cudaMemsetAsync(cnt, 0, 8, s)) != cudaSuccess) return cuda_fail(e, "counter clear");
-  if ((st = launch_capped_sigs(d, d_arenaR, d_offR, m, prefix_len, sigR, s)) != AS_OK) return st;
+  if ((st = launch_sig(d_arenaR, d_offR, m, sigR, s, 4, 0, 0, prefix_len)) != AS_OK) return st;
   if (m > 0) {
     uint64_t blocks = (m + 255) / 256;
     const uint64_t lim = (uint64_t)d->sms * 16;
     if (blocks > lim) blocks = lim;
     build_kernel<<<(unsigned)blocks, 256, 0, s>>>(slots, cap - 1, sigR, d_offR, m, flags, nullptr, 0, prefix_len);
   }
-  if ((st = launch_capped_sigs(d, d_arenaS, d_offS, n, prefix_len, sigS, s)) != AS_OK) return st;
+  if ((st = launch_sig(d_arenaS, d_offS, n, sigS, s, 4, 0, 0, prefix_len)) != AS_OK) return st;
   if (n > 0) {
     as_table t;
     memset(&t, 0, sizeof(t));

@@ -255,7 +255,8 @@ __device__ __forceinline__ uint32_t lk_blocks(uintptr_t abs, uint64_t len) {
 // arbitrary), so that each group of 32 consecutive entries has keys of
 // nearly equal length.  rows: an empty stage, the first 8 rows of which hold
 // the bins' counts.
-__device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_t wn, uintptr_t arena) {
+__device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_t wn, uintptr_t arena,
+                                               uint64_t cap_len) {
   const uint32_t lane = threadIdx.x & 31u;
   if (wn <= 32) {                                    // one group: nothing to balance
     W.order[lane] = (uint8_t)lane;
@@ -277,7 +278,7 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
     bin[j] = 0;
     rank[j] = 0;
     if (i < wn) {
-      const uint64_t ks = W.woff[i], len = W.woff[i + 1] - ks;
+      const uint64_t ks = W.woff[i], len = min(W.woff[i + 1] - ks, cap_len);
       const uint32_t nb = lk_blocks(arena + ks, len);
       bin[j] = nb < 255u ? nb : 255u;
       rank[j] = atomicAdd(&count(bin[j]), 1u);
@@ -316,13 +317,13 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
 // group g of the window (wb: its first key) into the lanes; returns the
 // group's block count (its longest key's, at least 1)
 __device__ __forceinline__ uint32_t lk_load_group(LKKey& k, const LKWarp& W, uint64_t wb, uint32_t wn, uint32_t g,
-                                                  const uint8_t* arena) {
+                                                  const uint8_t* arena, uint64_t cap_len) {
   const uint32_t r = 32u * g + (threadIdx.x & 31u);
   k.valid = r < wn;
   k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.c1 = 0; k.te = 0;
   if (k.valid) {
     const uint32_t i = W.order[r];
-    const uint64_t ks = W.woff[i], len = W.woff[i + 1] - ks;
+    const uint64_t ks = W.woff[i], len = min(W.woff[i + 1] - ks, cap_len);
     const uintptr_t abs = reinterpret_cast<uintptr_t>(arena) + ks;
     k.kq = wb + i;
     // blocks start on a 32-byte boundary (a DRAM sector each), but at the arena's first chunk where
@@ -538,20 +539,21 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
 }
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
-// relation): equal counts below kLKSearchFrom keys, else equal shares of the
+// relation): equal counts below kLKSearchFrom keys (or if by_count: keys cut
+// to a length are about equally long), else equal shares of the
 // work, key bytes + kLKKeyCost per key (in a batch, over the joins' keys back
 // to back).  Whole warp.
 template <bool BATCH, int kWarps>
 __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, int nj, int s_side,
                                               const uint64_t* __restrict__ off, uint64_t n, uint64_t warp,
-                                              uint64_t nwarps, uint64_t* lo, uint64_t* hi) {
+                                              uint64_t nwarps, bool by_count, uint64_t* lo, uint64_t* hi) {
   if (n <= 32 * nwarps) {                            // at most one group per warp
     const uint64_t u = (warp % kWarps) * gridDim.x + warp / kWarps;   // neighbouring groups on different SMs
     *lo = 32 * u < n ? 32 * u : n;
     *hi = 32 * u + 32 < n ? 32 * u + 32 : n;
     return;
   }
-  if (n < kLKSearchFrom) {
+  if (by_count || n < kLKSearchFrom) {
     *lo = (uint64_t)((unsigned __int128)n * warp / nwarps);
     *hi = (uint64_t)((unsigned __int128)n * (warp + 1) / nwarps);
     return;
@@ -604,12 +606,14 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
 
 // The signatures of n keys: the rows of a relation (BATCH false), or the
 // virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
-// describe the joins, and sig_out is indexed by virtual row).
+// describe the joins, and sig_out is indexed by virtual row); of each key's
+// first cap_len bytes.
 template <bool AT400, int NCOMP, int kLKWarps, int kLKDepth, bool BATCH>
 __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t* __restrict__ arena,
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
-                                                                const BatchJoin* __restrict__ J, int nj, int s_side) {
+                                                                const BatchJoin* __restrict__ J, int nj, int s_side,
+                                                                uint64_t cap_len) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int kStages = kLKDepth / kLKStep;
   static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
@@ -624,11 +628,11 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
   const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
   uint64_t k_lo, k_hi;
-  lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
+  lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
   uint64_t bytes;                                   // the relation's (or batch side's) key bytes
   if constexpr (BATCH) bytes = s_side ? __ldg(&J[nj].vbs) : __ldg(&J[nj].vbr);
   else bytes = __ldg(off + n) - __ldg(off);
-  const uint32_t win = bytes >= kLKNarrowFrom * n ? kLKNarrowWin : kLKWin;
+  const uint32_t win = min(bytes / max(n, (uint64_t)1), cap_len) >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, win, &wa) : 0u;
   if (wn) lk_prefetch_window(W, off, wa, wa + wn);
@@ -661,9 +665,9 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       ng = (wn + 31) / 32;
       cp_async_wait_all();
       __syncwarp();
-      lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena));
+      lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena), cap_len);
     }
-    const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena);
+    const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena, cap_len);
     if (++g == ng) {                                  // the window's offsets are free: fetch the next ones
       __syncwarp();
       if (wb + wn < k_hi) {

@@ -33,10 +33,6 @@ __device__ uint16_t g_log[65536];
 __device__ uint16_t g_alog[65536];
 // constant-multiply tables of the tile combination (rounds.cuh), set up once per device
 __device__ uint16_t g_const[17 * 512];
-// image of the shared-memory reduction tables (gf16.cuh: 256 rows, each entry
-// replicated once per bank), set up once per device and copied by the blocks
-// that need the tables, so that no block computes them
-__device__ uint4 g_red_img[256 * 64 / 4];
 }  // namespace algsig
 
 #include "rounds.cuh"
@@ -1001,39 +997,39 @@ static as_status cuda_fail(cudaError_t e, const char* where) {
 }
 
 // The instantiations of the signature kernel: table addressing (AT400),
-// components, shape (warps per block, blocks in flight per key) and whether
-// it runs over the virtual rows of a batch (4 components only).
+// net, shape (warps per block, blocks in flight per key) and whether it runs
+// over the virtual rows of a batch (four components over GF(2^16) only).
 static_assert(kLKShapeCount == 3, "one case per shape below");
-template <bool AT400, int NCOMP, int SHAPE, bool BATCH>
+template <bool AT400, class Net, int SHAPE, bool BATCH>
 static cudaError_t key_kernel_attr() {
   constexpr LKShape k = kLKShapes[SHAPE];
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(sig_key_kernel<AT400, NCOMP, k.warps, k.depth, BATCH>),
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk_smem_bytes(k.warps, k.depth));
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk_smem_bytes<Net>(k.warps, k.depth));
 }
-template <bool AT400, int NCOMP, bool BATCH>
+template <bool AT400, class Net, bool BATCH>
 static cudaError_t key_kernel_attrs() {
-  cudaError_t e = key_kernel_attr<AT400, NCOMP, 0, BATCH>();
-  if (e == cudaSuccess) e = key_kernel_attr<AT400, NCOMP, 1, BATCH>();
-  if (e == cudaSuccess) e = key_kernel_attr<AT400, NCOMP, 2, BATCH>();
+  cudaError_t e = key_kernel_attr<AT400, Net, 0, BATCH>();
+  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 1, BATCH>();
+  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 2, BATCH>();
   return e;
 }
-template <bool AT400, int NCOMP, int SHAPE, bool BATCH>
+template <bool AT400, class Net, int SHAPE, bool BATCH>
 static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
                               const BatchJoin* J, int nj, int s_side, uint64_t cap_len, cudaStream_t s) {
   constexpr LKShape k = kLKShapes[SHAPE];
   const uint64_t want = (n + 31) / 32;               // a group of 32 keys per block, until every SM has one
   const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
-  sig_key_kernel<AT400, NCOMP, k.warps, k.depth, BATCH>
-      <<<blocks, 32 * k.warps, lk_smem_bytes(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len);
+  sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>
+      <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len);
 }
-template <bool AT400, int NCOMP, bool BATCH>
+template <bool AT400, class Net, bool BATCH>
 static void key_kernel_launch_shape(int shape, int sms, const uint8_t* arena, const uint64_t* off, uint64_t n,
                                     uint64_t* out, const BatchJoin* J, int nj, int s_side, uint64_t cap_len,
                                     cudaStream_t s) {
   switch (shape) {
-    case 1: key_kernel_launch<AT400, NCOMP, 1, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
-    case 2: key_kernel_launch<AT400, NCOMP, 2, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
-    default: key_kernel_launch<AT400, NCOMP, 0, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    case 1: key_kernel_launch<AT400, Net, 1, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    case 2: key_kernel_launch<AT400, Net, 2, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    default: key_kernel_launch<AT400, Net, 0, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
   }
 }
 
@@ -1109,17 +1105,27 @@ static as_status ensure_device(DeviceState** out) {
       }
       if ((e = cudaMemcpyToSymbol(g_inv, h_inv, sizeof(h_inv))) != cudaSuccess) return cuda_fail(e, "table setup");
     }
-    {  // the reduction tables' shared-memory image: row b, word l: T16[b] (l < 32), T24[b] (l >= 32)
-      static uint32_t h_red[kRedWords];
+    {  // the signature kernel's reduction tables (gf16.cuh, gf8.cuh), and GF(2^8)'s logarithms
+      uint2 h_red[256], h_red8[256];
       for (uint32_t b = 0; b < 256; b++) {
-        uint32_t t16 = b, t24 = b;
+        uint32_t t16 = b, t24 = b, r8 = b, r16 = b;
         for (int i = 0; i < 16; i++) t16 = gf_times_x(t16);
         for (int i = 0; i < 24; i++) t24 = gf_times_x(t24);
-        t16 ^= b << 16;
-        t24 ^= b << 24;
-        for (int l = 0; l < 64; l++) h_red[b * 64 + l] = l < 32 ? t16 : t24;
+        for (int i = 0; i < 8; i++) r8 = gf8_times_x(r8);
+        for (int i = 0; i < 16; i++) r16 = gf8_times_x(r16);
+        h_red[b] = make_uint2(t16 ^ (b << 16), t24 ^ (b << 24));
+        h_red8[b] = make_uint2(r8 ^ (b << 8), r16 ^ (b << 16));
       }
-      if ((e = cudaMemcpyToSymbol(g_red_img, h_red, sizeof(h_red))) != cudaSuccess) return cuda_fail(e, "table setup");
+      uint8_t h_log8[kLog8Bytes] = {};
+      uint32_t x = 1;
+      for (int i = 0; i < kOrder8; i++, x = gf8_times_x(x)) {
+        h_log8[x] = (uint8_t)i;
+        h_log8[256 + i] = h_log8[256 + kOrder8 + i] = (uint8_t)x;
+      }
+      if ((e = cudaMemcpyToSymbol(g_red16, h_red, sizeof(h_red))) != cudaSuccess ||
+          (e = cudaMemcpyToSymbol(g_red8, h_red8, sizeof(h_red8))) != cudaSuccess ||
+          (e = cudaMemcpyToSymbol(g_log8, h_log8, sizeof(h_log8))) != cudaSuccess)
+        return cuda_fail(e, "table setup");
     }
     // prefix-scan tables: x^(-8 k 2^s) at (k-1)*kPLevels+s
     static uint16_t h_pconst[kPConst * 512];
@@ -1136,12 +1142,14 @@ static as_status ensure_device(DeviceState** out) {
     if ((e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
       return cuda_fail(e, "device query");
     {
-      if ((e = key_kernel_attrs<true, 4, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, 4, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<true, 2, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, 2, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<true, 4, true>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, 4, true>()) != cudaSuccess)
+      if ((e = key_kernel_attrs<true, Net16<4>, false>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<4>, false>()) != cudaSuccess ||
+          (e = key_kernel_attrs<true, Net16<2>, false>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<2>, false>()) != cudaSuccess ||
+          (e = key_kernel_attrs<true, Net16<4>, true>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<4>, true>()) != cudaSuccess ||
+          (e = key_kernel_attr<true, Net8, 0, false>()) != cudaSuccess ||
+          (e = key_kernel_attr<false, Net8, 0, false>()) != cudaSuccess)
         return cuda_fail(e, "kernel attribute");
     }
     // where dynamic shared memory starts (the tables are its first bytes)
@@ -1171,9 +1179,6 @@ static as_status ensure_device(DeviceState** out) {
                                                            kCapThreads, kSmemCapSig)) != cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.prefix_thread_blocks_per_sm < 1) d.prefix_thread_blocks_per_sm = 1;
-    if ((e = cudaFuncSetAttribute(sig8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemSig8)) !=
-        cudaSuccess)
-      return cuda_fail(e, "kernel attribute");
     if ((e = cudaFuncSetAttribute(bl_hash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBHash)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
@@ -1224,11 +1229,11 @@ static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t 
   if (max_blocks <= 0) max_blocks = d->sms;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
   if (ncomp == 2) {
-    if (d->tables_at400) key_kernel_launch_shape<true, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
-    else key_kernel_launch_shape<false, 2, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, Net16<2>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    else key_kernel_launch_shape<false, Net16<2>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
   } else {
-    if (d->tables_at400) key_kernel_launch_shape<true, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
-    else key_kernel_launch_shape<false, 4, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    else key_kernel_launch_shape<false, Net16<4>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
@@ -1241,8 +1246,8 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
                                   uint64_t* out, const BatchJoin* J, int nj, int s_side, int shape, cudaStream_t s) {
   if (n == 0) return AS_OK;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
-  if (d->tables_at400) key_kernel_launch_shape<true, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
-  else key_kernel_launch_shape<false, 4, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
+  if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
+  else key_kernel_launch_shape<false, Net16<4>, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "batch signature kernel launch");
   return AS_OK;
@@ -1350,9 +1355,12 @@ as_status as_sig_compute_gf8(const uint8_t* d_arena, const uint64_t* d_off, uint
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
-  const uint64_t want = (n + kG8Threads - 1) / kG8Threads;
-  const unsigned blocks = (unsigned)(want < (uint64_t)d->sms * 8 ? want : (uint64_t)d->sms * 8);
-  sig8_kernel<<<blocks, kG8Threads, kSmemSig8, (cudaStream_t)stream>>>(d_arena, d_off, n, d_sig_out);
+  if (d->tables_at400)
+    key_kernel_launch<true, Net8, 0, false>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
+                                            (cudaStream_t)stream);
+  else
+    key_kernel_launch<false, Net8, 0, false>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
+                                             (cudaStream_t)stream);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "byte-symbol signature kernel launch");
   return AS_OK;

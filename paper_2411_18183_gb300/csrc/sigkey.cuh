@@ -70,6 +70,8 @@ namespace algsig {
 // image of the shared-memory constant-multiply tables (quotient.cuh): those of
 // the quotient form, then those of the remainder form; set up once per device
 __device__ uint4 g_inv[4 * kInvEntries / 16];
+// entries of the reduction tables (gf16.cuh): {T16[b], T24[b]}; set up once per device
+__device__ uint2 g_red16[256];
 
 // Kernel shapes: warps per block (one block per SM) and 32-byte blocks of each
 // key in flight (a multiple of 4, one step).  The batch autotuner picks one per
@@ -117,18 +119,16 @@ constexpr int kLKShort = 3;
 // upper halves beside the tables serve the first 8 / stages warps, the lines
 // after them two warps side by side.  Then the constant-multiply tables, the
 // byte masks and the warps' windows.
-constexpr size_t kSmemLKInv = 4 * kInvEntries;
 constexpr size_t kSmemLKMasks = 17 * 16;
 constexpr uint32_t kLKStageBytes = 32 * kLKPitch;     // from one stage of a warp to the next
 __host__ __device__ constexpr size_t lk_line_bytes(int warps, int depth) {
   const int stages = depth / kLKStep, beside = 8 / stages;
   return (size_t)256 * kLKPitch + (size_t)((warps > beside ? warps - beside : 0) + 1) / 2 * stages * kLKStageBytes;
 }
+template <class Net>
 __host__ __device__ constexpr size_t lk_smem_bytes(int warps, int depth) {
-  return lk_line_bytes(warps, depth) + kSmemLKInv + kSmemLKMasks + (size_t)warps * sizeof(LKWarp);
+  return lk_line_bytes(warps, depth) + Net::kTabBytes + kSmemLKMasks + (size_t)warps * sizeof(LKWarp);
 }
-static_assert(lk_smem_bytes(16, 8) <= 232448 && lk_smem_bytes(10, 12) <= 232448 && lk_smem_bytes(8, 16) <= 232448,
-              "the shapes' shared memory");
 // byte offset of a warp's first stage
 template <int kStages>
 __device__ __forceinline__ uint32_t lk_stage_base(uint32_t w) {
@@ -476,6 +476,26 @@ __device__ __forceinline__ void lk_short_blocks(uint32_t (&st)[kLKState], const 
   }
 }
 
+// What the kernel computes: signatures over GF(2^16) with two or four
+// components.  A net names its shared-memory tables and has the digit rings and
+// finish of the quotient form; kShort: groups of at most this many blocks take
+// the remainder form.
+template <int NCOMP>
+struct Net16 : QNet<NCOMP> {
+  static constexpr int kComponents = NCOMP;
+  static constexpr int kShort = kLKShort;
+  static constexpr size_t kTabBytes = 4 * kInvEntries;
+  __device__ __forceinline__ static const uint2* red_image() { return g_red16; }
+  __device__ __forceinline__ static const uint4* tab_image() { return g_inv; }
+  template <class Cursor>
+  __device__ __forceinline__ uint64_t finish(uint32_t a, const uint8_t* tab, const Cursor& rc) const {
+    return QNet<NCOMP>::finish(a, reinterpret_cast<const uint16_t*>(tab), rc);
+  }
+};
+static_assert(lk_smem_bytes<Net16<4>>(16, 8) <= 232448 && lk_smem_bytes<Net16<4>>(10, 12) <= 232448 &&
+                  lk_smem_bytes<Net16<4>>(8, 16) <= 232448,
+              "the shapes' shared memory");
+
 // The state after a group of longer keys, by division in quotient form
 // (quotient.cuh): the digit rings, in st.  A stage is refilled with the step
 // kStages further down once it is computed.  The loop is unrolled over three
@@ -608,7 +628,7 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
 // virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
 // describe the joins, and sig_out is indexed by virtual row); of each key's
 // first cap_len bytes.
-template <bool AT400, int NCOMP, int kLKWarps, int kLKDepth, bool BATCH>
+template <bool AT400, class Net, int kLKWarps, int kLKDepth, bool BATCH>
 __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t* __restrict__ arena,
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
@@ -618,9 +638,9 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   constexpr int kStages = kLKDepth / kLKStep;
   static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
   constexpr size_t kLines = lk_line_bytes(kLKWarps, kLKDepth);
-  uint16_t* inv = reinterpret_cast<uint16_t*>(smem + kLines);
-  uint4* mt = reinterpret_cast<uint4*>(smem + kLines + kSmemLKInv);
-  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kLines + kSmemLKInv + kSmemLKMasks);
+  uint8_t* tab = smem + kLines;
+  uint4* mt = reinterpret_cast<uint4*>(smem + kLines + Net::kTabBytes);
+  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kLines + Net::kTabBytes + kSmemLKMasks);
   const int wib = threadIdx.x >> 5;
   const uint32_t lane = threadIdx.x & 31u;
   LKWarp& W = warps[wib];
@@ -637,11 +657,16 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, win, &wa) : 0u;
   if (wn) lk_prefetch_window(W, off, wa, wa + wn);
   lk_fill_masks(mt);
-  for (int i = threadIdx.x; i < (int)(kSmemLKInv / 16); i += blockDim.x)
-    reinterpret_cast<uint4*>(inv)[i] = g_inv[i];
-  // the reduction tables: line b is 16 copies of T16[b], then 16 of T24[b]
-  for (int i = threadIdx.x; i < 256 * 8; i += blockDim.x)
-    *reinterpret_cast<uint4*>(smem + (i >> 3) * kLKPitch + (i & 7) * 16) = g_red_img[(i >> 3) * 16 + (i & 4) * 2 + (i & 3)];
+  for (int i = threadIdx.x; i < (int)(Net::kTabBytes / 16); i += blockDim.x)
+    reinterpret_cast<uint4*>(tab)[i] = Net::tab_image()[i];
+  // the reduction tables: line b is 16 copies of one entry of b, then 16 of the other
+  for (int i = threadIdx.x; i < 256 * 2; i += blockDim.x) {
+    const uint2 e = __ldg(Net::red_image() + (i >> 1));
+    const uint32_t v = i & 1 ? e.y : e.x;
+    uint4* line = reinterpret_cast<uint4*>(smem + (i >> 1) * kLKPitch + (i & 1) * 64);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) line[j] = make_uint4(v, v, v, v);
+  }
   __syncthreads();
   if (k_lo >= k_hi) return;
   const LKCursor<AT400> rc(smem);
@@ -689,24 +714,28 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     const uint32_t G = G2;
     k = k2;
     uint32_t st[kLKState];
-    if (G <= (uint32_t)kLKShort) {
-      cp_async_wait_but<0>();
-      __syncwarp();
-      lk_trim(k, row, 0, mt);
-      lk_short_blocks<NCOMP>(st, k, G, row);
-      __syncwarp();
-    } else {
-      lk_long_blocks<QNet<NCOMP>, kStages>(st, k, G, copy, base, row, mt);
+    bool brief = false;
+    if constexpr (Net::kShort > 0) {
+      brief = G <= (uint32_t)Net::kShort;
+      if (brief) {
+        cp_async_wait_but<0>();
+        __syncwarp();
+        lk_trim(k, row, 0, mt);
+        lk_short_blocks<Net::kComponents>(st, k, G, row);
+        __syncwarp();
+      }
     }
+    if (!brief) lk_long_blocks<Net, kStages>(st, k, G, copy, base, row, mt);
     // the next group's first steps are in flight while this one's signatures are finished
     G2 = next_group();
-    uint64_t sig;
-    if (G <= (uint32_t)kLKShort) {
-      sig = lk_finish<NCOMP>(st, k.a, inv + kInvEntries, rc);
-    } else {
-      QNet<NCOMP> net;
+    uint64_t sig = 0;
+    if constexpr (Net::kShort > 0) {
+      if (brief) sig = lk_finish<Net::kComponents>(st, k.a, reinterpret_cast<const uint16_t*>(tab) + kInvEntries, rc);
+    }
+    if (!brief) {
+      Net net;
       net.get(st);
-      sig = net.finish(k.a, inv, rc);
+      sig = net.finish(k.a, tab, rc);
     }
     if (k.valid) sig_out[k.kq] = sig;
   }

@@ -28,6 +28,7 @@ def test_step_edges(cuda, first, n):
     end = (int(off[-1]) + 15) // 16 * 16
     host = rng.integers(0, 256, max(16, end), dtype=np.uint8)
     want = oracle.sig_batch(host, off, nthreads=4)
+    want8 = oracle.sig8_batch(host, off, nthreads=4)
     for shift in (0, 16):                                  # the arena at an even and an odd 16-byte boundary
         buf = torch.empty(host.size + shift, dtype=torch.uint8, device="cuda")
         arena = buf[shift:]
@@ -37,6 +38,7 @@ def test_step_edges(cuda, first, n):
             for nc in (4, 2):
                 got = ag.sig_compute(R, n_components=nc, shape=shape).cpu().numpy().view(np.uint64)
                 assert np.array_equal(got, want & np.uint64(oracle.component_mask(nc))), (shift, shape, nc)
+        assert np.array_equal(ag.sig_compute_gf8(R).cpu().numpy().view(np.uint64), want8), shift
 
 
 @pytest.mark.parametrize("lo,hi", [(1, 3000), (200, 280), (0, 12)])

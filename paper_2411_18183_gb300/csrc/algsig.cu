@@ -1148,6 +1148,16 @@ static as_status ensure_device(DeviceState** out) {
           (e = key_kernel_attrs<false, Net16<2>, false>()) != cudaSuccess ||
           (e = key_kernel_attrs<true, Net16<4>, true>()) != cudaSuccess ||
           (e = key_kernel_attrs<false, Net16<4>, true>()) != cudaSuccess ||
+          (e = cudaFuncSetAttribute(
+               reinterpret_cast<const void*>(
+                   sig_key_kernel<true, Net16<4>, kLKShapes[0].warps, kLKShapes[0].depth, false, true>),
+               cudaFuncAttributeMaxDynamicSharedMemorySize,
+               (int)lk_smem_bytes<Net16<4>>(kLKShapes[0].warps, kLKShapes[0].depth))) != cudaSuccess ||
+          (e = cudaFuncSetAttribute(
+               reinterpret_cast<const void*>(
+                   sig_key_kernel<false, Net16<4>, kLKShapes[0].warps, kLKShapes[0].depth, false, true>),
+               cudaFuncAttributeMaxDynamicSharedMemorySize,
+               (int)lk_smem_bytes<Net16<4>>(kLKShapes[0].warps, kLKShapes[0].depth))) != cudaSuccess ||
           (e = key_kernel_attr<true, Net8, 0, false>()) != cudaSuccess ||
           (e = key_kernel_attr<false, Net8, 0, false>()) != cudaSuccess)
         return cuda_fail(e, "kernel attribute");
@@ -1408,6 +1418,24 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
+  // the blocks' own signatures and their sums along each key, or one key per thread or warp (by_items: the
+  // kernels of the one that is not wanted return at once)
+  constexpr LKShape k = kLKShapes[0];
+  LKItems it;
+  it.first = d_pref_off;
+  it.keys = n;
+  it.block = block_bytes;
+  if (d->tables_at400)
+    sig_key_kernel<true, Net16<4>, k.warps, k.depth, false, true>
+        <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
+            d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
+  else
+    sig_key_kernel<false, Net16<4>, k.warps, k.depth, false, true>
+        <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
+            d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
+  const uint64_t scan_want = (n + kPThreads - 1) / kPThreads, scan_lim = (uint64_t)d->sms * 8;
+  prefix_scan_kernel<<<(unsigned)(scan_want < scan_lim ? scan_want : scan_lim), kPThreads, 0, (cudaStream_t)stream>>>(
+      d_off, n, block_bytes, d_pref_off, d_out);
   if (block_bytes >= 32) {
     // entries at most every other chunk: one thread per key, the suffix snapshots of prefix_thread_kernel
     const uint64_t want = (n + kCapThreads - 1) / kCapThreads;

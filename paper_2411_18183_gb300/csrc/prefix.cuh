@@ -98,16 +98,27 @@ __global__ void __launch_bounds__(kPThreads) prefix_count_kernel(const uint64_t*
   if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
 }
 
-// pass 2 (one block): exclusive scan of the block totals in place; pref_off[n] = the total
+// pass 2 (one block): exclusive scan of the block totals in place, eight per
+// thread and round; pref_off[n] = the total
 __global__ void __launch_bounds__(kPThreads) prefix_total_kernel(uint64_t* __restrict__ block_sums, uint64_t nblocks,
                                                                  uint64_t* __restrict__ pref_off, uint64_t n) {
+  constexpr int kPer = 8;
   uint64_t carry = 0;
-  for (uint64_t b0 = 0; b0 < nblocks; b0 += kPThreads) {
-    const uint64_t b = b0 + threadIdx.x;
-    const uint64_t v = b < nblocks ? block_sums[b] : 0;
+  for (uint64_t b0 = 0; b0 < nblocks; b0 += kPer * kPThreads) {
+    const uint64_t b = b0 + (uint64_t)threadIdx.x * kPer;
+    uint64_t v[kPer], s = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+      v[j] = b + j < nblocks ? block_sums[b + j] : 0;
+      s += v[j];
+    }
     uint64_t total;
-    const uint64_t ex = block_exclusive_scan(v, &total);
-    if (b < nblocks) block_sums[b] = carry + ex;
+    uint64_t run = carry + block_exclusive_scan(s, &total);
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+      if (b + j < nblocks) block_sums[b + j] = run;
+      run += v[j];
+    }
     carry += total;
   }
   if (threadIdx.x == 0) pref_off[n] = carry;
@@ -245,6 +256,7 @@ __global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __rest
                                                            uint32_t block_bytes,
                                                            const uint64_t* __restrict__ pref_off,
                                                            uint64_t* __restrict__ out) {
+  if (by_items(off, n, block_bytes)) return;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
@@ -324,6 +336,7 @@ __global__ void __launch_bounds__(kCapThreads) prefix_thread_kernel(const uint8_
                                                                     uint32_t block_bytes,
                                                                     const uint64_t* __restrict__ pref_off,
                                                                     uint64_t* __restrict__ out) {
+  if (by_items(off, n, block_bytes)) return;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
@@ -377,6 +390,68 @@ __global__ void __launch_bounds__(kCapThreads) prefix_thread_kernel(const uint8_
                                    (uint32_t)(v >> 48), e1);
     }
     o[nb - 1] = S;
+  }
+}
+
+// The cumulative signatures from those of the keys' blocks (the signature
+// kernel over items): C_j = sum_{i <= j} x^(k i B / 2) sig(block i), in place,
+// one thread per key; a key of more than 32 blocks is scanned by the warp.  The
+// factors go through the log / antilog tables.
+__global__ void __launch_bounds__(kPThreads) prefix_scan_kernel(const uint64_t* __restrict__ off, uint64_t n,
+                                                                uint32_t block_bytes,
+                                                                const uint64_t* __restrict__ pref_off,
+                                                                uint64_t* __restrict__ out) {
+  if (!by_items(off, n, block_bytes)) return;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t eb = (block_bytes / 2u) % kOrder;     // exponent from one block to the next
+  auto moved = [](uint64_t v, uint32_t e) {
+    return shift_chunk_value((uint32_t)v & 0xFFFFu, (uint32_t)(v >> 16) & 0xFFFFu, (uint32_t)(v >> 32) & 0xFFFFu,
+                             (uint32_t)(v >> 48), e);
+  };
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {   // warp-uniform
+    const uint64_t i = i0 + lane;
+    uint64_t p0 = 0, c = 0;
+    if (i < n) {
+      p0 = pref_off[i];
+      c = pref_off[i + 1] - p0;
+    }
+    if (c > 1 && c <= 32) {
+      uint64_t acc = out[p0];
+      uint32_t e = 0;
+      for (uint32_t j = 1; j < (uint32_t)c; j += 4) {      // four blocks' lookups at a time
+        uint64_t v[4];
+#pragma unroll
+        for (uint32_t t = 0; t < 4; ++t) {
+          v[t] = j + t < (uint32_t)c ? out[p0 + j + t] : 0ull;
+          e += eb;
+          if (e >= kOrder) e -= kOrder;
+          v[t] = moved(v[t], e);
+        }
+#pragma unroll
+        for (uint32_t t = 0; t < 4; ++t) {
+          acc ^= v[t];
+          if (j + t < (uint32_t)c) out[p0 + j + t] = acc;
+        }
+      }
+    }
+    for (uint32_t m = __ballot_sync(0xFFFFFFFFu, c > 32); m; m &= m - 1u) {
+      const int l = __ffs((int)m) - 1;
+      const uint64_t pl = __shfl_sync(0xFFFFFFFFu, p0, l), cl = __shfl_sync(0xFFFFFFFFu, c, l);
+      uint64_t carry = 0;
+      for (uint64_t b = 0; b < cl; b += 32) {
+        const uint64_t j = b + lane;
+        uint64_t v = j < cl ? moved(out[pl + j], (uint32_t)(j % kOrder * eb % kOrder)) : 0ull;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint64_t t = __shfl_up_sync(0xFFFFFFFFu, v, d);
+          if (lane >= (uint32_t)d) v ^= t;
+        }
+        v ^= carry;
+        if (j < cl) out[pl + j] = v;
+        carry = __shfl_sync(0xFFFFFFFFu, v, 31);
+      }
+    }
   }
 }
 

@@ -624,16 +624,98 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
   }
 }
 
+// Keys cut into pieces: key i's pieces of `block` bytes (the last one shorter;
+// one for an empty key) are items first[i] .. first[i + 1), first[keys] of them
+// in all, and the kernel signs items instead of keys.  Consecutive items are
+// consecutive bytes, so that an item ends where the next one starts.
+struct LKItems {
+  const uint64_t* first = nullptr;
+  uint64_t keys = 0;
+  uint32_t block = 0;
+};
+
+// Whether a relation's cumulative signatures are computed by items (or by the
+// kernels of prefix.cuh, one key per thread or warp): a question of the mean key
+// length, which only the device knows, so both kernels are launched and one
+// returns at once.  An item costs the finish of a signature whatever its length,
+// a thread of its own follows a key at 90 instructions per 16 bytes and with
+// 16-byte loads.  us, items against the others, 500k keys of 200-2000 bytes (2M
+// of 32-128): blocks of 16 2043 / 1410 (735 / 1602), 32 1173 / 1295 (430 / 318),
+// 64 724 / 956 (271 / 249), 256 299 / 669 (222 / 192), 4096 206 / 489.
+__device__ __forceinline__ bool by_items(const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
+  const uint64_t bytes = __ldg(off + n) - __ldg(off);
+  return block < 32u ? bytes < 192u * n : bytes >= (block < 64u ? 256u : 128u) * n;
+}
+
+// the starts of items [wb, wb + wn) and the end of the last one into the
+// window; kb: a key at or before the one that holds item wb, moved on to the key
+// that holds the last item; guess: keys to look at first, set to the keys the
+// window took (whole warp).  The keys' first items and starts are copied into
+// the empty stage at rows, up to 128 keys at a time (with 32 keys per wait and
+// no copy the call took as long).
+__device__ __forceinline__ void lk_item_window(LKWarp& W, uint8_t* rows, const uint64_t* __restrict__ off,
+                                               const LKItems& it, uint64_t wb, uint32_t wn, uint64_t& kb,
+                                               uint32_t& guess) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t we = wb + wn, k0 = kb;
+  // key x of the batch: its first item and its start, in row x / 8
+  auto pair = [&](uint32_t x) { return reinterpret_cast<uint64_t*>(rows + (x >> 3) * kLKPitch) + 2 * (x & 7u); };
+  for (uint64_t kk = kb;;) {
+    const uint32_t want = guess < 16u ? 16u : (guess > 128u ? 128u : guess);
+    const uint32_t nk = it.keys - kk < want ? (uint32_t)(it.keys - kk) : want;
+    for (uint32_t x = lane; x <= nk; x += 32) {
+      cp_async8(pair(x), it.first + kk + x);
+      cp_async8(pair(x) + 1, off + kk + x);
+    }
+    cp_async_commit();
+    cp_async_wait_all();
+    __syncwarp();
+    bool done = false;
+    for (uint32_t x0 = 0; x0 < nk && !done; x0 += 32) {
+      const uint32_t x = x0 + lane;
+      const bool have = x < nk;
+      const uint64_t p0 = have ? pair(x)[0] : ~0ull, s = have ? pair(x)[1] : 0;
+      const uint64_t p1 = have ? pair(x + 1)[0] : ~0ull;
+      // the key's items in the window: [a, a + c)
+      const uint64_t a = p0 > wb ? p0 : wb, z = p1 < we ? p1 : we;
+      const uint32_t c = have && a < z ? (uint32_t)(z - a) : 0u;
+      const bool many = c > 16u;
+      for (uint32_t j = 0; __any_sync(kFull, !many && j < c); ++j)
+        if (!many && j < c) W.woff[a - wb + j] = s + (a - p0 + j) * it.block;
+      for (uint32_t m = __ballot_sync(kFull, many); m; m &= m - 1u) {
+        const int l = __ffs((int)m) - 1;
+        const uint32_t cl = __shfl_sync(kFull, c, l);
+        const uint64_t al = __shfl_sync(kFull, a, l), pl = __shfl_sync(kFull, p0, l), sl = __shfl_sync(kFull, s, l);
+        for (uint32_t j = lane; j < cl; j += 32) W.woff[al - wb + j] = sl + (al - pl + j) * it.block;
+      }
+      const bool last = c > 0u && z == we;             // one key at most
+      if (last) W.woff[wn] = min(s + (we - p0) * it.block, pair(x + 1)[1]);
+      const uint32_t lm = __ballot_sync(kFull, last);
+      if (lm) {
+        kb = kk + x0 + (uint64_t)(__ffs((int)lm) - 1);
+        done = true;
+      }
+    }
+    __syncwarp();
+    kk += nk;
+    if (done || kk >= it.keys) break;                  // (some key holds item we - 1)
+  }
+  guess = kb - k0 < 128u ? (uint32_t)(kb - k0) + 2u : 128u;
+}
+
 // The signatures of n keys: the rows of a relation (BATCH false), or the
 // virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
 // describe the joins, and sig_out is indexed by virtual row); of each key's
-// first cap_len bytes.
-template <bool AT400, class Net, int kLKWarps, int kLKDepth, bool BATCH>
+// first cap_len bytes.  ITEMS: of the n keys' items.
+template <bool AT400, class Net, int kLKWarps, int kLKDepth, bool BATCH, bool ITEMS = false>
 __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t* __restrict__ arena,
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
                                                                 const BatchJoin* __restrict__ J, int nj, int s_side,
-                                                                uint64_t cap_len) {
+                                                                uint64_t cap_len, const LKItems items = LKItems()) {
+  if constexpr (ITEMS) {
+    if (!by_items(off, n, items.block)) return;
+  }
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int kStages = kLKDepth / kLKStep;
   static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
@@ -647,15 +729,22 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   // the warp's keys and its first window's offsets first, so that their loads overlap the tables' copy
   const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
   const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
-  uint64_t k_lo, k_hi;
-  lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
-  uint64_t bytes;                                   // the relation's (or batch side's) key bytes
-  if constexpr (BATCH) bytes = s_side ? __ldg(&J[nj].vbs) : __ldg(&J[nj].vbr);
-  else bytes = __ldg(off + n) - __ldg(off);
-  const uint32_t win = min(bytes / max(n, (uint64_t)1), cap_len) >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
+  uint64_t k_lo, k_hi, kb = 0;                      // kb (items): the key of the window's first item
+  uint32_t win;
+  if constexpr (ITEMS) {
+    lk_warp_range<false, kLKWarps>(J, nj, s_side, off, __ldg(items.first + n), warp, nwarps, true, &k_lo, &k_hi);
+    win = items.block >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
+    if (k_lo < k_hi) kb = warp_lower_bound(items.first, n, k_lo + 1) - 1;
+  } else {
+    lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
+    uint64_t bytes;                                 // the relation's (or batch side's) key bytes
+    if constexpr (BATCH) bytes = s_side ? __ldg(&J[nj].vbs) : __ldg(&J[nj].vbr);
+    else bytes = __ldg(off + n) - __ldg(off);
+    win = min(bytes / max(n, (uint64_t)1), cap_len) >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
+  }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, win, &wa) : 0u;
-  if (wn) lk_prefetch_window(W, off, wa, wa + wn);
+  if (wn && !ITEMS) lk_prefetch_window(W, off, wa, wa + wn);
   lk_fill_masks(mt);
   for (int i = threadIdx.x; i < (int)(Net::kTabBytes / 16); i += blockDim.x)
     reinterpret_cast<uint4*>(tab)[i] = Net::tab_image()[i];
@@ -674,7 +763,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   uint8_t* stages = smem + lk_stage_base<kStages>((uint32_t)wib);
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(stages);
   const uint32_t row = base + lane * kLKPitch + ((lane & 7u) << 4);
-  uint32_t g = 0, ng = 0;
+  uint32_t g = 0, ng = 0, guess = 64;
   LKKey k, k2;
   LKCopy copy;
   // The warp's next group into k2, its first steps requested; returns its block count, 0 when there is
@@ -690,12 +779,13 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       ng = (wn + 31) / 32;
       cp_async_wait_all();
       __syncwarp();
+      if constexpr (ITEMS) lk_item_window(W, stages, off, items, wb, wn, kb, guess);
       lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena), cap_len);
     }
     const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena, cap_len);
     if (++g == ng) {                                  // the window's offsets are free: fetch the next ones
       __syncwarp();
-      if (wb + wn < k_hi) {
+      if (!ITEMS && wb + wn < k_hi) {
         uint64_t na;
         const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, win, &na);
         lk_prefetch_window(W, off, na, na + nn);

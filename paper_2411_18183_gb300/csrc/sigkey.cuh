@@ -82,8 +82,8 @@ struct LKShape {
 constexpr LKShape kLKShapes[] = {{16, 8}, {10, 12}, {8, 16}};
 constexpr int kLKShapeCount = sizeof(kLKShapes) / sizeof(kLKShapes[0]);
 constexpr int kLKWin = 256;                           // most keys of a sorting window
-// Keys of at least kLKNarrowFrom bytes on average are sorted in windows of
-// kLKNarrowWin: neighbouring keys share a 128-byte line of DRAM, and with the
+// A window whose keys have kLKNarrowFrom bytes or more on average is cut to
+// kLKNarrowWin keys: neighbouring keys share a 128-byte line of DRAM, and with the
 // larger window the line is often gone from L2 when the second key is read
 // (2M keys of 256-1024 bytes: 1.47 GB read for 1.28 GB of keys, 283 against
 // 271 us); for keys of 32-128 bytes the sort's share counts (197 against 205 us).
@@ -93,12 +93,13 @@ constexpr uint64_t kLKNarrowFrom = 256;
 // search in the offsets); smaller ones by key count, which saves the search's
 // dependent loads where they would be a large share of the kernel's time
 constexpr uint64_t kLKSearchFrom = 1ull << 19;
-// A key's work in key-byte equivalents is its length + kLKKeyCost (the window
-// sort, masks and finishing): fitted to the kernel's rates on keys of 32-128
-// and 2048-8192 bytes, it gives the rate on 256-1024 bytes within 1 %.  The
-// warps' shares are cut on it, so that a relation (or batch) that mixes short
-// and long keys leaves no warp with far more keys than the others.
-constexpr uint64_t kLKKeyCost = 140;
+// A key's work in key-byte equivalents is its length + kLKKeyCost: short keys
+// cost their arithmetic (80 bytes as much as 240 of long ones), long ones their
+// bytes.  The warps' shares are cut on it, so that a relation (or batch) that
+// mixes short and long keys leaves no warp with far more work than the others
+// (a batch of joins of 32-128, 256-1024 and 2048-8192 bytes: 1.51, 1.45, 1.39,
+// 1.38 and 1.37 ms with 140, 170, 200, 240 and 300).
+constexpr uint64_t kLKKeyCost = 256;
 
 struct LKWarp {
   uint64_t woff[kLKWin + 2];       // offsets of the window's keys (woff[i] = off[wb + i]), i <= wn
@@ -537,13 +538,13 @@ __device__ __forceinline__ void lk_long_blocks(uint32_t (&st)[kLKState], const L
   net.put(st);
 }
 
-// The window of at most win keys starting at key wb (keys below k_hi): returns its key
+// The window of keys starting at key wb (keys below k_hi): returns its key
 // count and sets *wa to its first row in the relation.  In a batch the keys are
 // virtual rows (the joins' row ranges back to back) and a window ends with its
 // join's rows, so that its keys are consecutive rows of the relation.
 template <bool BATCH>
 __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, int nj, int s_side, uint64_t wb,
-                                              uint64_t k_hi, uint32_t win, uint64_t* wa) {
+                                              uint64_t k_hi, uint64_t* wa) {
   uint64_t lim = k_hi;
   *wa = wb;
   if constexpr (BATCH) {
@@ -555,7 +556,7 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
     if (v0 + (e - b) < lim) lim = v0 + (e - b);
   }
   const uint64_t left = lim - wb;
-  return left < win ? (uint32_t)left : win;
+  return left < (uint64_t)kLKWin ? (uint32_t)left : (uint32_t)kLKWin;
 }
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
@@ -730,20 +731,14 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
   const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
   uint64_t k_lo, k_hi, kb = 0;                      // kb (items): the key of the window's first item
-  uint32_t win;
   if constexpr (ITEMS) {
     lk_warp_range<false, kLKWarps>(J, nj, s_side, off, __ldg(items.first + n), warp, nwarps, true, &k_lo, &k_hi);
-    win = items.block >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
     if (k_lo < k_hi) kb = warp_lower_bound(items.first, n, k_lo + 1) - 1;
   } else {
     lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
-    uint64_t bytes;                                 // the relation's (or batch side's) key bytes
-    if constexpr (BATCH) bytes = s_side ? __ldg(&J[nj].vbs) : __ldg(&J[nj].vbr);
-    else bytes = __ldg(off + n) - __ldg(off);
-    win = min(bytes / max(n, (uint64_t)1), cap_len) >= kLKNarrowFrom ? kLKNarrowWin : kLKWin;
   }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
-  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, win, &wa) : 0u;
+  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, &wa) : 0u;
   if (wn && !ITEMS) lk_prefetch_window(W, off, wa, wa + wn);
   lk_fill_masks(mt);
   for (int i = threadIdx.x; i < (int)(Net::kTabBytes / 16); i += blockDim.x)
@@ -773,13 +768,17 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       if (ng) {
         wb += wn;
         if (wb >= k_hi) return 0u;
-        wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, win, &wa);
+        wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, &wa);
       }
       g = 0;
       ng = (wn + 31) / 32;
       cp_async_wait_all();
       __syncwarp();
       if constexpr (ITEMS) lk_item_window(W, stages, off, items, wb, wn, kb, guess);
+      if (wn == (uint32_t)kLKWin && min((W.woff[wn] - W.woff[0]) / kLKWin, cap_len) >= kLKNarrowFrom) {
+        wn = kLKNarrowWin;
+        ng = kLKNarrowWin / 32;
+      }
       lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena), cap_len);
     }
     const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena, cap_len);
@@ -787,7 +786,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       __syncwarp();
       if (!ITEMS && wb + wn < k_hi) {
         uint64_t na;
-        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, win, &na);
+        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, &na);
         lk_prefetch_window(W, off, na, na + nn);
       }
     }

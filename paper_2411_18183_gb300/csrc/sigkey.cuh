@@ -538,13 +538,13 @@ __device__ __forceinline__ void lk_long_blocks(uint32_t (&st)[kLKState], const L
   net.put(st);
 }
 
-// The window of keys starting at key wb (keys below k_hi): returns its key
+// The window of at most `most` keys starting at key wb (keys below k_hi): returns its key
 // count and sets *wa to its first row in the relation.  In a batch the keys are
 // virtual rows (the joins' row ranges back to back) and a window ends with its
 // join's rows, so that its keys are consecutive rows of the relation.
 template <bool BATCH>
 __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, int nj, int s_side, uint64_t wb,
-                                              uint64_t k_hi, uint64_t* wa) {
+                                              uint64_t k_hi, uint32_t most, uint64_t* wa) {
   uint64_t lim = k_hi;
   *wa = wb;
   if constexpr (BATCH) {
@@ -556,7 +556,7 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
     if (v0 + (e - b) < lim) lim = v0 + (e - b);
   }
   const uint64_t left = lim - wb;
-  return left < (uint64_t)kLKWin ? (uint32_t)left : (uint32_t)kLKWin;
+  return left < (uint64_t)most ? (uint32_t)left : most;
 }
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
@@ -731,14 +731,16 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
   const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
   uint64_t k_lo, k_hi, kb = 0;                      // kb (items): the key of the window's first item
+  uint32_t most = kLKWin;
   if constexpr (ITEMS) {
+    if (items.block >= kLKNarrowFrom) most = kLKNarrowWin;
     lk_warp_range<false, kLKWarps>(J, nj, s_side, off, __ldg(items.first + n), warp, nwarps, true, &k_lo, &k_hi);
     if (k_lo < k_hi) kb = warp_lower_bound(items.first, n, k_lo + 1) - 1;
   } else {
     lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
   }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
-  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, &wa) : 0u;
+  uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, most, &wa) : 0u;
   if (wn && !ITEMS) lk_prefetch_window(W, off, wa, wa + wn);
   lk_fill_masks(mt);
   for (int i = threadIdx.x; i < (int)(Net::kTabBytes / 16); i += blockDim.x)
@@ -768,14 +770,14 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       if (ng) {
         wb += wn;
         if (wb >= k_hi) return 0u;
-        wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, &wa);
+        wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, most, &wa);
       }
       g = 0;
       ng = (wn + 31) / 32;
       cp_async_wait_all();
       __syncwarp();
       if constexpr (ITEMS) lk_item_window(W, stages, off, items, wb, wn, kb, guess);
-      if (wn == (uint32_t)kLKWin && min((W.woff[wn] - W.woff[0]) / kLKWin, cap_len) >= kLKNarrowFrom) {
+      if (!ITEMS && wn == (uint32_t)kLKWin && min((W.woff[wn] - W.woff[0]) / kLKWin, cap_len) >= kLKNarrowFrom) {
         wn = kLKNarrowWin;
         ng = kLKNarrowWin / 32;
       }
@@ -786,7 +788,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
       __syncwarp();
       if (!ITEMS && wb + wn < k_hi) {
         uint64_t na;
-        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, &na);
+        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, most, &na);
         lk_prefetch_window(W, off, na, na + nn);
       }
     }

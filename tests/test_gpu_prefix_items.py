@@ -35,3 +35,26 @@ def test_blocks_sum_up(cuda, name, block):
     for i, k in enumerate(keys):
         if len(k) <= 3000 or i == 1:
             assert out[pref[i]:pref[i + 1]].tolist() == oracle.sig_prefixes(k, block), (i, len(k))
+
+
+@pytest.mark.parametrize("block", [256, 512, 1024])
+def test_many_windows_per_warp(cuda, block):
+    """More than a million blocks, so that every warp walks several windows, most of which end inside
+    a key: each key's last entry is the signature of the whole key."""
+    ag = cuda
+    rng = np.random.default_rng(block)
+    lens = rng.integers(block, 5 * block, 420_000).astype(np.uint64)
+    off = np.zeros(lens.size + 1, np.uint64)
+    off[1:] = np.cumsum(lens)
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(block)
+    arena = torch.empty((int(off[-1]) + 15) // 16 * 16 + 16, dtype=torch.uint8, device="cuda").random_(0, 256, generator=gen)
+    D = ag.DeviceRelation(arena, torch.as_tensor(off.view(np.int64)).cuda())
+    pref, out = ag.sig_prefixes(D, block)
+    assert torch.equal(out[pref[1:] - 1], ag.sig_compute(D))
+    some = rng.integers(0, lens.size, 40)
+    pref, host = pref.cpu().numpy(), out.cpu().numpy().view(np.uint64)
+    for i in some:
+        key = arena[int(off[i]):int(off[i + 1])].cpu().numpy().tobytes()
+        assert host[pref[i]:pref[i + 1]].tolist() == oracle.sig_prefixes(key, block), i

@@ -44,7 +44,7 @@
  * Streams: every call is asynchronous on the given stream (a cudaStream_t
  * passed as void*, NULL = legacy default stream) unless it is given a host
  * pointer to return a count, in which case it synchronises that stream.
- * as_join, as_join_batch_run and as_baseline_join run
+ * as_join_batch_run and as_baseline_join run
  * S's signatures (or hashes) on a side stream of the library (four per
  * device, created with the tables) forked from the given stream and joined
  * back into it before the probe, so that they overlap R's signatures and the
@@ -327,8 +327,8 @@ size_t as_join_ws_bytes(uint64_t m, uint64_t n, float load_factor);
  * signatures of R, build, probe with S (signatures, verification, compaction).
  * Arguments as for as_join_build and as_join_probe; d_ws must hold
  * as_join_ws_bytes(m, load_factor) bytes.  d_count may be NULL (the counter
- * then lives in the workspace).  S's signatures run on a side stream, beside
- * R's signatures and the build where those leave SMs idle.
+ * then lives in the workspace).  R's and S's signatures are one launch, in which
+ * the two share the SMs where both relations are small.
  */
 as_status as_join(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_t* d_idR, uint64_t m,
                   const uint8_t* d_arenaS, const uint64_t* d_offS, const uint32_t* d_idS, uint64_t n,

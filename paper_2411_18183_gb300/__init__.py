@@ -347,7 +347,7 @@ def join(R: DeviceRelation, S: DeviceRelation, load_factor: float = 0.5, cap_pai
     dev = R.arena.device
     ws = alloc_ws(join_ws_bytes(R.n, S.n, load_factor), dev)
     cap = cap_pairs if cap_pairs is not None else max(1024, S.n)
-    count = torch.zeros(1, dtype=torch.int64, device=dev)
+    count = torch.empty(1, dtype=torch.int64, device=dev)      # the call clears it
     while True:
         pairs = torch.empty(2 * max(cap, 1), dtype=torch.int32, device=dev)
         st, cnt = join_into(R, S, ws, pairs, count, load_factor, sync=True, stream=stream, allow_capacity=True)
@@ -380,7 +380,7 @@ def join_prefix(R: DeviceRelation, S: DeviceRelation, prefix_len: int, load_fact
     dev = R.arena.device
     ws = alloc_ws(join_prefix_ws_bytes(R.n, S.n, load_factor), dev)
     cap = cap_pairs if cap_pairs is not None else max(1024, S.n)
-    count = torch.zeros(1, dtype=torch.int64, device=dev)
+    count = torch.empty(1, dtype=torch.int64, device=dev)      # the call clears it
     while True:
         pairs = torch.empty(2 * max(cap, 1), dtype=torch.int32, device=dev)
         st, cnt = join_prefix_into(R, S, prefix_len, ws, pairs, count, load_factor, sync=True, stream=stream,
@@ -417,7 +417,7 @@ def join_partitioned(R: DeviceRelation, S: DeviceRelation, load_factor: float = 
     dev = R.arena.device
     ws = alloc_ws(join_part_ws_bytes(R.n, S.n, load_factor, part_bits), dev)
     cap = cap_pairs if cap_pairs is not None else max(1024, S.n)
-    count = torch.zeros(1, dtype=torch.int64, device=dev)
+    count = torch.empty(1, dtype=torch.int64, device=dev)      # the call clears it
     while True:
         pairs = torch.empty(2 * max(cap, 1), dtype=torch.int32, device=dev)
         st, cnt = join_partitioned_into(R, S, ws, pairs, count, load_factor, part_bits, sync=True, stream=stream,
@@ -451,7 +451,7 @@ def baseline_join(R: DeviceRelation, S: DeviceRelation, load_factor: float = 0.5
     dev = R.arena.device
     ws = alloc_ws(baseline_ws_bytes(R.n, S.n, load_factor), dev)
     cap = cap_pairs if cap_pairs is not None else max(1024, S.n)
-    count = torch.zeros(1, dtype=torch.int64, device=dev)
+    count = torch.empty(1, dtype=torch.int64, device=dev)      # the call clears it
     while True:
         pairs = torch.empty(2 * max(cap, 1), dtype=torch.int32, device=dev)
         st, cnt = baseline_join_into(R, S, ws, pairs, count, load_factor, tagged, sync=True, stream=stream,

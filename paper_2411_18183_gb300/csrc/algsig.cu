@@ -1013,14 +1013,23 @@ static cudaError_t key_kernel_attrs() {
   if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 2, BATCH>();
   return e;
 }
+// a group of 32 keys per block, until every one of max_blocks has one
+static unsigned sig_blocks(uint64_t n, int max_blocks) {
+  const uint64_t want = (n + 31) / 32;
+  return (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
+}
 template <bool AT400, class Net, int SHAPE, bool BATCH>
 static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
-                              const BatchJoin* J, int nj, int s_side, uint64_t cap_len, cudaStream_t s) {
+                              const BatchJoin* J, int nj, int s_side, uint64_t cap_len, cudaStream_t s,
+                              LKSecond second = LKSecond(), int second_blocks = 0) {
   constexpr LKShape k = kLKShapes[SHAPE];
-  const uint64_t want = (n + 31) / 32;               // a group of 32 keys per block, until every SM has one
-  const unsigned blocks = (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
+  unsigned blocks = sig_blocks(n, max_blocks);
+  if (second_blocks > 0) {
+    second.from = blocks;
+    blocks += sig_blocks(second.n, second_blocks);
+  }
   sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>
-      <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len);
+      <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len, LKItems(), second);
 }
 template <bool AT400, class Net, bool BATCH>
 static void key_kernel_launch_shape(int shape, int sms, const uint8_t* arena, const uint64_t* off, uint64_t n,
@@ -1049,6 +1058,32 @@ struct DeviceState {
 
 static std::mutex g_dev_mu;
 static DeviceState g_dev[kMaxDevices];
+
+// Page-locked slots for the results that calls wait for, 64 of them for the
+// process (usable with every device), made with the first device's state; a
+// call holds one while it waits.
+constexpr int kResultSlots = 64;
+static uint64_t* g_results = nullptr;                 // two words per slot; null: none could be had
+static std::atomic<bool> g_result_taken[kResultSlots];
+class ResultSlot {
+  int i_ = -1;
+
+ public:
+  ResultSlot() {
+    if (!g_results) return;
+    for (int i = 0; i < kResultSlots; ++i)
+      if (!g_result_taken[i].exchange(true, std::memory_order_acquire)) {
+        i_ = i;
+        return;
+      }
+  }
+  ~ResultSlot() {
+    if (i_ >= 0) g_result_taken[i_].store(false, std::memory_order_release);
+  }
+  ResultSlot(const ResultSlot&) = delete;
+  ResultSlot& operator=(const ResultSlot&) = delete;
+  uint64_t* get() const { return i_ >= 0 ? g_results + 2 * i_ : nullptr; }
+};
 
 // GF tables by repeated multiplication by x (host), copied to the device once;
 // kernel attributes set once per device.
@@ -1196,6 +1231,13 @@ static as_status ensure_device(DeviceState** out) {
         cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.verify_blocks_per_sm < 1) d.verify_blocks_per_sm = 1;
+    if (!g_results) {
+      void* h = nullptr;
+      if (cudaHostAlloc(&h, kResultSlots * 16, cudaHostAllocPortable) == cudaSuccess)
+        g_results = static_cast<uint64_t*>(h);
+      else
+        cudaGetLastError();                            // without them results go to the stack
+    }
     d.ready = true;
   }
   *out = &d;
@@ -1208,6 +1250,27 @@ static unsigned walk_blocks(uint64_t n, int sms) {
   uint64_t want = (n + per_block - 1) / per_block;
   if (want > (uint64_t)sms) want = (uint64_t)sms;
   return (unsigned)(want < 1 ? 1 : want);
+}
+
+// One launch for what a join clears before it starts: bytes of table to all
+// ones (bytes a multiple of 16; the table 16-byte aligned), the error flags and
+// the counters to zero.  (Three memset calls took 4 us each on the host.)
+__global__ void clear_kernel(uint4* __restrict__ table, uint64_t chunks, uint32_t* flags, uint64_t* counts,
+                             uint64_t ncounts) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (uint64_t i = i0; i < chunks; i += stride) table[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  for (uint64_t i = i0; i < ncounts; i += stride) counts[i] = 0;
+  if (i0 == 0) *flags = 0;
+}
+static as_status launch_clear(const DeviceState* d, void* table, uint64_t bytes, uint32_t* flags, uint64_t* counts,
+                              uint64_t ncounts, cudaStream_t s) {
+  const uint64_t chunks = bytes / 16;
+  uint64_t blocks = ((chunks > ncounts ? chunks : ncounts) + 1023) / 1024;
+  const uint64_t lim = (uint64_t)d->sms * 8;
+  blocks = blocks < 1 ? 1 : (blocks < lim ? blocks : lim);
+  clear_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<uint4*>(table), chunks, flags, counts, ncounts);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? AS_OK : cuda_fail(e, "table clear");
 }
 
 static bool misaligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
@@ -1250,6 +1313,49 @@ static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t 
   return AS_OK;
 }
 
+// Blocks for R (m keys) and S (n keys) of a join in one launch.  A block of the signature kernel takes a whole SM, so
+// where there are at most four groups of 32 keys per warp of the device the SMs
+// are divided: R gets a warp for every group if that takes no more than a
+// quarter of them, else its share by key count.  Larger relations take all SMs
+// one after the other, which needs no guess about the keys' lengths.
+static void split_sms(int sms, uint64_t m, uint64_t n, int* blocks_r, int* blocks_s) {
+  const int warps = kLKShapes[0].warps;
+  const uint64_t groups = (m + 31) / 32 + (n + 31) / 32;
+  *blocks_r = *blocks_s = sms;
+  if (m == 0 || n == 0 || sms < 4 || groups > 4ull * sms * warps) return;
+  const int all = (int)(((m + 31) / 32 + warps - 1) / warps);   // a warp per group of R
+  const int share = (int)((double)sms * (double)m / (double)(m + n) + 0.5);
+  const int r = all <= sms / 4 ? all : share;
+  *blocks_r = r < 1 ? 1 : (r > sms - 1 ? sms - 1 : r);
+  *blocks_s = sms - *blocks_r;
+}
+
+// The signatures of a join's two relations in one launch (shape 0, four components).
+static as_status launch_sig_two(const DeviceState* d, const uint8_t* arenaR, const uint64_t* offR, uint64_t m,
+                                uint64_t* sigR, const uint8_t* arenaS, const uint64_t* offS, uint64_t n, uint64_t* sigS,
+                                uint64_t cap_len, cudaStream_t s) {
+  if (m == 0 || n == 0) {
+    if (m > 0) return launch_sig(arenaR, offR, m, sigR, s, 4, 0, 0, cap_len);
+    return launch_sig(arenaS, offS, n, sigS, s, 4, 0, 0, cap_len);
+  }
+  int blocks_r, blocks_s;
+  split_sms(d->sms, m, n, &blocks_r, &blocks_s);
+  LKSecond second;
+  second.arena = arenaS;
+  second.off = offS;
+  second.n = n;
+  second.sig_out = sigS;
+  if (d->tables_at400)
+    key_kernel_launch<true, Net16<4>, 0, false>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
+                                                blocks_s);
+  else
+    key_kernel_launch<false, Net16<4>, 0, false>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
+                                                 blocks_s);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
+  return AS_OK;
+}
+
 // The signatures of one side of a batch over its joins' row ranges (n virtual
 // rows; out indexed by virtual row), with the one-key-per-lane kernel.
 static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, const uint64_t* off, uint64_t n,
@@ -1261,25 +1367,6 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "batch signature kernel launch");
   return AS_OK;
-}
-
-// Blocks of the passes over R (m keys) and S (n keys) of a join whose two passes
-// run at the same time.  A block of the signature kernel takes a whole SM, so
-// where a pass has at most four groups of 32 keys per warp of the device the
-// SMs are divided and both run beside each other.  R's pass, which the build
-// waits for, gets a warp for every group if that takes no more than a quarter
-// of the SMs, else its share by key count.  Larger passes take all SMs one after
-// the other, which needs no guess about the keys' lengths.
-static void split_sms(int sms, uint64_t m, uint64_t n, int* blocks_r, int* blocks_s) {
-  const int warps = kLKShapes[0].warps;
-  const uint64_t groups = (m + 31) / 32 + (n + 31) / 32;
-  *blocks_r = *blocks_s = sms;
-  if (m == 0 || n == 0 || sms < 4 || groups > 4ull * sms * warps) return;
-  const int all = (int)(((m + 31) / 32 + warps - 1) / warps);   // a warp per group of R
-  const int share = (int)((double)sms * (double)m / (double)(m + n) + 0.5);
-  const int r = all <= sms / 4 ? all : share;
-  *blocks_r = r < 1 ? 1 : (r > sms - 1 ? sms - 1 : r);
-  *blocks_s = sms - *blocks_r;
 }
 
 // Work that may overlap the caller's stream s: fork() makes a side stream
@@ -1500,13 +1587,22 @@ size_t as_join_ws_bytes(uint64_t m, uint64_t n, float load_factor) {
 
 }  // extern "C"
 
-// as_join_build's work; max_blocks: most blocks of the signature kernel over R (0: one per SM).  R's
-// signatures and the insertions are two kernels: inserting each group right after its signatures makes
-// the signature kernel's 16 warps per SM wait for the table (1M keys of 256-1024 bytes: 326 us against
-// 160 + 55 us apart).
-static as_status build_impl(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
-                            const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
-                            as_stream stream, int max_blocks) {
+// R rows into the cleared table
+static as_status launch_build(const DeviceState* d, Slot* slots, uint64_t cap, const uint64_t* sigR, const uint64_t* offR,
+                              uint64_t m, uint32_t* flags, cudaStream_t s, uint64_t cap_len = ~0ull) {
+  if (m == 0) return AS_OK;
+  uint64_t blocks = (m + 255) / 256;
+  const uint64_t lim = (uint64_t)d->sms * 16;
+  if (blocks > lim) blocks = lim;
+  build_kernel<<<(unsigned)blocks, 256, 0, s>>>(slots, cap - 1, sigR, offR, m, flags, nullptr, 0, cap_len);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? AS_OK : cuda_fail(e, "build kernel launch");
+}
+
+// Checks of as_join_build's arguments, and its table's description over the workspace
+static as_status table_setup(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, const uint64_t* d_offR,
+                             const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor,
+                             as_table* out) {
   if (!out) return fail(AS_ERR_INVALID, "as_join_build: null table");
   uint64_t cap;
   uint32_t l2;
@@ -1518,36 +1614,14 @@ static as_status build_impl(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR
   const size_t need = as_join_table_bytes(m, load_factor);
   if (ws_bytes < need)
     return fail(AS_ERR_NOMEM, "as_join_build: workspace of %zu bytes, need %zu", ws_bytes, need);
-  DeviceState* d = nullptr;
-  as_status st = ensure_device(&d);
-  if (st != AS_OK) return st;
-  cudaStream_t s = (cudaStream_t)stream;
   uint8_t* ws = (uint8_t*)d_ws;
-  Slot* slots = (Slot*)ws;
   uint64_t* sig_ws = (uint64_t*)(ws + round256(cap * 16));
-  uint32_t* flags = (uint32_t*)(ws + round256(cap * 16) + round256(m * 8));
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(slots, 0xFF, cap * 16, s)) != cudaSuccess) return cuda_fail(e, "table clear");
-  if ((e = cudaMemsetAsync(flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
-  const uint64_t* sigR = d_sigR;
-  if (!sigR && m > 0) {
-    st = launch_sig(d_arenaR, d_offR, m, sig_ws, s, 4, 0, max_blocks);
-    if (st != AS_OK) return st;
-    sigR = sig_ws;
-  }
-  if (m > 0) {
-    uint64_t blocks = (m + 255) / 256;
-    const uint64_t lim = (uint64_t)d->sms * 16;
-    if (blocks > lim) blocks = lim;
-    build_kernel<<<(unsigned)blocks, 256, 0, s>>>(slots, cap - 1, sigR, d_offR, m, flags, nullptr, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "build kernel launch");
-  }
-  out->slots = reinterpret_cast<uint64_t*>(slots);
-  out->sigR = sigR ? sigR : sig_ws;
+  out->slots = reinterpret_cast<uint64_t*>(ws);
+  out->sigR = d_sigR ? d_sigR : sig_ws;
   out->arenaR = d_arenaR;
   out->offR = d_offR;
   out->idR = d_idR;
-  out->flags = flags;
+  out->flags = (uint32_t*)(ws + round256(cap * 16) + round256(m * 8));
   out->m = m;
   out->cap = cap;
   out->log2cap = l2;
@@ -1562,7 +1636,21 @@ as_status as_join_build(void* d_ws, size_t ws_bytes, const uint8_t* d_arenaR, co
                         const uint32_t* d_idR, uint64_t m, const uint64_t* d_sigR, float load_factor, as_table* out,
                         as_stream stream) {
   NvtxRange nvtx_range("as_join_build");
-  return build_impl(d_ws, ws_bytes, d_arenaR, d_offR, d_idR, m, d_sigR, load_factor, out, stream, 0);
+  as_table t;
+  as_status st = table_setup(d_ws, ws_bytes, d_arenaR, d_offR, d_idR, m, d_sigR, load_factor, out ? &t : nullptr);
+  if (st != AS_OK) return st;
+  DeviceState* d = nullptr;
+  if ((st = ensure_device(&d)) != AS_OK) return st;
+  cudaStream_t s = (cudaStream_t)stream;
+  Slot* slots = reinterpret_cast<Slot*>(t.slots);
+  if ((st = launch_clear(d, slots, t.cap * 16, t.flags, nullptr, 0, s)) != AS_OK) return st;
+  // (signatures and insertions are two kernels: inserting each group right after its signatures makes the
+  // signature kernel's 16 warps per SM wait for the table, 326 us for 1M keys of 256-1024 bytes against
+  // 160 + 55 us apart)
+  if (!d_sigR && (st = launch_sig(d_arenaR, d_offR, m, const_cast<uint64_t*>(t.sigR), s)) != AS_OK) return st;
+  if ((st = launch_build(d, slots, t.cap, t.sigR, d_offR, m, t.flags, s)) != AS_OK) return st;
+  *out = t;
+  return AS_OK;
 }
 
 size_t as_join_probe_ws_bytes(uint64_t n) { return (size_t)(round256(n * 8) + 256); }
@@ -1614,18 +1702,37 @@ static as_status launch_verify(DeviceState* d, const as_table* t, const uint8_t*
   return AS_OK;
 }
 
+// The pair count and the error flags at the end of a call that returns them:
+// copied to a page-locked slot and waited for once (a copy to pageable memory
+// waits by itself, 12 us a copy).  All slots taken, by more threads than there
+// are slots, or none to be had: copies to the stack.
+static as_status read_result(const uint64_t* d_count, const uint32_t* d_flags, uint64_t* cnt, uint32_t* flags,
+                             const char* what, cudaStream_t s) {
+  ResultSlot slot;
+  uint64_t stack[2] = {0, 0};
+  uint64_t* h = slot.get() ? slot.get() : stack;
+  h[1] = 0;
+  cudaError_t e;
+  if ((e = cudaMemcpyAsync(&h[0], d_count, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    return cuda_fail(e, "count readback");
+  if ((e = cudaMemcpyAsync(&h[1], d_flags, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess) {
+    cudaStreamSynchronize(s);                          // the first copy still writes the slot
+    return cuda_fail(e, "flag readback");
+  }
+  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, what);
+  *cnt = h[0];
+  memcpy(flags, &h[1], 4);
+  return AS_OK;
+}
+
 // optional synchronous count readback and error-flag check
 static as_status finish_probe(const char* fn, const as_table* t, uint64_t cap_pairs, uint64_t* d_count,
                               uint64_t* h_count, cudaStream_t s) {
   if (!h_count) return AS_OK;
   uint64_t cnt = 0;
   uint32_t flags = 0;
-  cudaError_t e;
-  if ((e = cudaMemcpyAsync(&cnt, d_count, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-    return cuda_fail(e, "count readback");
-  if ((e = cudaMemcpyAsync(&flags, t->flags, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-    return cuda_fail(e, "flag readback");
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "probe");
+  const as_status st = read_result(d_count, t->flags, &cnt, &flags, "probe", s);
+  if (st != AS_OK) return st;
   *h_count = cnt;
   if (flags & kFlagTableFull) return fail(AS_ERR_TABLE_FULL, "%s: the build could not place every row", fn);
   if (cnt > cap_pairs)
@@ -1750,23 +1857,17 @@ as_status as_join(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_
   uint64_t* cnt = d_count ? d_count : (uint64_t*)rest;
   cudaStream_t s = (cudaStream_t)stream;
   as_table t;
-  // S's signatures on a side stream, concurrently with R's signatures and the build (kernels of small
-  // relations leave SMs idle), then the probe
-  SideStream side;
-  int blocks_r, blocks_s;
-  split_sms(d->sms, m, n, &blocks_r, &blocks_s);
-  if (n > 0) {
-    if ((st = side.fork(d, s)) != AS_OK) return st;
-    if ((st = launch_sig(d_arenaS, d_offS, n, sigS, side.side, 4, 0, blocks_s)) != AS_OK) {
-      side.join();
-      return st;
-    }
-  }
-  st = build_impl(d_ws, tb, d_arenaR, d_offR, d_idR, m, nullptr, load_factor, &t, stream, blocks_r);
-  const as_status js = side.join();
-  if (st != AS_OK) return st;
-  if (js != AS_OK) return js;
-  return as_join_probe_sigs(&t, d_arenaS, d_offS, d_idS, n, sigS, d_pairs, cap_pairs, cnt, h_count, stream);
+  if ((st = table_setup(d_ws, tb, d_arenaR, d_offR, d_idR, m, nullptr, load_factor, &t)) != AS_OK) return st;
+  if ((st = probe_args("as_join", &t, d_arenaS, d_offS, n, d_pairs, cap_pairs, cnt)) != AS_OK) return st;
+  Slot* slots = reinterpret_cast<Slot*>(t.slots);
+  if ((st = launch_clear(d, slots, t.cap * 16, t.flags, cnt, 1, s)) != AS_OK) return st;
+  if ((st = launch_sig_two(d, d_arenaR, d_offR, m, const_cast<uint64_t*>(t.sigR), d_arenaS, d_offS, n, sigS, ~0ull,
+                           s)) != AS_OK)
+    return st;
+  if ((st = launch_build(d, slots, t.cap, t.sigR, d_offR, m, t.flags, s)) != AS_OK) return st;
+  if (n > 0 && (st = launch_verify(d, &t, d_arenaS, d_offS, d_idS, n, sigS, d_pairs, cap_pairs, cnt, s)) != AS_OK)
+    return st;
+  return finish_probe("as_join", &t, cap_pairs, cnt, h_count, s);
 }
 
 // ----------------------------------------------------------------------------
@@ -1813,17 +1914,9 @@ as_status as_join_prefix(const uint8_t* d_arenaR, const uint64_t* d_offR, const 
   uint32_t* flags = (uint32_t*)tail;
   uint64_t* cnt = d_count ? d_count : (uint64_t*)(tail + 256);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(slots, 0xFF, cap * 16, s)) != cudaSuccess) return cuda_fail(e, "table clear");
-  if ((e = cudaMemsetAsync(flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
-  if ((e = cudaMemsetAsync(cnt, 0, 8, s)) != cudaSuccess) return cuda_fail(e, "counter clear");
-  if ((st = launch_sig(d_arenaR, d_offR, m, sigR, s, 4, 0, 0, prefix_len)) != AS_OK) return st;
-  if (m > 0) {
-    uint64_t blocks = (m + 255) / 256;
-    const uint64_t lim = (uint64_t)d->sms * 16;
-    if (blocks > lim) blocks = lim;
-    build_kernel<<<(unsigned)blocks, 256, 0, s>>>(slots, cap - 1, sigR, d_offR, m, flags, nullptr, 0, prefix_len);
-  }
-  if ((st = launch_sig(d_arenaS, d_offS, n, sigS, s, 4, 0, 0, prefix_len)) != AS_OK) return st;
+  if ((st = launch_clear(d, slots, cap * 16, flags, cnt, 1, s)) != AS_OK) return st;
+  if ((st = launch_sig_two(d, d_arenaR, d_offR, m, sigR, d_arenaS, d_offS, n, sigS, prefix_len, s)) != AS_OK) return st;
+  if ((st = launch_build(d, slots, cap, sigR, d_offR, m, flags, s, prefix_len)) != AS_OK) return st;
   if (n > 0) {
     as_table t;
     memset(&t, 0, sizeof(t));
@@ -1844,10 +1937,7 @@ as_status as_join_prefix(const uint8_t* d_arenaR, const uint64_t* d_offR, const 
   if (h_count) {
     uint64_t c = 0;
     uint32_t flags_h = 0;
-    if ((e = cudaMemcpyAsync(&c, cnt, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e, "count readback");
-    if ((e = cudaMemcpyAsync(&flags_h, flags, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-      return cuda_fail(e, "flag readback");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "prefix join");
+    if ((st = read_result(cnt, flags, &c, &flags_h, "prefix join", s)) != AS_OK) return st;
     *h_count = c;
     if (flags_h & kFlagTableFull) return fail(AS_ERR_TABLE_FULL, "as_join_prefix: build overflow");
     if (c > cap_pairs)
@@ -1975,10 +2065,7 @@ as_status as_join_partitioned(const uint8_t* d_arenaR, const uint64_t* d_offR, c
   if (h_count) {
     uint64_t c = 0;
     uint32_t flags_h = 0;
-    if ((e = cudaMemcpyAsync(&c, cnt, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e, "count readback");
-    if ((e = cudaMemcpyAsync(&flags_h, flags, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-      return cuda_fail(e, "flag readback");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "partitioned join");
+    if ((st = read_result(cnt, flags, &c, &flags_h, "partitioned join", s)) != AS_OK) return st;
     *h_count = c;
     if (flags_h & kFlagTableFull) return fail(AS_ERR_TABLE_FULL, "as_join_partitioned: build overflow");
     if (c > cap_pairs)
@@ -2103,10 +2190,7 @@ as_status as_baseline_join(const uint8_t* d_arenaR, const uint64_t* d_offR, cons
   if (h_count) {
     uint64_t c = 0;
     uint32_t flags_h = 0;
-    if ((e = cudaMemcpyAsync(&c, cnt, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return cuda_fail(e, "count readback");
-    if ((e = cudaMemcpyAsync(&flags_h, flags, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-      return cuda_fail(e, "flag readback");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "baseline join");
+    if ((st = read_result(cnt, flags, &c, &flags_h, "baseline join", s)) != AS_OK) return st;
     *h_count = c;
     if (flags_h & kFlagTableFull) return fail(AS_ERR_TABLE_FULL, "as_baseline_join: build overflow");
     if (c > cap_pairs)
@@ -2222,9 +2306,7 @@ as_status as_join_batch_run(const as_batch* b, const uint8_t* d_arenaR, const ui
   BatchJoin* J = reinterpret_cast<BatchJoin*>(b->descs);
   const int nj = (int)b->n_joins;
   Slot* slots = reinterpret_cast<Slot*>(b->slots);
-  if ((e = cudaMemsetAsync(slots, 0xFF, b->slots_total * 16, s)) != cudaSuccess) return cuda_fail(e, "table clear");
-  if ((e = cudaMemsetAsync(b->flags, 0, 4, s)) != cudaSuccess) return cuda_fail(e, "flag clear");
-  if ((e = cudaMemsetAsync(d_counts, 0, 8 * b->n_joins, s)) != cudaSuccess) return cuda_fail(e, "counter clear");
+  if ((st = launch_clear(d, slots, b->slots_total * 16, b->flags, d_counts, b->n_joins, s)) != AS_OK) return st;
   batch_bytes_kernel<<<1, 1024, 0, s>>>(J, nj, d_offR, d_offS);
   // S's signatures on a side stream, concurrently with R's signatures and the builds
   SideStream side;

@@ -569,7 +569,7 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
                                               const uint64_t* __restrict__ off, uint64_t n, uint64_t warp,
                                               uint64_t nwarps, bool by_count, uint64_t* lo, uint64_t* hi) {
   if (n <= 32 * nwarps) {                            // at most one group per warp
-    const uint64_t u = (warp % kWarps) * gridDim.x + warp / kWarps;   // neighbouring groups on different SMs
+    const uint64_t u = (warp % kWarps) * (nwarps / kWarps) + warp / kWarps;   // neighbouring groups on different SMs
     *lo = 32 * u < n ? 32 * u : n;
     *hi = 32 * u + 32 < n ? 32 * u + 32 : n;
     return;
@@ -704,6 +704,17 @@ __device__ __forceinline__ void lk_item_window(LKWarp& W, uint8_t* rows, const u
   guess = kb - k0 < 128u ? (uint32_t)(kb - k0) + 2u : 128u;
 }
 
+// A second relation that the same launch signs, with the blocks from `from` on
+// (a join's S beside its R: one launch, and the two share the SMs where both
+// are small).
+struct LKSecond {
+  const uint8_t* arena = nullptr;
+  const uint64_t* off = nullptr;
+  uint64_t n = 0;
+  uint64_t* sig_out = nullptr;
+  uint32_t from = 0xFFFFFFFFu;
+};
+
 // The signatures of n keys: the rows of a relation (BATCH false), or the
 // virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
 // describe the joins, and sig_out is indexed by virtual row); of each key's
@@ -713,7 +724,8 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
                                                                 const BatchJoin* __restrict__ J, int nj, int s_side,
-                                                                uint64_t cap_len, const LKItems items = LKItems()) {
+                                                                uint64_t cap_len, const LKItems items = LKItems(),
+                                                                const LKSecond second = LKSecond()) {
   if constexpr (ITEMS) {
     if (!by_items(off, n, items.block)) return;
   }
@@ -728,8 +740,21 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   const uint32_t lane = threadIdx.x & 31u;
   LKWarp& W = warps[wib];
   // the warp's keys and its first window's offsets first, so that their loads overlap the tables' copy
-  const uint64_t warp = (uint64_t)blockIdx.x * kLKWarps + wib;
-  const uint64_t nwarps = (uint64_t)gridDim.x * kLKWarps;
+  uint32_t block = blockIdx.x, nblocks = gridDim.x;
+  if constexpr (!BATCH && !ITEMS) {
+    if (block >= second.from) {
+      arena = second.arena;
+      off = second.off;
+      n = second.n;
+      sig_out = second.sig_out;
+      block -= second.from;
+      nblocks -= second.from;
+    } else if (second.from < nblocks) {
+      nblocks = second.from;
+    }
+  }
+  const uint64_t warp = (uint64_t)block * kLKWarps + wib;
+  const uint64_t nwarps = (uint64_t)nblocks * kLKWarps;
   uint64_t k_lo, k_hi, kb = 0;                      // kb (items): the key of the window's first item
   uint32_t most = kLKWin;
   if constexpr (ITEMS) {

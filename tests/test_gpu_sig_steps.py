@@ -57,3 +57,21 @@ def test_ranges_cut_by_work(cuda, lo, hi):
     out = torch.full((n,), -1, dtype=torch.int64, device="cuda")
     got = ag.sig_compute(R, out).cpu().numpy().view(np.uint64)
     assert np.array_equal(got, oracle.sig_batch(host, off, nthreads=8))
+
+
+@pytest.mark.parametrize("groups,rest", [(1, -1), (1, 0), (1, 1), (2, 31), (3, 0), (6, 17)])
+def test_ranges_of_whole_groups(cuda, groups, rest):
+    """Below 2^19 keys the warps get whole groups of 32 keys: around one, two, three and six groups per
+    warp of each block shape, every key is signed exactly once."""
+    ag = cuda
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for shape, (warps, _) in enumerate(ag.sig_shapes()):
+        n = 32 * sms * warps * groups + rest
+        rng = np.random.default_rng(n)
+        off = np.zeros(n + 1, np.uint64)
+        off[1:] = np.cumsum(rng.integers(0, 70, n).astype(np.uint64))
+        host = rng.integers(0, 256, workloads.padded_size(int(off[-1])), dtype=np.uint8)
+        R = ag.DeviceRelation.from_host(host, off)
+        out = torch.full((n,), -1, dtype=torch.int64, device="cuda")
+        got = ag.sig_compute(R, out, shape=shape).cpu().numpy().view(np.uint64)
+        assert np.array_equal(got, oracle.sig_batch(host, off, nthreads=8)), shape

@@ -461,13 +461,18 @@ __device__ __forceinline__ void flush_stage(const Stage& st, uint32_t np, const 
 // that gain.)
 struct Cand {
   uint4 a;                   // S start (64 bits), S row (64 bits); while verified: the aligned bases of S and R
-  uint4 b;                   // R row, length (32 bits), join of a batch, lane; while verified: end, alignment, row, join or lane
-};
+  uint4 b;                   // R row, length (32 bits), tag; while verified: end, alignment, R row, tag
+};                           // (tag: the join of a batch, or which of the warp's rows with an open record)
 constexpr uint32_t kVDrain = 32;             // candidates verified at a time
 constexpr uint32_t kVQueue = 80;             // a probe step (32 new ones at most) runs while 48 or fewer wait
+// Where S rows' own records may be asked for: the groups of 32 S rows whose candidates are verified together
+// and whose records are put out then.  One group's candidates rarely fill the warp's 32 places (semi-join of
+// 500k rows of 200-2000 bytes, a fifth of them in R, signatures and probe: 1 group 320 us, 4 310, 8 308, 16 313).
+constexpr uint32_t kVOpen = 4;
 struct CandQueue {
   Cand q[kVQueue];
   uint64_t ids[kVDrain];     // the ids of the candidates being verified
+  uint32_t matched[kVOpen];  // a bit per S row of the open groups: a candidate was verified
 };
 // Chunks of each lane in flight: with 4 blocks of 64 registers two fit without spills (large join, blocks x
 // chunks: 4 x 2 2.83 ms, 3 x 4 2.85, 3 x 3 2.96, 4 x 3 3.02, 4 x 1 3.11)
@@ -479,12 +484,12 @@ constexpr uint32_t kVFourMax = 2048;
 
 // the candidates of a probe step (lanes with `cand`) to the end of the queue
 __device__ __forceinline__ void queue_push(Cand* q, uint32_t& cnt, bool cand, uint64_t start, uint64_t srow,
-                                           uint32_t row, uint32_t l32, uint32_t jn) {
+                                           uint32_t row, uint32_t l32, uint32_t tag) {
   const uint32_t m = __ballot_sync(kFull, cand);
   if (cand) {
     Cand& e = q[cnt + (uint32_t)__popc(m & lanemask_lt())];
     e.a = make_uint4((uint32_t)start, (uint32_t)(start >> 32), (uint32_t)srow, (uint32_t)(srow >> 32));
-    e.b = make_uint4(row, l32, jn, threadIdx.x & 31u);
+    e.b = make_uint4(row, l32, tag, 0u);
   }
   cnt += (uint32_t)__popc(m);
   __syncwarp();
@@ -571,12 +576,13 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
 }
 
 // Verify the nc (at most 32) candidates at q and put out what the mode asks for
-// each verified one; returns a bit per lane that queued a verified candidate.
+// each verified one; returns whether the lane's candidate is verified, its tag
+// in *tag_out.
 // Between its parts the candidates' fields are in shared memory, not in
 // registers: the comparison needs those for the bytes in flight.
 template <bool BATCH, bool INNER>
-__device__ __forceinline__ uint32_t queue_verify(Cand* q, uint64_t* ids, uint32_t nc, const VerifyParams& P,
-                                                 const uint4* emask) {
+__device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc, const VerifyParams& P,
+                                             const uint4* emask, uint32_t* tag_out) {
   const uint32_t lane = threadIdx.x & 31u;
   const int mode = BATCH || INNER ? (int)AS_JOIN_INNER : P.mode;
   const bool pairs = mode == AS_JOIN_INNER || mode == AS_JOIN_OUTER_S || mode == AS_JOIN_OUTER_R ||
@@ -593,7 +599,7 @@ __device__ __forceinline__ uint32_t queue_verify(Cand* q, uint64_t* ids, uint32_
       srow = (uint64_t)a.z | ((uint64_t)a.w << 32);
       row = b.x;
       l32 = b.y;
-      tag = BATCH ? b.z : b.w;
+      tag = b.z;
       rs = __ldg(P.offR + row);
       if (pairs) {
         uint64_t rb = 0, sb = 0;
@@ -655,9 +661,9 @@ __device__ __forceinline__ uint32_t queue_verify(Cand* q, uint64_t* ids, uint32_
       }
     }
   }
-  const uint32_t m = INNER || BATCH ? 0u : __reduce_or_sync(kFull, eq ? 1u << (tag & 31u) : 0u);
+  *tag_out = tag;
   __syncwarp();
-  return m;
+  return eq;
 }
 
 // BATCH: the S rows of a batch's joins; INNER: the plain inner join of one
@@ -671,10 +677,11 @@ __global__ void __launch_bounds__(kVThreads, kVBlocks) verify_kernel(const __gri
   const uint32_t lane = threadIdx.x & 31u;
   CandQueue& Q = queue_all[threadIdx.x >> 5];
   uint32_t cnt = 0;                                  // candidates waiting
-  uint32_t matched = 0;                              // a bit per lane whose S row has a verified match
   const uint64_t ngroups = (P.n + 31) / 32;
   const uint64_t nwarps = (uint64_t)gridDim.x * kVWarps;
-  constexpr bool kRows = !BATCH && !INNER;           // a group's rows may have to know their matches
+  constexpr bool kRows = !BATCH && !INNER;           // S rows' own records may be asked for
+  uint32_t open = 0;                                 // then: the group among the open ones
+  if (kRows && lane < kVOpen) Q.matched[lane] = 0;
   bool resume = false;                               // a group was left with lanes on their way, for a full queue
   volatile uint64_t saved[3];                        // then: the lane's place in its bucket sequence, and whether it goes on
   for (uint64_t grp = (uint64_t)blockIdx.x * kVWarps + (threadIdx.x >> 5); grp < ngroups;) {
@@ -737,7 +744,7 @@ __global__ void __launch_bounds__(kVThreads, kVBlocks) verify_kernel(const __gri
             }
           }
         }
-        queue_push(Q.q, cnt, cand, start, i, row, l32, jn);
+        queue_push(Q.q, cnt, cand, start, i, row, l32, BATCH ? jn : 32u * open + lane);
         resume = __any_sync(kFull, live);
       } while (resume && cnt <= kVQueue - kVDrain);
       if (resume) {
@@ -746,24 +753,37 @@ __global__ void __launch_bounds__(kVThreads, kVBlocks) verify_kernel(const __gri
         saved[2] = live ? 1u : 0u;
       }
     }
-    const bool flush = resume || kRows || grp + nwarps >= ngroups;
+    const bool last = grp + nwarps >= ngroups, close = kRows && !resume && (open + 1 == kVOpen || last);
+    const bool flush = resume || last || close;
     while (cnt >= kVDrain || (flush && cnt)) {
       const uint32_t nc = cnt < kVDrain ? cnt : kVDrain;
       cnt -= nc;
-      matched |= queue_verify<BATCH, INNER>(Q.q + cnt, Q.ids, nc, P, emask);
+      uint32_t tag;
+      const bool eq = queue_verify<BATCH, INNER>(Q.q + cnt, Q.ids, nc, P, emask, &tag);
+      if (kRows && eq) atomicOr(&Q.matched[tag >> 5], 1u << (tag & 31u));
     }
     if (resume) continue;                            // the same group's next steps
-    if (kRows && (P.mode == AS_JOIN_SEMI || P.mode == AS_JOIN_ANTI || P.mode == AS_JOIN_OUTER_S)) {
-      // one (AS_NO_ROW, s_id) per selected S row
-      const bool emit = vi < P.n && (((matched >> lane) & 1u) != 0u) == (P.mode == AS_JOIN_SEMI);
-      const uint32_t em = __ballot_sync(kFull, emit);
-      unsigned long long base = 0;
-      if (lane == 0 && em) base = atomicAdd(P.count, (unsigned long long)__popc(em));
-      base = __shfl_sync(kFull, base, 0) + (unsigned long long)__popc(em & lanemask_lt());
-      if (emit && base < P.cap)
-        reinterpret_cast<uint64_t*>(P.pairs)[base] = pair_ids(AS_NO_ROW, vi, P.idR, P.idS, 0, 0);
+    if (close) {
+      if (P.mode == AS_JOIN_SEMI || P.mode == AS_JOIN_ANTI || P.mode == AS_JOIN_OUTER_S) {
+        // one (AS_NO_ROW, s_id) per selected S row
+        __syncwarp();
+#pragma unroll 1
+        for (uint32_t u = 0; u <= open; ++u) {
+          const uint64_t r = (grp - (open - u) * nwarps) * 32 + lane;
+          const bool emit = r < P.n && (((Q.matched[u] >> lane) & 1u) != 0u) == (P.mode == AS_JOIN_SEMI);
+          const uint32_t em = __ballot_sync(kFull, emit);
+          unsigned long long base = 0;
+          if (lane == 0 && em) base = atomicAdd(P.count, (unsigned long long)__popc(em));
+          base = __shfl_sync(kFull, base, 0) + (unsigned long long)__popc(em & lanemask_lt());
+          if (emit && base < P.cap)
+            reinterpret_cast<uint64_t*>(P.pairs)[base] = pair_ids(AS_NO_ROW, r, P.idR, P.idS, 0, 0);
+        }
+      }
+      __syncwarp();
+      if (lane < kVOpen) Q.matched[lane] = 0;
+      __syncwarp();
     }
-    matched = 0;
+    if (kRows) open = close ? 0u : open + 1u;
     grp += nwarps;
   }
 }

@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(kVThreads, kVBlocks) part_probe_kernel(const _
     while (cnt >= kVDrain || (flush && cnt)) {
       const uint32_t nc = cnt < kVDrain ? cnt : kVDrain;
       cnt -= nc;
-      queue_verify<false, true>(W.q + cnt, W.ids, nc, P, emask);
+      uint32_t tag;
+      queue_verify<false, true>(W.q + cnt, W.ids, nc, P, emask, &tag);
     }
     if (!resume) grp += nwarps;
   }

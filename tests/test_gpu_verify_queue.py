@@ -95,3 +95,38 @@ def test_many_groups_per_warp(cuda, mode):
     assert np.array_equal(got[:, 1], np.nonzero(rows)[0])
     want_r = np.where(miss | (mode in ("semi", "anti")), NO_ROW, src)[rows]
     assert np.array_equal(got[:, 0], want_r)
+
+
+@pytest.mark.parametrize("per_warp,rest", [(1, 1), (4, 0), (4, 33), (5, 5), (9, 31)])
+@pytest.mark.parametrize("mode", ["outer_s", "semi", "anti"])
+def test_open_groups(cuda, mode, per_warp, rest):
+    """S rows' records are put out for a few groups of 32 rows at a time: around those groups, with
+    one or several equal R keys (so that the queue also drains, or is left full, between them)."""
+    ag = cuda
+    rng = np.random.default_rng(10 * per_warp + rest)
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 16
+    m, n, w = 400, 32 * warps * per_warp + rest, 8
+    r = rng.integers(0, 256, (m, w), dtype=np.uint8)
+    r[m // 2:m // 2 + 9] = r[0]                            # ten equal R keys
+    src = rng.integers(0, m, n)
+    src[n // 3:n // 3 + 64] = 0                            # two groups that overfill the queue
+    s = r[src].copy()
+    miss = rng.random(n) < 0.6
+    miss[n // 3:n // 3 + 64] = False
+    s[miss] ^= 255
+    mk = lambda a, k: ag.DeviceRelation.from_host(np.concatenate([a.ravel(), np.zeros(16, np.uint8)]),
+                                                  np.arange(k + 1, dtype=np.uint64) * np.uint64(w))
+    dR, dS = mk(r, m), mk(s, n)
+    ws = ag.alloc_ws(ag.join_table_bytes(m))
+    table = ag.join_build(dR, ws)
+    keys = {}
+    for i, k in enumerate(r):
+        keys.setdefault(k.tobytes(), []).append(i)
+    hits = [keys.get(k.tobytes(), []) for k in s]
+    want = {"semi": [(NO_ROW, j) for j in range(n) if hits[j]], "anti": [(NO_ROW, j) for j in range(n) if not hits[j]],
+            "outer_s": [(i, j) for j in range(n) for i in (hits[j] or [NO_ROW])]}[mode]
+    pairs = torch.empty(2 * (len(want) + 1), dtype=torch.int32, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    cnt = ag.join_probe_mode(table, dS, ag.sig_compute(dS), pairs, count, mode=mode)
+    got = pairs[:2 * cnt].cpu().numpy().view(np.uint32).reshape(-1, 2)
+    assert sorted(map(tuple, got.tolist())) == sorted(want)

@@ -479,7 +479,8 @@ struct CandQueue {
 constexpr int kVAhead = 2;
 // Longest key compared by eight lanes: the whole warp's 512 bytes in a row take fewer requests (400k
 // candidates of 2-8 KB: 821 us with eight lanes, 750 us with the warp, when the line was drawn; 679 us now),
-// eight lanes fewer instructions and waits per candidate (5M of 256-1024 bytes: 1.3 against 1.7 ms)
+// eight lanes fewer instructions and waits per candidate (5M of 256-1024 bytes: 1.3 against 1.7 ms, both in the
+// queue's order)
 constexpr uint32_t kVFourMax = 2048;
 
 // the candidates of a probe step (lanes with `cand`) to the end of the queue
@@ -575,6 +576,27 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
   return __reduce_or_sync(kFull, diff != 0u ? 1u << c : 0u);
 }
 
+// The place of the lane-th shortest of the nc candidates at q: those compared side by side are then about
+// equally long, and the long ones among them come last.  A bitonic sorting network over the warp (Batcher,
+// 1968), left out where all are equally long.  (Large join 1321 -> 1230 us, 2-8 KB 682 -> 630, semi-join of
+// 200-2000 bytes 82 -> 68.  Neither chunks without bounds checks inside all four keys nor prefetching the next
+// candidates' keys into L2 gave more: no single unit is full, ALU 65 %, L1 55 %, DRAM 45 %.)
+__device__ __forceinline__ uint32_t by_length(const Cand* q, uint32_t nc) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t len = q[lane < nc ? lane : 0u].b.y;
+  if (__reduce_min_sync(kFull, len) == __reduce_max_sync(kFull, len)) return lane;
+  uint32_t key = (lane < nc ? min(len, 0x7FFFFFEu) : 0x7FFFFFFu) << 5 | lane;
+#pragma unroll
+  for (uint32_t k = 2; k <= 32u; k <<= 1) {
+#pragma unroll
+    for (uint32_t j = k >> 1; j; j >>= 1) {
+      const uint32_t other = __shfl_xor_sync(kFull, key, (int)j);
+      key = ((lane & j) != 0u) != ((lane & k & 31u) != 0u) ? max(key, other) : min(key, other);
+    }
+  }
+  return key & 31u;
+}
+
 // Verify the nc (at most 32) candidates at q and put out what the mode asks for
 // each verified one; returns whether the lane's candidate is verified, its tag
 // in *tag_out.
@@ -588,13 +610,14 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
   const bool pairs = mode == AS_JOIN_INNER || mode == AS_JOIN_OUTER_S || mode == AS_JOIN_OUTER_R ||
                      mode == AS_JOIN_SIG_ONLY;
   const bool bytes = BATCH || mode != AS_JOIN_SIG_ONLY;   // signature-only: no byte comparison
-  uint32_t todo, bad = 0, lg = 3u;
+  uint32_t todo, bad = 0, few;                       // few: how many are compared by eight lanes
   {
+    const uint32_t at = by_length(q, nc);
     const bool have = lane < nc;
     uint64_t start = 0, srow = 0, rs = 0;
     uint32_t row = 0, l32 = 0, tag = 0;
     if (have) {
-      const uint4 a = q[lane].a, b = q[lane].b;
+      const uint4 a = q[at].a, b = q[at].b;
       start = (uint64_t)a.x | ((uint64_t)a.y << 32);
       srow = (uint64_t)a.z | ((uint64_t)a.w << 32);
       row = b.x;
@@ -612,7 +635,7 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
     }
     const bool wide = have && l32 >= kNarrowLen;       // lengths that the slot's 32-bit field saturates
     todo = __ballot_sync(kFull, have && !wide && bytes && l32 > 0u);
-    if (__any_sync(kFull, have && l32 > kVFourMax)) lg = 5u;
+    few = (uint32_t)__popc(__ballot_sync(kFull, have && l32 <= kVFourMax));
     for (uint32_t wm = __ballot_sync(kFull, wide); wm; wm &= wm - 1u) {   // one by one, in 64-bit offsets
       const int c = __ffs((int)wm) - 1;
       const uint64_t rsc = __shfl_sync(kFull, rs, c), ssc = __shfl_sync(kFull, start, c);
@@ -634,10 +657,9 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
     }
     __syncwarp();
   }
-  if (lg == 3u)
-    for (uint32_t r = 0; r < nc; r += 4u) bad |= compare_some<3>(q, r, todo, emask);
-  else
-    for (uint32_t r = 0; r < nc; ++r) bad |= compare_some<5>(q, r, todo, emask);
+  uint32_t r = 0;
+  for (; r < few; r += 4u) bad |= compare_some<3>(q, r, todo, emask);
+  for (; r < nc; ++r) bad |= compare_some<5>(q, r, todo, emask);
   const bool eq = lane < nc && !((bad >> lane) & 1u);
   const uint32_t row = q[lane].b.z, tag = q[lane].b.w;   // (defined where eq)
   if (!BATCH && !INNER && eq && mode >= AS_JOIN_OUTER_R) atomicOr(P.matched + (row >> 5), 1u << (row & 31u));

@@ -6,10 +6,11 @@
 //   3. probe with S         sig_key_kernel on S, then verify_kernel: table
 //                           walk, byte-exact verification, output compaction
 //                           (formulas 4-5)
-// sig_key_kernel computes one key per lane (keys grouped by length, a
-// bit-sliced Horner state for three of the four components).  A batch whose
-// joins' rows are not one run of the relation uses sig_kernel, the warp tile
-// walk of rounds.cuh over the joins' row ranges.
+// sig_key_kernel computes one key per lane (keys grouped by length, bit-sliced
+// states); a whole join signs both relations in one launch of it, and a batch
+// runs it over the joins' rows.  The other kernels' own files: partition.cuh
+// (the radix-partitioned join), prefix.cuh (cumulative signatures),
+// baseline.cuh (the comparison join on full strings).
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -51,11 +52,6 @@ constexpr uint32_t kFlagTableFull = 1u;
 constexpr uint64_t kMaxPrefixLen = 0xFFFFFFF0ull;  // the prefix join's L: one prefix block of at most this many bytes
 constexpr int kMaxDevices = 64;
 
-// shared memory: reduction tables | their scratch | per-warp double buffers | per-warp pair buffers
-constexpr size_t kSmemTables = (size_t)kRedBytes + 512 * 4;
-constexpr size_t kSmemBufs = (size_t)kWarpsPerBlock * 2 * kBufBytes;
-constexpr size_t kSmemSig = kSmemTables + kConstBytes + kSmemBufs;
-static_assert(kConstEntries == 17 * 512, "constant table size");
 
 // ----------------------------------------------------------------------------
 // Batches of joins
@@ -244,9 +240,9 @@ __global__ void build_kernel(Slot* __restrict__ slots, uint64_t mask, const uint
 
 // ----------------------------------------------------------------------------
 // Probe: table walk + byte-exact verification + output compaction.  The S
-// signatures come from sig_kernel; this kernel needs no large shared memory,
-// so it runs at full occupancy and hides the latency of its random accesses
-// (slots, R offsets, key bytes) behind many warps.
+// signatures come from sig_key_kernel; this kernel needs little shared memory,
+// so that 32 warps per SM hide the latency of its random accesses (slots, R
+// offsets, key bytes).
 // ----------------------------------------------------------------------------
 
 constexpr int kVThreads = 256;
@@ -323,7 +319,7 @@ __device__ __noinline__ bool warp_equal_wide(const uint8_t* __restrict__ aR, uin
   return true;
 }
 
-// Keys below kNarrowLen (loopbounds.h) are compared with 32-bit offsets (warp_equal).
+// Keys below kNarrowLen (loopbounds.h) are compared with 32-bit offsets (compare_some, warp_equal).
 
 // emask[e]: the first e bytes of a 16-byte chunk (e = 0..16), in shared memory.
 __device__ __forceinline__ void fill_emask(uint4* emask) {
@@ -338,15 +334,6 @@ __device__ __forceinline__ void fill_emask(uint4* emask) {
   }
 }
 
-// Byte equality of the len-byte keys at pR and pS (len < kNarrowLen) by the
-// whole warp, 512 bytes per step.  Offsets count from the aligned chunk bS
-// that holds the S key's first byte: S key bytes are [sa, sa + len); bR is
-// the aligned R chunk that holds the R byte matching bS + 0 minus its
-// misalignment d, so that lane l's S chunk [off, off + 16) meets the R bytes
-// [off + d, off + d + 16) of the two aligned R chunks at bR + off and
-// bR + off + 16, realigned by a funnel shift of d bytes (the word part of d is
-// warp-uniform).  Only aligned chunks that hold a key byte are read.  Only the
-// steps that hold the key's first or last byte apply byte masks.
 // realigned R words of one lane for the misalignment d (word part warp-uniform)
 __device__ __forceinline__ void realign_r(const uint4& ra, const uint4& rb, uint32_t d, uint32_t sh, uint32_t& r0,
                                           uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -379,7 +366,8 @@ __device__ __forceinline__ void realign_r(const uint4& ra, const uint4& rb, uint
 // misalignment d).  Both halves' loads are issued before either is compared,
 // so a key of up to 1 KB costs one memory round trip.  Only aligned chunks
 // that hold a key byte are read; only the steps that hold the key's first or
-// last byte apply byte masks.
+// last byte apply byte masks.  (The comparison join's; the probe's candidates go
+// through compare_some.)
 __device__ __forceinline__ bool warp_equal(const uint8_t* __restrict__ pR, const uint8_t* __restrict__ pS,
                                            uint32_t len, const uint4* __restrict__ emask) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -422,7 +410,7 @@ __device__ __forceinline__ bool warp_equal(const uint8_t* __restrict__ pR, const
   return true;
 }
 
-// Verified pairs staged per warp as rows; their ids are looked up when the
+// The comparison join's verified pairs staged per warp as rows; their ids are looked up when the
 // stage is flushed, by all lanes at once (a per-pair lookup would make the
 // warp wait on memory once more per pair).
 struct Stage {
@@ -1071,7 +1059,8 @@ static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64
     blocks += sig_blocks(second.n, second_blocks);
   }
   sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>
-      <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len, LKItems(), second);
+      <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len,
+                                                                           LKItems(), second);
 }
 template <bool AT400, class Net, bool BATCH>
 static void key_kernel_launch_shape(int shape, int sms, const uint8_t* arena, const uint64_t* off, uint64_t n,
@@ -1095,8 +1084,6 @@ struct DeviceState {
   cudaStream_t side[kSideStreams] = {};   // side streams (SideStream), created with the state
   std::atomic<unsigned> side_next{0};
 };
-
-// launch the signature kernel instantiation that matches the device
 
 static std::mutex g_dev_mu;
 static DeviceState g_dev[kMaxDevices];
@@ -1240,10 +1227,11 @@ static as_status ensure_device(DeviceState** out) {
         return cuda_fail(e, "kernel attribute");
     }
     // where dynamic shared memory starts (the tables are its first bytes)
-    if ((e = cudaFuncSetAttribute(dyn_smem_base_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemSig)) !=
+    constexpr size_t kSmemKey = lk_smem_bytes<Net16<4>>(kLKShapes[0].warps, kLKShapes[0].depth);
+    if ((e = cudaFuncSetAttribute(dyn_smem_base_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKey)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
-    dyn_smem_base_kernel<<<1, 32, kSmemSig>>>();
+    dyn_smem_base_kernel<<<1, 32, kSmemKey>>>();
     uint32_t base = 0;
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "shared memory probe");
     if ((e = cudaMemcpyFromSymbol(&base, g_dyn_smem_base, sizeof(base))) != cudaSuccess)
@@ -1260,17 +1248,17 @@ static as_status ensure_device(DeviceState** out) {
       return cuda_fail(e, "occupancy query");
     if (d.prefix_blocks_per_sm < 1) d.prefix_blocks_per_sm = 1;
     if ((e = cudaFuncSetAttribute(prefix_thread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemCapSig)) != cudaSuccess)
+                                  (int)kSmemPThread)) != cudaSuccess)
       return cuda_fail(e, "kernel attribute");
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.prefix_thread_blocks_per_sm, prefix_thread_kernel,
-                                                           kCapThreads, kSmemCapSig)) != cudaSuccess)
+                                                           kPThreadThreads, kSmemPThread)) != cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.prefix_thread_blocks_per_sm < 1) d.prefix_thread_blocks_per_sm = 1;
     if ((e = cudaFuncSetAttribute(bl_hash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBHash)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.verify_blocks_per_sm, verify_kernel<false, true>, kVThreads, 0)) !=
-        cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.verify_blocks_per_sm, verify_kernel<false, true>,
+                                                           kVThreads, 0)) != cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.verify_blocks_per_sm < 1) d.verify_blocks_per_sm = 1;
     if (!g_results) {
@@ -1567,10 +1555,10 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
       d_off, n, block_bytes, d_pref_off, d_out);
   if (block_bytes >= 32) {
     // entries at most every other chunk: one thread per key, the suffix snapshots of prefix_thread_kernel
-    const uint64_t want = (n + kCapThreads - 1) / kCapThreads;
+    const uint64_t want = (n + kPThreadThreads - 1) / kPThreadThreads;
     const uint64_t lim = (uint64_t)d->sms * (uint64_t)d->prefix_thread_blocks_per_sm;
     const unsigned blocks = (unsigned)(want < lim ? want : lim);
-    prefix_thread_kernel<<<blocks, kCapThreads, kSmemCapSig, (cudaStream_t)stream>>>(d_arena, d_off, n, block_bytes,
+    prefix_thread_kernel<<<blocks, kPThreadThreads, kSmemPThread, (cudaStream_t)stream>>>(d_arena, d_off, n, block_bytes,
                                                                                        d_pref_off, d_out);
   } else {
     // an entry after every chunk: one warp per key, the scan of D over the lanes

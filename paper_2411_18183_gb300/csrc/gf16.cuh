@@ -71,29 +71,19 @@ __device__ __forceinline__ uint32_t tab_index(uint32_t u, uint32_t base, uint32_
 }
 
 // Per-lane table cursors: the lane's two offsets (4*l and 4*l + 128), and
-// the load of the word at byte offset idx of the tables.  RedCursor takes the
-// tables' shared address at run time; RedCursorAt400 has it as the load's
-// immediate offset (one add less per lookup), valid when the tables start the
-// dynamic shared memory and that begins right after the 1 KB every block
-// reserves (shared address 0x400; the host checks this once per device).
+// the load of the word at byte offset idx of the tables, whose shared address
+// is taken at run time.
 struct RedCursor {
   uint32_t tab;       // shared byte address of the tables
   uint32_t off16;     // 4*lane
   uint32_t off24;     // 4*lane + 128
-  uint32_t k16, nk16, k256;
+  uint32_t k16, nk16;
   __device__ __forceinline__ uint32_t load(uint32_t idx) const { return lds32(tab + idx); }
 };
 __device__ uint32_t g_k16 = 0x10000u;   // 2^16, read at run time so the compiler keeps multiplies by it
-struct RedCursorAt400 {
-  uint32_t off16;
-  uint32_t off24;
-  uint32_t k16, nk16, k256;
-  __device__ __forceinline__ uint32_t load(uint32_t idx) const {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+1024];" : "=r"(v) : "r"(idx));
-    return v;
-  }
-};
+// Where dynamic shared memory begins right after the 1 KB every block reserves
+// (the host checks this once per device), tables at its start are loaded by an
+// immediate offset (sigkey.cuh: one add less per lookup).
 constexpr uint32_t kTablesAt400 = 0x400u;
 
 __device__ __forceinline__ RedCursor red_cursor(const uint32_t* red) {
@@ -101,17 +91,9 @@ __device__ __forceinline__ RedCursor red_cursor(const uint32_t* red) {
   c.tab = (uint32_t)__cvta_generic_to_shared(red);
   c.off16 = 4u * (threadIdx.x & 31u);
   c.off24 = c.off16 + 128u;
-  c.k16 = *(volatile uint32_t*)&g_k16; c.nk16 = 0u - c.k16; c.k256 = c.k16 >> 8;
+  c.k16 = *(volatile uint32_t*)&g_k16; c.nk16 = 0u - c.k16;
   return c;
 }
-__device__ __forceinline__ RedCursorAt400 red_cursor_at400() {
-  RedCursorAt400 c;
-  c.off16 = 4u * (threadIdx.x & 31u);
-  c.off24 = c.off16 + 128u;
-  c.k16 = *(volatile uint32_t*)&g_k16; c.nk16 = 0u - c.k16; c.k256 = c.k16 >> 8;
-  return c;
-}
-
 // PRMT selectors: result byte0 = base byte0 (index 4), byte1 = u byte 2 or 3,
 // bytes 2, 3 = base byte 1 (index 5, zero)
 constexpr uint32_t kSel16 = 0x5524u;
@@ -162,16 +144,6 @@ __device__ __forceinline__ void horner_chunk(uint32_t v0, uint32_t v1, uint32_t 
   a4 = red32(u, rc);
   u = (a4 << 16) ^ l0 ^ (h0 << 4) ^ (l1 << 8) ^ (h1 << 12);
   a4 = red32(u, rc);
-}
-
-// Mask of bytes [b0, b1) of a 16-byte chunk, for its 32-bit word j.
-__device__ __forceinline__ uint32_t byte_range_mask(int b0, int b1, int j) {
-  int lo = b0 - 4 * j, hi = b1 - 4 * j;
-  lo = lo < 0 ? 0 : (lo > 4 ? 4 : lo);
-  hi = hi < 0 ? 0 : (hi > 4 ? 4 : hi);
-  const uint32_t mhi = hi >= 4 ? 0xFFFFFFFFu : ((1u << (8 * hi)) - 1u);
-  const uint32_t mlo = lo >= 4 ? 0xFFFFFFFFu : ((1u << (8 * lo)) - 1u);
-  return mhi & ~mlo;
 }
 
 // Murmur3 64-bit finaliser: bucket hash of (signature, length).

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __rest
   }
 }
 
-constexpr int kCapThreads = 1024;       // threads per block of prefix_thread_kernel
+constexpr int kPThreadThreads = 1024;       // threads per block of prefix_thread_kernel
 
 // Cumulative signatures, one thread per key.  The thread runs the backward
 // Horner rule over the key's realigned chunks; since B is a
@@ -331,7 +331,7 @@ constexpr int kCapThreads = 1024;       // threads per block of prefix_thread_ke
 //     C_j = S + x^(8 k c_j - k lo/2) acc'_j
 // (prefix = whole key minus suffix, the suffix moved to its place), formed
 // through the log / antilog tables, once per stored entry.
-__global__ void __launch_bounds__(kCapThreads) prefix_thread_kernel(const uint8_t* __restrict__ arena,
+__global__ void __launch_bounds__(kPThreadThreads) prefix_thread_kernel(const uint8_t* __restrict__ arena,
                                                                     const uint64_t* __restrict__ off, uint64_t n,
                                                                     uint32_t block_bytes,
                                                                     const uint64_t* __restrict__ pref_off,
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kPThreads) prefix_scan_kernel(const uint64_t* 
   }
 }
 
-constexpr size_t kSmemCapSig = (size_t)kRedBytes + 512 * 4 + 512 * 2;
+constexpr size_t kSmemPThread = (size_t)kRedBytes + 512 * 4 + 512 * 2;
 
 constexpr size_t kSmemPrefix = (size_t)kRedBytes + 512 * 4 + (size_t)kPConst * 512 * 2;
 

@@ -1,10 +1,8 @@
-// rounds.cuh -- warp-level helpers shared by the kernels: async copies,
-// the split of a relation's keys over warps in equal shares of key bytes
-// (+ an optional cost per key; a 32-ary search in the offsets by one warp), the offsets a warp loads for a round of 32 keys,
-// the constant-multiply tables, and the geometry of the 16-byte chunk grid
-// that the comparison join's string hash (baseline.cuh) walks in tiles of
-// kTile bytes (a key starting at an odd byte is read funnel-shifted by one
-// byte, so that its symbols sit on 16-bit boundaries).
+// rounds.cuh -- warp-level helpers shared by the kernels: async copies, the
+// split of a relation's keys over warps in equal shares of key bytes (+ an
+// optional cost per key; a 32-ary search in the offsets by one warp), the
+// offsets a warp loads for a round of 32 keys, and the constant-multiply tables
+// of the cumulative signatures' tiles of kTile bytes.
 #pragma once
 #include <cstdint>
 
@@ -17,9 +15,6 @@ namespace algsig {
 #endif
 constexpr int kTileChunks = ALGSIG_TILE_CHUNKS;       // 16-byte chunks per tile
 constexpr int kTile = 16 * kTileChunks;               // bytes of realigned key per tile
-constexpr int kSpanChunks = 32 * kTileChunks + 2;     // chunks of a round's span, worst case
-// one 16-byte pad per tile-length of span, so that tiles kTile bytes apart hit different banks
-constexpr int kBufBytes = 16 * (kSpanChunks + (kSpanChunks + kTileChunks - 1) / kTileChunks) + 16;
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 
 // g_log / g_alog: GF(2^16) logarithm / antilogarithm of x, defined (and set
@@ -42,9 +37,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// shared-memory byte offset of span offset `rel` (16-byte pad after every kTile bytes)
-__device__ __forceinline__ uint32_t padded(uint32_t rel) { return rel + (rel / (uint32_t)kTile) * 16u; }
 
 // ---------------------------------------------------------------------------
 // warp range: keys [k_lo, k_hi) whose starts fall in this warp's share of the

@@ -1247,6 +1247,9 @@ static as_status ensure_device(DeviceState** out) {
                                                            kSmemPrefix)) != cudaSuccess)
       return cuda_fail(e, "occupancy query");
     if (d.prefix_blocks_per_sm < 1) d.prefix_blocks_per_sm = 1;
+    if ((e = cudaFuncSetAttribute(prefix_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPScan)) !=
+        cudaSuccess)
+      return cuda_fail(e, "kernel attribute");
     if ((e = cudaFuncSetAttribute(prefix_thread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kSmemPThread)) != cudaSuccess)
       return cuda_fail(e, "kernel attribute");
@@ -1550,9 +1553,9 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
     sig_key_kernel<false, Net16<4>, k.warps, k.depth, false, true>
         <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
             d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
-  const uint64_t scan_want = (n + kPThreads - 1) / kPThreads, scan_lim = (uint64_t)d->sms * 8;
-  prefix_scan_kernel<<<(unsigned)(scan_want < scan_lim ? scan_want : scan_lim), kPThreads, 0, (cudaStream_t)stream>>>(
-      d_off, n, block_bytes, d_pref_off, d_out);
+  const uint64_t scan_want = (n + kPScanThreads - 1) / kPScanThreads;
+  prefix_scan_kernel<<<(unsigned)(scan_want < (uint64_t)d->sms ? scan_want : (uint64_t)d->sms), kPScanThreads, kSmemPScan,
+                       (cudaStream_t)stream>>>(d_off, n, block_bytes, d_pref_off, d_out);
   if (block_bytes >= 32) {
     // entries at most every other chunk: one thread per key, the suffix snapshots of prefix_thread_kernel
     const uint64_t want = (n + kPThreadThreads - 1) / kPThreadThreads;

@@ -395,18 +395,63 @@ __global__ void __launch_bounds__(kPThreadThreads) prefix_thread_kernel(const ui
 
 // The cumulative signatures from those of the keys' blocks (the signature
 // kernel over items): C_j = sum_{i <= j} x^(k i B / 2) sig(block i), in place,
-// one thread per key; a key of more than 32 blocks is scanned by the warp.  The
-// factors go through the log / antilog tables.
-__global__ void __launch_bounds__(kPThreads) prefix_scan_kernel(const uint64_t* __restrict__ off, uint64_t n,
-                                                                uint32_t block_bytes,
-                                                                const uint64_t* __restrict__ pref_off,
-                                                                uint64_t* __restrict__ out) {
-  if (!by_items(off, n, block_bytes)) return;
+// one thread per key; a key of more than 32 blocks is scanned by the warp.
+// The factor of block i = 16 q + l is applied as x^(k l B / 2) and x^(16 k q B / 2),
+// each by two tables of 256 entries (low and high byte) in shared memory that
+// every block makes for itself, for l < 16 and q < 32; the keys of more than 512
+// blocks go through the log / antilog tables.  What bounds it is the gathers:
+// through the log / antilog tables, eight per entry from 128 KB tables in L1, each
+// up to 32 lines, 500k keys of 200-2000 bytes at B = 256 took 50 us, 23 now
+// (whole call 290 -> 265 us; at B = 64 720 -> 565; three keys of 1.4 MB on average
+// at B = 256 780 -> 605).
+constexpr int kPScanThreads = 1024;
+constexpr uint32_t kPScanLow = 16, kPScanHigh = 32;   // factors l and q: 0..15 and 0..31
+constexpr uint32_t kPScanTables = (kPScanLow - 1 + kPScanHigh - 1) * 8;
+constexpr size_t kSmemPScan = (size_t)kPScanTables * 512;
+__global__ void __launch_bounds__(kPScanThreads, 1) prefix_scan_kernel(const uint64_t* __restrict__ off, uint64_t n,
+                                                                    uint32_t block_bytes,
+                                                                    const uint64_t* __restrict__ pref_off,
+                                                                    uint64_t* __restrict__ out) {
+  if (!by_items(off, n, block_bytes) || pref_off[n] == n) return;   // no key of two blocks: nothing to add
+  extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t eb = (block_bytes / 2u) % kOrder;     // exponent from one block to the next
-  auto moved = [](uint64_t v, uint32_t e) {
+  // table t = 8 f + 2 (k - 1) + h, f a factor (l - 1, then 15 + q - 1): its products with a byte at bits
+  // 8 h..8 h + 7; a lane makes the entries 8 lane..8 lane + 7 from the products with single bits
+  for (uint32_t t = threadIdx.x >> 5; t < kPScanTables; t += kPScanThreads / 32) {
+    const uint32_t f = t >> 3, i = f < kPScanLow - 1 ? f + 1 : kPScanLow * (f - (kPScanLow - 2));
+    const uint32_t e0 = (uint32_t)((uint64_t)i * (((t >> 1) & 3u) + 1) * eb % kOrder) + 8u * (t & 1u);
+    uint32_t bit = 0;                                  // lanes 0..7: x^(k i eb) x^(8 h + lane)
+    if (lane < 8u) bit = __ldg(&g_alog[(e0 + lane) % kOrder]);
+    uint32_t v = 0;
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+      const uint32_t x = __shfl_sync(0xFFFFFFFFu, bit, 3 + s);
+      if (lane >> s & 1u) v ^= x;
+    }
+    const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, bit, 0), b1 = __shfl_sync(0xFFFFFFFFu, bit, 1);
+    const uint32_t b2 = __shfl_sync(0xFFFFFFFFu, bit, 2);
+    const uint32_t w0 = v * 0x10001u ^ b0 << 16, p1 = b1 * 0x10001u, p2 = b2 * 0x10001u;
+    reinterpret_cast<uint4*>(smem)[t * 32u + lane] = make_uint4(w0, w0 ^ p1, w0 ^ p2, w0 ^ p1 ^ p2);
+  }
+  __syncthreads();
+  auto times = [&](uint64_t v, uint32_t f) -> uint64_t {
+    const uint16_t* tab = reinterpret_cast<const uint16_t*>(smem) + f * 2048u;
+    const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
+    const uint32_t s1 = tab[lo & 0xFFu] ^ tab[256u + (lo >> 8 & 0xFFu)];
+    const uint32_t s2 = tab[512u + (lo >> 16 & 0xFFu)] ^ tab[768u + (lo >> 24)];
+    const uint32_t s3 = tab[1024u + (hi & 0xFFu)] ^ tab[1280u + (hi >> 8 & 0xFFu)];
+    const uint32_t s4 = tab[1536u + (hi >> 16 & 0xFFu)] ^ tab[1792u + (hi >> 24)];
+    return (uint64_t)(s1 | s2 << 16) | (uint64_t)(s3 | s4 << 16) << 32;
+  };
+  auto moved = [&](uint64_t v, uint32_t i) -> uint64_t {     // block i's value in its place, i < 512
+    if (i & (kPScanLow - 1)) v = times(v, (i & (kPScanLow - 1)) - 1);
+    if (i / kPScanLow) v = times(v, kPScanLow - 2 + i / kPScanLow);
+    return v;
+  };
+  auto moved_far = [&](uint64_t v, uint64_t i) {
     return shift_chunk_value((uint32_t)v & 0xFFFFu, (uint32_t)(v >> 16) & 0xFFFFu, (uint32_t)(v >> 32) & 0xFFFFu,
-                             (uint32_t)(v >> 48), e);
+                             (uint32_t)(v >> 48), (uint32_t)(i % kOrder * eb % kOrder));
   };
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {   // warp-uniform
@@ -418,30 +463,27 @@ __global__ void __launch_bounds__(kPThreads) prefix_scan_kernel(const uint64_t* 
     }
     if (c > 1 && c <= 32) {
       uint64_t acc = out[p0];
-      uint32_t e = 0;
       for (uint32_t j = 1; j < (uint32_t)c; j += 4) {      // four blocks' lookups at a time
         uint64_t v[4];
 #pragma unroll
-        for (uint32_t t = 0; t < 4; ++t) {
-          v[t] = j + t < (uint32_t)c ? out[p0 + j + t] : 0ull;
-          e += eb;
-          if (e >= kOrder) e -= kOrder;
-          v[t] = moved(v[t], e);
-        }
+        for (uint32_t t = 0; t < 4; ++t) v[t] = j + t < (uint32_t)c ? out[p0 + j + t] : 0ull;
 #pragma unroll
-        for (uint32_t t = 0; t < 4; ++t) {
-          acc ^= v[t];
-          if (j + t < (uint32_t)c) out[p0 + j + t] = acc;
-        }
+        for (uint32_t t = 0; t < 4; ++t)
+          if (j + t < (uint32_t)c) {
+            acc ^= moved(v[t], j + t);
+            out[p0 + j + t] = acc;
+          }
       }
     }
     for (uint32_t m = __ballot_sync(0xFFFFFFFFu, c > 32); m; m &= m - 1u) {
       const int l = __ffs((int)m) - 1;
       const uint64_t pl = __shfl_sync(0xFFFFFFFFu, p0, l), cl = __shfl_sync(0xFFFFFFFFu, c, l);
-      uint64_t carry = 0;
+      uint64_t carry = 0, next = out[pl + lane];           // (cl > 32)
       for (uint64_t b = 0; b < cl; b += 32) {
         const uint64_t j = b + lane;
-        uint64_t v = j < cl ? moved(out[pl + j], (uint32_t)(j % kOrder * eb % kOrder)) : 0ull;
+        uint64_t v = next;
+        next = j + 32 < cl ? out[pl + j + 32] : 0ull;
+        v = cl <= kPScanLow * kPScanHigh ? moved(v, (uint32_t)j) : moved_far(v, j);
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
           const uint64_t t = __shfl_up_sync(0xFFFFFFFFu, v, d);

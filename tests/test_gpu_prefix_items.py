@@ -58,3 +58,34 @@ def test_many_windows_per_warp(cuda, block):
     for i in some:
         key = arena[int(off[i]):int(off[i + 1])].cpu().numpy().tobytes()
         assert host[pref[i]:pref[i + 1]].tolist() == oracle.sig_prefixes(key, block), i
+
+
+@pytest.mark.parametrize("block", [32, 80, 256])
+def test_blocks_around_the_scan_factors(cuda, block):
+    """Block counts around the factors that the scan splits a block's place into (16), the keys that
+    one thread sums (32) and the tables' end (512)."""
+    ag = cuda
+    rng = np.random.default_rng(block)
+    counts = [2, 3, 4, 5, 6, 15, 16, 17, 18, 31, 32, 33, 34, 47, 48, 49, 63, 64, 65, 511, 512, 513, 545]
+    keys = [rng.integers(0, 256, c * block - int(rng.integers(0, block)), dtype=np.uint8).tobytes() for c in counts]
+    rel = relation_from_keys(keys)
+    D = ag.DeviceRelation.from_host(rel.arena, rel.off)
+    pref, out = ag.sig_prefixes(D, block)
+    pref, out = pref.cpu().numpy(), out.cpu().numpy().view(np.uint64)
+    assert np.array_equal(np.diff(pref), counts)
+    for i, k in enumerate(keys):
+        assert out[pref[i]:pref[i + 1]].tolist() == oracle.sig_prefixes(k, block), counts[i]
+
+
+@pytest.mark.parametrize("block", [131056, 131072, 262128])
+def test_blocks_whose_factors_wrap(cuda, block):
+    """Blocks of nearly, exactly one more than and nearly twice the order of x in symbols."""
+    ag = cuda
+    rng = np.random.default_rng(block)
+    keys = [rng.integers(0, 256, n, dtype=np.uint8).tobytes() for n in (block + 1, 2 * block + 77, 4 * block, 9)]
+    rel = relation_from_keys(keys)
+    pref, out = ag.sig_prefixes(ag.DeviceRelation.from_host(rel.arena, rel.off), block)
+    pref, out = pref.cpu().numpy(), out.cpu().numpy().view(np.uint64)
+    want = [k[:(j + 1) * block] for k in keys for j in range(max(1, -(-len(k) // block)))]
+    ref = relation_from_keys(want)
+    assert np.array_equal(out, oracle.sig_batch(ref.arena, ref.off, nthreads=4))

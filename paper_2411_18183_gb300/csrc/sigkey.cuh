@@ -55,7 +55,7 @@
 // Measured (signatures of 2M keys of 256-1024 bytes, 1.28 GB: 346 us with the
 // register loads and the remainder form, 265 us now, 4.8 TB/s; 300k keys of
 // 2048-8192 bytes, two components: 375 and 277 us; 4M keys of 32-128 bytes: 204
-// and 193 us, bound by the arithmetic per key).
+// and 181 us, bound by the arithmetic and the shared-memory wavefronts per key).
 // In a batch the keys are the joins' row ranges back to back ("virtual
 // rows"): the warps split them by work across the joins, and a window
 // ends with its join's rows so that its keys are consecutive in the relation.
@@ -255,7 +255,9 @@ __device__ __forceinline__ uint32_t lk_blocks(uintptr_t abs, uint64_t len) {
 // counts (255 and more share the last bin; the order within a bin is
 // arbitrary), so that each group of 32 consecutive entries has keys of
 // nearly equal length.  rows: an empty stage, the first 8 rows of which hold
-// the bins' counts.
+// the bins' counts.  (Short keys are bound by shared-memory wavefronts, 76 % of
+// the peak for 4M keys of 32-128 bytes: with the bins moved eight words at a time
+// and lk_copy_setup's rows in different banks that call takes 181 us, 197 before.)
 __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_t wn, uintptr_t arena,
                                                uint64_t cap_len) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -267,9 +269,8 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
   auto count = [&](uint32_t b) -> uint32_t& {
     return reinterpret_cast<uint32_t*>(rows + (b >> 5) * kLKPitch)[b & 31u];
   };
-  uint32_t* mine = &count(8 * lane);                  // the lane's 8 consecutive bins
-#pragma unroll
-  for (int t = 0; t < 8; ++t) mine[t] = 0u;
+  uint4* mine = reinterpret_cast<uint4*>(&count(8 * lane));   // the lane's 8 consecutive bins
+  mine[0] = mine[1] = make_uint4(0, 0, 0, 0);
   __syncwarp();
   constexpr int kPer = kLKWin / 32;                   // entries per lane
   uint32_t bin[kPer], rank[kPer];
@@ -287,25 +288,18 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
   }
   __syncwarp();
   // exclusive prefix sum over the bins, 8 consecutive bins per lane
-  uint32_t h[8], sum = 0;
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    h[t] = mine[t];
-    sum += h[t];
-  }
+  const uint4 h0 = mine[0], h1 = mine[1];
+  const uint32_t sum = h0.x + h0.y + h0.z + h0.w + h1.x + h1.y + h1.z + h1.w;
   uint32_t incl = sum;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const uint32_t o = __shfl_up_sync(kFull, incl, d);
     if (lane >= (uint32_t)d) incl += o;
   }
-  uint32_t base = incl - sum;
+  const uint32_t b0 = incl - sum, b1 = b0 + h0.x + h0.y + h0.z + h0.w;
   __syncwarp();
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    mine[t] = base;
-    base += h[t];
-  }
+  mine[0] = make_uint4(b0, b0 + h0.x, b0 + h0.x + h0.y, b0 + h0.x + h0.y + h0.z);
+  mine[1] = make_uint4(b1, b1 + h1.x, b1 + h1.x + h1.y, b1 + h1.x + h1.y + h1.z);
   __syncwarp();
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
@@ -370,11 +364,13 @@ __device__ __forceinline__ void lk_copy_setup(LKCopy& y, const LKKey& k, uint32_
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t b = reinterpret_cast<uint64_t>(k.base);
   __syncwarp();
-  sts128(st + kLKPitch * lane, make_uint4((uint32_t)b, (uint32_t)(b >> 32), k.c1, 0u));
+  // (a row's place for it is the chunk of the row's number mod 8, so that neighbouring rows' are in different banks)
+  sts128(st + kLKPitch * lane + ((lane & 7u) << 4), make_uint4((uint32_t)b, (uint32_t)(b >> 32), k.c1, 0u));
   __syncwarp();
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const uint4 v = lds128(st + kLKPitch * (4 * i + (lane >> 3)));
+    const uint32_t r = 4 * i + (lane >> 3);
+    const uint4 v = lds128(st + kLKPitch * r + ((r & 7u) << 4));
     y.src[i] = reinterpret_cast<const uint8_t*>((uint64_t)v.x | ((uint64_t)v.y << 32)) + 16 * (lane & 7u);
     y.c1[i] = v.z;
   }

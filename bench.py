@@ -266,7 +266,7 @@ def batch_leg(ag, steps: int):
             "tuples_per_s": total_s / (total_ms * 1e-3), "key_GBps": total_bytes / (total_ms * 1e-3) / 1e9,
             "joins_per_s": spec.n_joins / (total_ms * 1e-3), "oracle_checked_joins": sampled,
             "pair_counts": "every join equals the generator's count", "wall_s": round(time.time() - t0, 1),
-            "l2": "inputs of each wave far larger than L2", "gpu_launches_per_batch": 5, "cuda_graph": True}
+            "l2": "inputs of each wave far larger than L2", "gpu_launches_per_batch": 6, "cuda_graph": True}
 
 
 def plan_rows(specs, field):

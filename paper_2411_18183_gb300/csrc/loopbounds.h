@@ -1,6 +1,7 @@
 // loopbounds.h -- loop bounds of the warp-wide byte comparison (the exact
-// verification of every candidate pair that makes the join exact), shared by
-// the device code and a host-compiled check of the bounds.
+// verification of every candidate pair that makes the join exact) and of the
+// signature kernel's copies, shared by the device code and a host-compiled
+// check of the bounds.
 //
 // The comparison of two len-byte keys runs in 32-bit offsets from the aligned
 // 16-byte chunk that holds the S key's first byte (that byte at offset
@@ -32,6 +33,26 @@ ALGSIG_HD uint32_t narrow_steps(uint32_t sa, uint32_t len) { return (uint32_t)((
 // key's misalignment
 ALGSIG_HD uint64_t narrow_offset_end(uint32_t sa, uint32_t len, uint32_t d) {
   return (uint64_t)narrow_steps(sa, len) * 1024u + d + 16u;
+}
+
+// Where a key of len > 0 bytes ends in the signature kernel's blocks of 32
+// bytes (four to a step, two 16-byte chunks each), its first byte being byte
+// a < 32 of block 0: it has `blocks` blocks, `full` of them with both chunks,
+// and `rest` bytes of its last chunk (0: all 16).  Counted in blocks, so that
+// every key below 2^32 blocks fits 32 bits (a key of 64 GiB has 2^32 chunks).
+struct KeyEnd {
+  uint32_t blocks, full, rest;
+};
+ALGSIG_HD KeyEnd key_end(uint32_t a, uint64_t len) {
+  const uint64_t e = a + len, b = (e + 31) >> 5, f = (e + 15) >> 5;
+  return {b < 0xFFFFFFFFull ? (uint32_t)b : 0xFFFFFFFFu, (uint32_t)f, (uint32_t)e & 15u};
+}
+// whether chunk q of eight of step s is the key's; have: `blocks` for the even chunks, `full` for the odd ones
+ALGSIG_HD bool has_chunk(uint32_t s, uint32_t q, uint32_t have) { return 4u * s + (q >> 1) < have; }
+// step of the key's last chunk, and its place of eight in it
+ALGSIG_HD uint32_t last_step(uint32_t blocks) { return (blocks - 1u) >> 2; }
+ALGSIG_HD uint32_t last_place(uint32_t blocks, uint32_t full) {
+  return 2u * ((blocks - 1u) & 3u) + (full == blocks ? 1u : 0u);
 }
 
 }  // namespace algsig

@@ -143,7 +143,7 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem_src) : "memory");
 }
-// chunk c of a key of n chunks, at src + s * kStep, to shared memory; zeros (nothing read) past the key
+// the 16 bytes at src + s * step to shared memory; zeros (nothing read) where c >= n
 __device__ __forceinline__ void cp_async16_below(uint32_t smem_dst, const uint8_t* src, uint32_t s, uint32_t step,
                                                  uint32_t c, uint32_t n) {
   asm volatile(
@@ -227,8 +227,8 @@ struct LKKey {
   const uint8_t* base;  // 32-byte aligned address of the key's first block
   uint32_t nb;          // 32-byte blocks (0: empty key)
   uint32_t a;           // offset of the key's first byte in its first block (0..31)
-  uint32_t c1;          // 16-byte chunks from base up to the key's last byte
-  uint32_t te;          // key bytes of the last of them (0: all 16)
+  uint32_t full;        // of its blocks, those with both 16-byte chunks (loopbounds.h's key_end)
+  uint32_t te;          // key bytes of its last chunk (0: all 16)
   bool valid;
 };
 
@@ -315,7 +315,7 @@ __device__ __forceinline__ uint32_t lk_load_group(LKKey& k, const LKWarp& W, uin
                                                   const uint8_t* arena, uint64_t cap_len) {
   const uint32_t r = 32u * g + (threadIdx.x & 31u);
   k.valid = r < wn;
-  k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.c1 = 0; k.te = 0;
+  k.kq = 0; k.base = arena; k.nb = 0; k.a = 0; k.full = 0; k.te = 0;
   if (k.valid) {
     const uint32_t i = W.order[r];
     const uint64_t ks = W.woff[i], len = min(W.woff[i + 1] - ks, cap_len);
@@ -326,10 +326,11 @@ __device__ __forceinline__ uint32_t lk_load_group(LKKey& k, const LKWarp& W, uin
     k.base = reinterpret_cast<const uint8_t*>(abs & ~(uintptr_t)31);
     if (k.base < arena) k.base += 16;
     k.a = (uint32_t)(abs - reinterpret_cast<uintptr_t>(k.base));
-    k.nb = len ? (uint32_t)min((uint64_t)0xFFFFFFFFu, (k.a + len + 31) >> 5) : 0u;
-    if (k.nb) {
-      k.c1 = (uint32_t)((k.a + len + 15) >> 4);
-      k.te = (uint32_t)(k.a + len) & 15u;
+    if (len) {
+      const KeyEnd e = key_end(k.a, len);
+      k.nb = e.blocks;
+      k.full = e.full;
+      k.te = e.rest;
     }
   }
   const uint32_t G = __reduce_max_sync(kFull, k.nb);
@@ -350,10 +351,10 @@ __device__ __forceinline__ void lk_fill_masks(uint4* mt) {
 }
 
 // The copies of a group's steps: lane l copies chunk l % 8 of the rows of keys
-// l / 8, l / 8 + 4, ..., whose addresses and chunk counts it holds here.
+// l / 8, l / 8 + 4, ..., whose addresses and ends it holds here.
 struct LKCopy {
   const uint8_t* src[8];   // base + 16 (l % 8) of the key
-  uint32_t c1[8];          // the key's chunk count from base
+  uint32_t have[8];        // the key's blocks that have such a chunk (has_chunk)
 };
 
 // chunk c of the lane's row at shared address row (the lane's swizzle folded in)
@@ -365,14 +366,14 @@ __device__ __forceinline__ void lk_copy_setup(LKCopy& y, const LKKey& k, uint32_
   const uint64_t b = reinterpret_cast<uint64_t>(k.base);
   __syncwarp();
   // (a row's place for it is the chunk of the row's number mod 8, so that neighbouring rows' are in different banks)
-  sts128(st + kLKPitch * lane + ((lane & 7u) << 4), make_uint4((uint32_t)b, (uint32_t)(b >> 32), k.c1, 0u));
+  sts128(st + kLKPitch * lane + ((lane & 7u) << 4), make_uint4((uint32_t)b, (uint32_t)(b >> 32), k.nb, k.full));
   __syncwarp();
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const uint32_t r = 4 * i + (lane >> 3);
     const uint4 v = lds128(st + kLKPitch * r + ((r & 7u) << 4));
     y.src[i] = reinterpret_cast<const uint8_t*>((uint64_t)v.x | ((uint64_t)v.y << 32)) + 16 * (lane & 7u);
-    y.c1[i] = v.z;
+    y.have[i] = lane & 1u ? v.w : v.z;
   }
   __syncwarp();
 }
@@ -380,19 +381,19 @@ __device__ __forceinline__ void lk_copy_setup(LKCopy& y, const LKKey& k, uint32_
 // request step s of the group's keys into the stage at shared address st
 __device__ __forceinline__ void lk_copy_step(const LKCopy& y, uint32_t st, uint32_t s) {
   const uint32_t lane = threadIdx.x & 31u, q = lane & 7u, r = lane >> 3;
-  const uint32_t c = 8u * s + q;
+  const uint32_t c = 4u * s + (q >> 1);              // has_chunk
   // row 4 i + r, chunk q: its place is q ^ (row % 8), and row % 8 = 4 (i % 2) + r
   const uint32_t d0 = st + r * kLKPitch + ((q ^ r) << 4), d1 = st + r * kLKPitch + ((q ^ (r + 4u)) << 4);
 #pragma unroll
   for (int i = 0; i < 8; ++i)
-    cp_async16_below((i & 1 ? d1 : d0) + 4 * i * kLKPitch, y.src[i], s, kLKRow, c, y.c1[i]);
+    cp_async16_below((i & 1 ? d1 : d0) + 4 * i * kLKPitch, y.src[i], s, kLKRow, c, y.have[i]);
 }
 
 // zero what is not the key's in the rows that hold its ends: the bytes after
 // its last (in the step that holds it) and before its first (in step 0)
 __device__ __forceinline__ void lk_trim(const LKKey& k, uint32_t row, uint32_t s, const uint4* mt) {
-  if (k.te && (k.c1 - 1) >> 3 == s) {
-    const uint32_t p = lk_chunk(row, (k.c1 - 1) & 7u);
+  if (k.te && last_step(k.nb) == s) {
+    const uint32_t p = lk_chunk(row, last_place(k.nb, k.full));
     uint4 v = lds128(p);
     const uint4 m = mt[k.te];
     v.x &= m.x; v.y &= m.y; v.z &= m.z; v.w &= m.w;

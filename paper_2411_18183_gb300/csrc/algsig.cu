@@ -466,10 +466,11 @@ struct CandQueue {
 // chunks: 4 x 2 2.83 ms, 3 x 4 2.85, 3 x 3 2.96, 4 x 3 3.02, 4 x 1 3.11)
 constexpr int kVAhead = 2;
 // Longest key compared by eight lanes: the whole warp's 512 bytes in a row take fewer requests (400k
-// candidates of 2-8 KB: 821 us with eight lanes, 750 us with the warp, when the line was drawn; 679 us now),
-// eight lanes fewer instructions and waits per candidate (5M of 256-1024 bytes: 1.3 against 1.7 ms, both in the
-// queue's order)
-constexpr uint32_t kVFourMax = 2048;
+// candidates of 2-8 KB: 821 us with eight lanes, 750 us with the warp, when first compared) and are left where the
+// keys differ, eight lanes take fewer instructions and waits per candidate (5M of 256-1024 bytes: 1.3 against 1.7 ms,
+// both in the queue's order).  500k equal ones of 1000-2048 bytes: 297, 281 and 285 us with 1024, 1536 and 2048;
+// 100k of 2 KB that differ at once: 75 and 105 us with 1536 and 2048.
+constexpr uint32_t kVFourMax = 1536;
 
 // the candidates of a probe step (lanes with `cand`) to the end of the queue
 __device__ __forceinline__ void queue_push(Cand* q, uint32_t& cnt, bool cand, uint64_t start, uint64_t srow,
@@ -511,7 +512,14 @@ __device__ __forceinline__ uint4 chunk_diff(const uint4& sv, const uint4& ra, co
 // of a candidate's lanes takes the 16-byte S chunks i, i + 2^lg, ... and the two
 // aligned R chunks under each, kVAhead at a time; the last chunk, where it is
 // partial, is compared apart.  Only aligned chunks that hold a key byte are read.
-template <uint32_t lg>
+// A candidate of the whole warp's is left at its first 1 KB if that differs
+// (signatures collide where a caller gives its own, or two components), then every
+// 4 KB (PIECES, up to 10 KB not again) or every 1 KB; those of eight lanes, 1.5 KB
+// at most, are read to their ends.  (20k candidates of 32 KB that differ in their first
+// KB: 707 us read to the end, 60 now; 100k of 2 KB 105 and 75.  Equal keys of 2-8 KB
+// take 784 us read to the end, 781 with PIECES and 795 left every 1 KB; in the
+// kernel of the output modes PIECES spills, 310 against 290 us for 1-2 KB.)
+template <uint32_t lg, bool PIECES>
 __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint32_t todo,
                                                  const uint4* __restrict__ emask) {
   const uint32_t lane = threadIdx.x & 31u, li = lane & ((1u << lg) - 1u), c = r + (lane >> lg);
@@ -531,7 +539,8 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
     if (16u < rem + d) tb = ld16(pR + off + 16);
   }
   const uint32_t nmax = __reduce_max_sync(kFull, nfull);
-  for (uint32_t c0 = 0; c0 < nmax; c0 += (uint32_t)kVAhead << lg) {   // warp-uniform
+  // one trip: the chunks from c0 on that the lanes have in flight
+  auto trip = [&](uint32_t c0) {
     uint4 sv[kVAhead], ra[kVAhead], rb[kVAhead];
 #pragma unroll
     for (int u = 0; u < kVAhead; ++u) {
@@ -553,6 +562,32 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
         x.x &= ~m.x; x.y &= ~m.y; x.z &= ~m.z; x.w &= ~m.w;
       }
       diff |= (x.x | x.y) | (x.z | x.w);
+    }
+  };
+  constexpr uint32_t kTrip = (uint32_t)kVAhead << lg;  // (all bounds below are warp-uniform)
+  auto trips = [&](uint32_t c0, uint32_t end) {
+    for (; c0 < end; c0 += kTrip) trip(c0);
+  };
+  if constexpr (lg < 5u) {
+    trips(0u, nmax);
+  } else if constexpr (!PIECES) {
+    for (uint32_t c0 = 0; c0 < nmax; c0 += kTrip) {
+      trip(c0);
+      if (__any_sync(kFull, diff != 0u)) break;
+    }
+  } else {
+    trips(0u, min(kTrip, nmax));
+    if (nmax > kTrip && !__any_sync(kFull, diff != 0u)) {
+      if (nmax <= 640u) {
+        trips(kTrip, nmax);
+      } else {
+        uint32_t c0 = kTrip;
+#pragma unroll 1
+        do {
+          trips(c0, min(c0 + 256u, nmax));
+          c0 += 256u;
+        } while (c0 < nmax && !__any_sync(kFull, diff != 0u));
+      }
     }
   }
   if (__any_sync(kFull, tail)) {
@@ -646,8 +681,8 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
     __syncwarp();
   }
   uint32_t r = 0;
-  for (; r < few; r += 4u) bad |= compare_some<3>(q, r, todo, emask);
-  for (; r < nc; ++r) bad |= compare_some<5>(q, r, todo, emask);
+  for (; r < few; r += 4u) bad |= compare_some<3, false>(q, r, todo, emask);
+  for (; r < nc; ++r) bad |= compare_some<5, BATCH || INNER>(q, r, todo, emask);
   const bool eq = lane < nc && !((bad >> lane) & 1u);
   const uint32_t row = q[lane].b.z, tag = q[lane].b.w;   // (defined where eq)
   if (!BATCH && !INNER && eq && mode >= AS_JOIN_OUTER_R) atomicOr(P.matched + (row >> 5), 1u << (row & 31u));

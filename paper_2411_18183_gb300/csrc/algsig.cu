@@ -1062,20 +1062,21 @@ static as_status cuda_fail(cudaError_t e, const char* where) {
 }
 
 // The instantiations of the signature kernel: table addressing (AT400),
-// net, shape (warps per block, blocks in flight per key) and whether it runs
-// over the virtual rows of a batch (four components over GF(2^16) only).
+// net, shape (warps per block, blocks in flight per key) and whose signatures
+// (the rows of a batch, first bytes and items: four components over GF(2^16)
+// only, the latter two in shape 0).
 static_assert(kLKShapeCount == 3, "one case per shape below");
-template <bool AT400, class Net, int SHAPE, bool BATCH>
+template <bool AT400, class Net, int SHAPE, LKOf OF>
 static cudaError_t key_kernel_attr() {
   constexpr LKShape k = kLKShapes[SHAPE];
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>),
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(sig_key_kernel<AT400, Net, k.warps, k.depth, OF>),
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk_smem_bytes<Net>(k.warps, k.depth));
 }
-template <bool AT400, class Net, bool BATCH>
+template <bool AT400, class Net, LKOf OF>
 static cudaError_t key_kernel_attrs() {
-  cudaError_t e = key_kernel_attr<AT400, Net, 0, BATCH>();
-  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 1, BATCH>();
-  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 2, BATCH>();
+  cudaError_t e = key_kernel_attr<AT400, Net, 0, OF>();
+  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 1, OF>();
+  if (e == cudaSuccess) e = key_kernel_attr<AT400, Net, 2, OF>();
   return e;
 }
 // a group of 32 keys per block, until every one of max_blocks has one
@@ -1083,7 +1084,7 @@ static unsigned sig_blocks(uint64_t n, int max_blocks) {
   const uint64_t want = (n + 31) / 32;
   return (unsigned)(want < (uint64_t)max_blocks ? (want < 1 ? 1 : want) : (uint64_t)max_blocks);
 }
-template <bool AT400, class Net, int SHAPE, bool BATCH>
+template <bool AT400, class Net, int SHAPE, LKOf OF>
 static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out,
                               const BatchJoin* J, int nj, int s_side, uint64_t cap_len, cudaStream_t s,
                               LKSecond second = LKSecond(), int second_blocks = 0) {
@@ -1093,18 +1094,17 @@ static void key_kernel_launch(int max_blocks, const uint8_t* arena, const uint64
     second.from = blocks;
     blocks += sig_blocks(second.n, second_blocks);
   }
-  sig_key_kernel<AT400, Net, k.warps, k.depth, BATCH>
+  sig_key_kernel<AT400, Net, k.warps, k.depth, OF>
       <<<blocks, 32 * k.warps, lk_smem_bytes<Net>(k.warps, k.depth), s>>>(arena, off, n, out, J, nj, s_side, cap_len,
                                                                            LKItems(), second);
 }
-template <bool AT400, class Net, bool BATCH>
+template <bool AT400, class Net, LKOf OF>
 static void key_kernel_launch_shape(int shape, int sms, const uint8_t* arena, const uint64_t* off, uint64_t n,
-                                    uint64_t* out, const BatchJoin* J, int nj, int s_side, uint64_t cap_len,
-                                    cudaStream_t s) {
+                                    uint64_t* out, const BatchJoin* J, int nj, int s_side, cudaStream_t s) {
   switch (shape) {
-    case 1: key_kernel_launch<AT400, Net, 1, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
-    case 2: key_kernel_launch<AT400, Net, 2, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
-    default: key_kernel_launch<AT400, Net, 0, BATCH>(sms, arena, off, n, out, J, nj, s_side, cap_len, s); break;
+    case 1: key_kernel_launch<AT400, Net, 1, OF>(sms, arena, off, n, out, J, nj, s_side, ~0ull, s); break;
+    case 2: key_kernel_launch<AT400, Net, 2, OF>(sms, arena, off, n, out, J, nj, s_side, ~0ull, s); break;
+    default: key_kernel_launch<AT400, Net, 0, OF>(sms, arena, off, n, out, J, nj, s_side, ~0ull, s); break;
   }
 }
 
@@ -1241,24 +1241,18 @@ static as_status ensure_device(DeviceState** out) {
     if ((e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
       return cuda_fail(e, "device query");
     {
-      if ((e = key_kernel_attrs<true, Net16<4>, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, Net16<4>, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<true, Net16<2>, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, Net16<2>, false>()) != cudaSuccess ||
-          (e = key_kernel_attrs<true, Net16<4>, true>()) != cudaSuccess ||
-          (e = key_kernel_attrs<false, Net16<4>, true>()) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(
-               reinterpret_cast<const void*>(
-                   sig_key_kernel<true, Net16<4>, kLKShapes[0].warps, kLKShapes[0].depth, false, true>),
-               cudaFuncAttributeMaxDynamicSharedMemorySize,
-               (int)lk_smem_bytes<Net16<4>>(kLKShapes[0].warps, kLKShapes[0].depth))) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(
-               reinterpret_cast<const void*>(
-                   sig_key_kernel<false, Net16<4>, kLKShapes[0].warps, kLKShapes[0].depth, false, true>),
-               cudaFuncAttributeMaxDynamicSharedMemorySize,
-               (int)lk_smem_bytes<Net16<4>>(kLKShapes[0].warps, kLKShapes[0].depth))) != cudaSuccess ||
-          (e = key_kernel_attr<true, Net8, 0, false>()) != cudaSuccess ||
-          (e = key_kernel_attr<false, Net8, 0, false>()) != cudaSuccess)
+      if ((e = key_kernel_attrs<true, Net16<4>, LKOf::kRows>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<4>, LKOf::kRows>()) != cudaSuccess ||
+          (e = key_kernel_attrs<true, Net16<2>, LKOf::kRows>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<2>, LKOf::kRows>()) != cudaSuccess ||
+          (e = key_kernel_attrs<true, Net16<4>, LKOf::kBatchRows>()) != cudaSuccess ||
+          (e = key_kernel_attrs<false, Net16<4>, LKOf::kBatchRows>()) != cudaSuccess ||
+          (e = key_kernel_attr<true, Net16<4>, 0, LKOf::kPrefixes>()) != cudaSuccess ||
+          (e = key_kernel_attr<false, Net16<4>, 0, LKOf::kPrefixes>()) != cudaSuccess ||
+          (e = key_kernel_attr<true, Net16<4>, 0, LKOf::kItems>()) != cudaSuccess ||
+          (e = key_kernel_attr<false, Net16<4>, 0, LKOf::kItems>()) != cudaSuccess ||
+          (e = key_kernel_attr<true, Net8, 0, LKOf::kRows>()) != cudaSuccess ||
+          (e = key_kernel_attr<false, Net8, 0, LKOf::kRows>()) != cudaSuccess)
         return cuda_fail(e, "kernel attribute");
     }
     // where dynamic shared memory starts (the tables are its first bytes)
@@ -1362,19 +1356,18 @@ static bool table_geometry(uint64_t m, float lf, uint64_t* cap, uint32_t* log2ca
 }
 
 static as_status launch_sig(const uint8_t* arena, const uint64_t* off, uint64_t n, uint64_t* out, cudaStream_t s,
-                            int ncomp = 4, int shape = 0, int max_blocks = 0, uint64_t cap_len = ~0ull) {
+                            int ncomp = 4, int shape = 0) {
   DeviceState* d = nullptr;
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
-  if (max_blocks <= 0) max_blocks = d->sms;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
   if (ncomp == 2) {
-    if (d->tables_at400) key_kernel_launch_shape<true, Net16<2>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
-    else key_kernel_launch_shape<false, Net16<2>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, Net16<2>, LKOf::kRows>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
+    else key_kernel_launch_shape<false, Net16<2>, LKOf::kRows>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
   } else {
-    if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
-    else key_kernel_launch_shape<false, Net16<4>, false>(shape, max_blocks, arena, off, n, out, nullptr, 0, 0, cap_len, s);
+    if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, LKOf::kRows>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
+    else key_kernel_launch_shape<false, Net16<4>, LKOf::kRows>(shape, d->sms, arena, off, n, out, nullptr, 0, 0, s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
@@ -1398,27 +1391,33 @@ static void split_sms(int sms, uint64_t m, uint64_t n, int* blocks_r, int* block
   *blocks_s = sms - *blocks_r;
 }
 
-// The signatures of a join's two relations in one launch (shape 0, four components).
+// The signatures of a join's two relations in one launch (shape 0, four
+// components): of the whole rows, or of their first cap_len bytes.
+template <LKOf OF>
 static as_status launch_sig_two(const DeviceState* d, const uint8_t* arenaR, const uint64_t* offR, uint64_t m,
                                 uint64_t* sigR, const uint8_t* arenaS, const uint64_t* offS, uint64_t n, uint64_t* sigS,
-                                uint64_t cap_len, cudaStream_t s) {
-  if (m == 0 || n == 0) {
-    if (m > 0) return launch_sig(arenaR, offR, m, sigR, s, 4, 0, 0, cap_len);
-    return launch_sig(arenaS, offS, n, sigS, s, 4, 0, 0, cap_len);
-  }
-  int blocks_r, blocks_s;
-  split_sms(d->sms, m, n, &blocks_r, &blocks_s);
+                                cudaStream_t s, uint64_t cap_len = ~0ull) {
+  if (m == 0 && n == 0) return AS_OK;
   LKSecond second;
-  second.arena = arenaS;
-  second.off = offS;
-  second.n = n;
-  second.sig_out = sigS;
+  int blocks_r = d->sms, blocks_s = 0;
+  if (m == 0) {
+    arenaR = arenaS;
+    offR = offS;
+    m = n;
+    sigR = sigS;
+  } else if (n > 0) {
+    split_sms(d->sms, m, n, &blocks_r, &blocks_s);
+    second.arena = arenaS;
+    second.off = offS;
+    second.n = n;
+    second.sig_out = sigS;
+  }
   if (d->tables_at400)
-    key_kernel_launch<true, Net16<4>, 0, false>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
-                                                blocks_s);
+    key_kernel_launch<true, Net16<4>, 0, OF>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
+                                             blocks_s);
   else
-    key_kernel_launch<false, Net16<4>, 0, false>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
-                                                 blocks_s);
+    key_kernel_launch<false, Net16<4>, 0, OF>(blocks_r, arenaR, offR, m, sigR, nullptr, 0, 0, cap_len, s, second,
+                                              blocks_s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "signature kernel launch");
   return AS_OK;
@@ -1430,8 +1429,8 @@ static as_status launch_sig_batch(const DeviceState* d, const uint8_t* arena, co
                                   uint64_t* out, const BatchJoin* J, int nj, int s_side, int shape, cudaStream_t s) {
   if (n == 0) return AS_OK;
   if (shape < 0 || shape >= kLKShapeCount) return fail(AS_ERR_INVALID, "signature kernel shape %d", shape);
-  if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
-  else key_kernel_launch_shape<false, Net16<4>, true>(shape, d->sms, arena, off, n, out, J, nj, s_side, ~0ull, s);
+  if (d->tables_at400) key_kernel_launch_shape<true, Net16<4>, LKOf::kBatchRows>(shape, d->sms, arena, off, n, out, J, nj, s_side, s);
+  else key_kernel_launch_shape<false, Net16<4>, LKOf::kBatchRows>(shape, d->sms, arena, off, n, out, J, nj, s_side, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "batch signature kernel launch");
   return AS_OK;
@@ -1521,10 +1520,10 @@ as_status as_sig_compute_gf8(const uint8_t* d_arena, const uint64_t* d_off, uint
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
   if (d->tables_at400)
-    key_kernel_launch<true, Net8, 0, false>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
+    key_kernel_launch<true, Net8, 0, LKOf::kRows>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
                                             (cudaStream_t)stream);
   else
-    key_kernel_launch<false, Net8, 0, false>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
+    key_kernel_launch<false, Net8, 0, LKOf::kRows>(d->sms, d_arena, d_off, n, d_sig_out, nullptr, 0, 0, ~0ull,
                                              (cudaStream_t)stream);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "byte-symbol signature kernel launch");
@@ -1581,11 +1580,11 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
   it.keys = n;
   it.block = block_bytes;
   if (d->tables_at400)
-    sig_key_kernel<true, Net16<4>, k.warps, k.depth, false, true>
+    sig_key_kernel<true, Net16<4>, k.warps, k.depth, LKOf::kItems>
         <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
             d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
   else
-    sig_key_kernel<false, Net16<4>, k.warps, k.depth, false, true>
+    sig_key_kernel<false, Net16<4>, k.warps, k.depth, LKOf::kItems>
         <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
             d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
   const uint64_t scan_want = (n + kPScanThreads - 1) / kPScanThreads;
@@ -1929,8 +1928,8 @@ as_status as_join(const uint8_t* d_arenaR, const uint64_t* d_offR, const uint32_
   if ((st = probe_args("as_join", &t, d_arenaS, d_offS, n, d_pairs, cap_pairs, cnt)) != AS_OK) return st;
   Slot* slots = reinterpret_cast<Slot*>(t.slots);
   if ((st = launch_clear(d, slots, t.cap * 16, t.flags, cnt, 1, s)) != AS_OK) return st;
-  if ((st = launch_sig_two(d, d_arenaR, d_offR, m, const_cast<uint64_t*>(t.sigR), d_arenaS, d_offS, n, sigS, ~0ull,
-                           s)) != AS_OK)
+  if ((st = launch_sig_two<LKOf::kRows>(d, d_arenaR, d_offR, m, const_cast<uint64_t*>(t.sigR), d_arenaS, d_offS, n, sigS,
+                                        s)) != AS_OK)
     return st;
   if ((st = launch_build(d, slots, t.cap, t.sigR, d_offR, m, t.flags, s)) != AS_OK) return st;
   if (n > 0 && (st = launch_verify(d, &t, d_arenaS, d_offS, d_idS, n, sigS, d_pairs, cap_pairs, cnt, s)) != AS_OK)
@@ -1983,7 +1982,9 @@ as_status as_join_prefix(const uint8_t* d_arenaR, const uint64_t* d_offR, const 
   uint64_t* cnt = d_count ? d_count : (uint64_t*)(tail + 256);
   cudaError_t e;
   if ((st = launch_clear(d, slots, cap * 16, flags, cnt, 1, s)) != AS_OK) return st;
-  if ((st = launch_sig_two(d, d_arenaR, d_offR, m, sigR, d_arenaS, d_offS, n, sigS, prefix_len, s)) != AS_OK) return st;
+  if ((st = launch_sig_two<LKOf::kPrefixes>(d, d_arenaR, d_offR, m, sigR, d_arenaS, d_offS, n, sigS, s, prefix_len)) !=
+      AS_OK)
+    return st;
   if ((st = launch_build(d, slots, cap, sigR, d_offR, m, flags, s, prefix_len)) != AS_OK) return st;
   if (n > 0) {
     as_table t;

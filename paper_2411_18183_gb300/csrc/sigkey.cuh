@@ -103,6 +103,8 @@ constexpr uint64_t kLKKeyCost = 256;
 
 struct LKWarp {
   uint64_t woff[kLKWin + 2];       // offsets of the window's keys (woff[i] = off[wb + i]), i <= wn
+  uint64_t full, rest_lo, rest_hi; // keys cut to a length: the end of the full bands, the warp's keys after them
+  uint64_t pad;
   uint8_t order[kLKWin];           // window entries by block count
 };
 static_assert(kLKWin == 256, "the window sort: 8 entries and 8 bins per lane, entries in a byte");
@@ -558,8 +560,7 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
 // relation): equal counts of whole groups below kLKSearchFrom keys (or if
-// by_count: keys cut to a length are about equally long), for a group takes as
-// long with one key as with 32 (100k keys of 64-256 bytes, 41 per warp: 14.9 us
+// by_count), for a group takes as long with one key as with 32 (100k keys of 64-256 bytes, 41 per warp: 14.9 us
 // cut by keys, 11.7 us by groups; 300k keys of 256-1024 bytes, 123 per warp: 45.4
 // and 43.9 us; 100k keys of 2-8 KB: 120 and 102 us), else equal shares of the
 // work, key bytes + kLKKeyCost per key (in a batch, over the joins' keys back
@@ -625,6 +626,44 @@ __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, i
     *lo = cut(warp);
     *hi = cut(warp + 1);
   }
+}
+
+// Keys of which only the first bytes are signed (a prefix join's): the work of a
+// range of keys is not to be had from the offsets, and their lengths differ where
+// the cap is above some.  So a warp takes kLKBand keys at a time, in bands of
+// kLKBand keys per warp over the whole relation (bands' neighbours go to different
+// SMs), and what is left, or a relation of less than two bands, in equal counts
+// of whole groups.  A run of long keys is then spread over all warps.  (Join on
+// prefixes of 4 KB of 2M keys of 64 bytes followed by 60k of 8 KB: 292 us, 836 with one
+// range of equally many keys per warp.)
+constexpr uint32_t kLKBand = 256;
+template <int kWarps>
+__device__ __forceinline__ void lk_first_band(LKWarp& W, uint64_t n, uint64_t warp, uint64_t nwarps, uint64_t* lo,
+                                              uint64_t* hi) {
+  const uint64_t place = (warp % kWarps) * (nwarps / kWarps) + warp / kWarps;
+  const uint64_t band = kLKBand * nwarps, full = n < 2 * band ? 0 : n / band * band;
+  const uint64_t groups = (n - full + 31) / 32;
+  const uint64_t rest_lo = full + 32 * (groups * warp / nwarps);
+  uint64_t rest_hi = full + 32 * (groups * (warp + 1) / nwarps);
+  if (rest_hi > n) rest_hi = n;
+  if ((threadIdx.x & 31u) == 0) {
+    W.full = full;
+    W.rest_lo = rest_lo;
+    W.rest_hi = rest_hi;
+  }
+  *lo = full ? kLKBand * place : rest_lo;
+  *hi = full ? kLKBand * (place + 1) : rest_hi;
+}
+// the warp's keys after its keys [.., hi); false: none
+__device__ __forceinline__ bool lk_next_band(const LKWarp& W, uint64_t nwarps, uint64_t* lo, uint64_t* hi) {
+  if (*hi > W.full) return false;
+  *lo = *hi + kLKBand * (nwarps - 1);
+  *hi = *lo + kLKBand;
+  if (*lo >= W.full) {
+    *lo = W.rest_lo;
+    *hi = W.rest_hi;
+  }
+  return *lo < *hi;
 }
 
 // Keys cut into pieces: key i's pieces of `block` bytes (the last one shorter;
@@ -717,17 +756,21 @@ struct LKSecond {
   uint32_t from = 0xFFFFFFFFu;
 };
 
-// The signatures of n keys: the rows of a relation (BATCH false), or the
-// virtual rows of one side of a batch (BATCH true; s_side picks S, J and nj
-// describe the joins, and sig_out is indexed by virtual row); of each key's
-// first cap_len bytes.  ITEMS: of the n keys' items.
-template <bool AT400, class Net, int kLKWarps, int kLKDepth, bool BATCH, bool ITEMS = false>
+// Whose signatures the kernel computes: of the rows of a relation, of the virtual
+// rows of one side of a batch (s_side picks S, J and nj describe the joins, and
+// sig_out is indexed by virtual row), of the first cap_len bytes of a relation's
+// rows, or of the items of its rows.
+enum class LKOf { kRows, kBatchRows, kPrefixes, kItems };
+
+template <bool AT400, class Net, int kLKWarps, int kLKDepth, LKOf OF>
 __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t* __restrict__ arena,
                                                                 const uint64_t* __restrict__ off, uint64_t n,
                                                                 uint64_t* __restrict__ sig_out,
                                                                 const BatchJoin* __restrict__ J, int nj, int s_side,
-                                                                uint64_t cap_len, const LKItems items = LKItems(),
+                                                                uint64_t cap, const LKItems items = LKItems(),
                                                                 const LKSecond second = LKSecond()) {
+  constexpr bool BATCH = OF == LKOf::kBatchRows, ITEMS = OF == LKOf::kItems, CAPPED = OF == LKOf::kPrefixes;
+  const uint64_t cap_len = CAPPED ? cap : ~0ull;
   if constexpr (ITEMS) {
     if (!by_items(off, n, items.block)) return;
   }
@@ -764,7 +807,11 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     lk_warp_range<false, kLKWarps>(J, nj, s_side, off, __ldg(items.first + n), warp, nwarps, true, &k_lo, &k_hi);
     if (k_lo < k_hi) kb = warp_lower_bound(items.first, n, k_lo + 1) - 1;
   } else {
-    lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, cap_len != ~0ull, &k_lo, &k_hi);
+    if (CAPPED && lane == 0) W.full = 0;            // one range of keys
+    if (CAPPED && n > 32 * nwarps)
+      lk_first_band<kLKWarps>(W, n, warp, nwarps, &k_lo, &k_hi);
+    else
+      lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, false, &k_lo, &k_hi);
   }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, most, &wa) : 0u;
@@ -796,7 +843,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     if (g == ng) {                                    // the next window, as prefetched
       if (ng) {
         wb += wn;
-        if (wb >= k_hi) return 0u;
+        if (wb >= k_hi && (!CAPPED || !lk_next_band(W, nwarps, &wb, &k_hi))) return 0u;
         wn = lk_window<BATCH>(J, nj, s_side, wb, k_hi, most, &wa);
       }
       g = 0;
@@ -813,9 +860,9 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena, cap_len);
     if (++g == ng) {                                  // the window's offsets are free: fetch the next ones
       __syncwarp();
-      if (!ITEMS && wb + wn < k_hi) {
-        uint64_t na;
-        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, wb + wn, k_hi, most, &na);
+      uint64_t nb = wb + wn, nh = k_hi, na;
+      if (!ITEMS && (nb < nh || (CAPPED && lk_next_band(W, nwarps, &nb, &nh)))) {
+        const uint32_t nn = lk_window<BATCH>(J, nj, s_side, nb, nh, most, &na);
         lk_prefetch_window(W, off, na, na + nn);
       }
     }

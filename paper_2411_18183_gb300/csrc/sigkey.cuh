@@ -559,23 +559,23 @@ __device__ __forceinline__ uint32_t lk_window(const BatchJoin* __restrict__ J, i
 }
 
 // A warp's keys [lo, hi) of n (virtual rows of a batch side, or rows of a
-// relation): equal counts of whole groups below kLKSearchFrom keys (or if
-// by_count), for a group takes as long with one key as with 32 (100k keys of 64-256 bytes, 41 per warp: 14.9 us
-// cut by keys, 11.7 us by groups; 300k keys of 256-1024 bytes, 123 per warp: 45.4
-// and 43.9 us; 100k keys of 2-8 KB: 120 and 102 us), else equal shares of the
-// work, key bytes + kLKKeyCost per key (in a batch, over the joins' keys back
-// to back).  Whole warp.
+// relation): equal counts of whole groups below kLKSearchFrom keys, for a group
+// takes as long with one key as with 32 (100k keys of 64-256 bytes, 41 per warp:
+// 14.9 us cut by keys, 11.7 us by groups; 300k keys of 256-1024 bytes, 123 per
+// warp: 45.4 and 43.9 us; 100k keys of 2-8 KB: 120 and 102 us), else equal shares
+// of the work, key bytes + kLKKeyCost per key (in a batch, over the joins' keys
+// back to back).  Whole warp.
 template <bool BATCH, int kWarps>
 __device__ __forceinline__ void lk_warp_range(const BatchJoin* __restrict__ J, int nj, int s_side,
                                               const uint64_t* __restrict__ off, uint64_t n, uint64_t warp,
-                                              uint64_t nwarps, bool by_count, uint64_t* lo, uint64_t* hi) {
+                                              uint64_t nwarps, uint64_t* lo, uint64_t* hi) {
   if (n <= 32 * nwarps) {                            // at most one group per warp
     const uint64_t u = (warp % kWarps) * (nwarps / kWarps) + warp / kWarps;   // neighbouring groups on different SMs
     *lo = 32 * u < n ? 32 * u : n;
     *hi = 32 * u + 32 < n ? 32 * u + 32 : n;
     return;
   }
-  if (by_count || n < kLKSearchFrom) {
+  if (n < kLKSearchFrom) {
     const uint64_t groups = (n + 31) / 32;
     *lo = 32 * (groups * warp / nwarps);             // (64-bit products: a 128-bit division costs 1 us here)
     *hi = 32 * (groups * (warp + 1) / nwarps);
@@ -687,6 +687,60 @@ struct LKItems {
 __device__ __forceinline__ bool by_items(const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
   const uint64_t bytes = __ldg(off + n) - __ldg(off);
   return block < 32u ? bytes < 192u * n : bytes >= (block < 64u ? 256u : 128u) * n;
+}
+
+// A warp's items [lo, hi), whole groups of 32 but at the end, and a key at or
+// before the one that holds item lo.  Up to a group per warp one group each;
+// else equal shares of the work, the items' bytes + kLKKeyCost per item, for
+// blocks of more than a few hundred bytes differ in length as keys do.  (2M keys
+// of 64 bytes followed by 60k of 8 KB, with equally many items per warp instead:
+// 820 us for blocks of 4 KB, 257 now; 500k keys of 200-2000 bytes unchanged.)  Both
+// ends are searched for in the same loads, 32 keys at a time.
+template <int kWarps>
+__device__ __forceinline__ void lk_item_range(const uint64_t* __restrict__ off, const LKItems& it, uint64_t warp,
+                                              uint64_t nwarps, uint64_t* lo, uint64_t* hi, uint64_t* key) {
+  const uint64_t lane = threadIdx.x & 31u, n = it.keys, items = __ldg(it.first + n);
+  if (items <= 32 * nwarps) {
+    const uint64_t u = (warp % kWarps) * (nwarps / kWarps) + warp / kWarps;   // neighbouring groups on different SMs
+    *lo = min(32 * u, items);
+    *hi = min(32 * u + 32, items);
+    *key = *lo < *hi ? warp_lower_bound(it.first, n, *lo + 1) - 1 : 0;
+    return;
+  }
+  const uint64_t base = __ldg(off), total = __ldg(off + n) - base + kLKKeyCost * items;
+  auto work = [&](uint64_t k) { return __ldg(off + k) - base + kLKKeyCost * __ldg(it.first + k); };   // before key k
+  uint64_t t[2], a[2] = {0, 0}, b[2] = {n, n};       // the first key with more work before it than t: in [a, b]
+  const uint64_t share = total / nwarps, rest = total - share * nwarps;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)                        // total (warp + j) / nwarps
+    t[j] = share * (warp + j) + (uint32_t)rest * (uint32_t)(warp + j) / (uint32_t)nwarps;
+  while (a[0] < b[0] || a[1] < b[1]) {               // warp-uniform
+    uint64_t step[2];
+    bool before[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      step[j] = (b[j] - a[j] + 31) / 32;
+      const uint64_t i = a[j] + lane * step[j];
+      before[j] = i < b[j] && work(i) <= t[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {                    // lanes 0..cnt - 1 are before t, the next one is not
+      const uint64_t cnt = (uint64_t)__popc(__ballot_sync(kFull, before[j]));
+      const uint64_t next = a[j] + cnt * step[j];
+      if (cnt) a[j] = next - step[j] + 1;
+      b[j] = min(next, b[j]);
+    }
+  }
+  uint64_t cut[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const uint64_t k = a[j] ? a[j] - 1 : 0, f = __ldg(it.first + k);
+    const uint64_t in = min((t[j] - work(k)) / (it.block + kLKKeyCost), __ldg(it.first + k + 1) - f);
+    cut[j] = min((f + in + 31) / 32 * 32, items);
+    if (j == 0) *key = k;
+  }
+  *lo = cut[0];
+  *hi = warp + 1 >= nwarps ? items : cut[1];
 }
 
 // the starts of items [wb, wb + wn) and the end of the last one into the
@@ -804,14 +858,13 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   uint32_t most = kLKWin;
   if constexpr (ITEMS) {
     if (items.block >= kLKNarrowFrom) most = kLKNarrowWin;
-    lk_warp_range<false, kLKWarps>(J, nj, s_side, off, __ldg(items.first + n), warp, nwarps, true, &k_lo, &k_hi);
-    if (k_lo < k_hi) kb = warp_lower_bound(items.first, n, k_lo + 1) - 1;
+    lk_item_range<kLKWarps>(off, items, warp, nwarps, &k_lo, &k_hi, &kb);
   } else {
     if (CAPPED && lane == 0) W.full = 0;            // one range of keys
     if (CAPPED && n > 32 * nwarps)
       lk_first_band<kLKWarps>(W, n, warp, nwarps, &k_lo, &k_hi);
     else
-      lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, false, &k_lo, &k_hi);
+      lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
   }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, most, &wa) : 0u;

@@ -1113,8 +1113,6 @@ struct DeviceState {
   bool ready = false;
   int sms = 0;
   int verify_blocks_per_sm = 1;
-  int prefix_blocks_per_sm = 1;
-  int prefix_thread_blocks_per_sm = 1;
   bool tables_at400 = false;   // dynamic shared memory starts at shared address 0x400
   cudaStream_t side[kSideStreams] = {};   // side streams (SideStream), created with the state
   std::atomic<unsigned> side_next{0};
@@ -1269,23 +1267,9 @@ static as_status ensure_device(DeviceState** out) {
     for (int i = 0; i < kSideStreams; ++i)
       if ((e = cudaStreamCreateWithFlags(&d.side[i], cudaStreamNonBlocking)) != cudaSuccess)
         return cuda_fail(e, "side stream");
-    if ((e = cudaFuncSetAttribute(prefix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPrefix)) !=
+    if ((e = cudaFuncSetAttribute(prefix_rest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPScan)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.prefix_blocks_per_sm, prefix_kernel, kPThreads,
-                                                           kSmemPrefix)) != cudaSuccess)
-      return cuda_fail(e, "occupancy query");
-    if (d.prefix_blocks_per_sm < 1) d.prefix_blocks_per_sm = 1;
-    if ((e = cudaFuncSetAttribute(prefix_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPScan)) !=
-        cudaSuccess)
-      return cuda_fail(e, "kernel attribute");
-    if ((e = cudaFuncSetAttribute(prefix_thread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kSmemPThread)) != cudaSuccess)
-      return cuda_fail(e, "kernel attribute");
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.prefix_thread_blocks_per_sm, prefix_thread_kernel,
-                                                           kPThreadThreads, kSmemPThread)) != cudaSuccess)
-      return cuda_fail(e, "occupancy query");
-    if (d.prefix_thread_blocks_per_sm < 1) d.prefix_thread_blocks_per_sm = 1;
     if ((e = cudaFuncSetAttribute(bl_hash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBHash)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
@@ -1572,8 +1556,8 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
   as_status st = ensure_device(&d);
   if (st != AS_OK) return st;
   if (n == 0) return AS_OK;
-  // the blocks' own signatures and their sums along each key, or one key per thread or warp (by_items: the
-  // kernels of the one that is not wanted return at once)
+  // the blocks' own signatures, then their sums along each key or, without the former, one key per thread or
+  // warp (by_items picks on the device)
   constexpr LKShape k = kLKShapes[0];
   LKItems it;
   it.first = d_pref_off;
@@ -1587,25 +1571,20 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
     sig_key_kernel<false, Net16<4>, k.warps, k.depth, LKOf::kItems>
         <<<d->sms, 32 * k.warps, lk_smem_bytes<Net16<4>>(k.warps, k.depth), (cudaStream_t)stream>>>(
             d_arena, d_off, n, d_out, nullptr, 0, 0, ~0ull, it);
-  const uint64_t scan_want = (n + kPScanThreads - 1) / kPScanThreads;
-  prefix_scan_kernel<<<(unsigned)(scan_want < (uint64_t)d->sms ? scan_want : (uint64_t)d->sms), kPScanThreads, kSmemPScan,
-                       (cudaStream_t)stream>>>(d_off, n, block_bytes, d_pref_off, d_out);
-  if (block_bytes >= 32) {
-    // entries at most every other chunk: one thread per key, the suffix snapshots of prefix_thread_kernel
-    const uint64_t want = (n + kPThreadThreads - 1) / kPThreadThreads;
-    const uint64_t lim = (uint64_t)d->sms * (uint64_t)d->prefix_thread_blocks_per_sm;
-    const unsigned blocks = (unsigned)(want < lim ? want : lim);
-    prefix_thread_kernel<<<blocks, kPThreadThreads, kSmemPThread, (cudaStream_t)stream>>>(d_arena, d_off, n, block_bytes,
-                                                                                       d_pref_off, d_out);
-  } else {
-    // an entry after every chunk: one warp per key, the scan of D over the lanes
-    const uint64_t want = (n + kPThreads / 32 - 1) / (kPThreads / 32);
-    const uint64_t lim = (uint64_t)d->sms * (uint64_t)d->prefix_blocks_per_sm;   // persistent: one wave
-    const unsigned blocks = (unsigned)(want < lim ? want : lim);
-    prefix_kernel<<<blocks, kPThreads, kSmemPrefix, (cudaStream_t)stream>>>(d_arena, d_off, n, block_bytes, d_pref_off,
-                                                                            d_out);
-  }
   cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "prefix kernel launch");
+  const uint64_t want = block_bytes < 32 ? n : (n + 31) / 32;   // a block for every warp with work, up to a block per SM
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(want < (uint64_t)d->sms ? want : (uint64_t)d->sms));
+  cfg.blockDim = dim3(kPRestThreads);
+  cfg.dynamicSmemBytes = kSmemPScan;
+  cfg.stream = (cudaStream_t)stream;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, prefix_rest_kernel, d_arena, d_off, n, block_bytes, d_pref_off, d_out);
   if (e != cudaSuccess) return cuda_fail(e, "prefix kernel launch");
   return AS_OK;
 }

@@ -11,29 +11,38 @@
 //
 // Kernels.  prefix_count_kernel / prefix_total_kernel / prefix_offset_kernel
 // lay out the output: key i's entries start at pref_off[i], an exclusive scan
-// of max(1, ceil(len_i / B)).  For B >= 32, prefix_thread_kernel (below)
-// computes the entries, one thread per key.  For B = 16 (an entry after every
-// chunk) prefix_kernel computes them: one warp per
-// key, 512 key bytes per step, lane l taking the key's 16-byte chunk c = 32 s + l
-// (realigned to the key's first byte from two aligned chunks, the word part of
-// the realignment warp-uniform).  The chunk's value T_c = sum_j q_j x^(k j) is a
-// Horner step from zero (gf16.cuh).  With C(c) = sum_{c' <= c} x^(8 k c') T_c'
-// the prefix through chunk c, the warp carries D(c) = x^(-8 k c) C(c), which
-// obeys D(c) = x^(-8 k) D(c-1) + T_c: an inclusive scan over the lanes whose
-// level s multiplies by the constant x^(-8 k 2^s) (tables in shared memory),
-// with the previous step's last D entering at lane 0.  Only the lanes whose
-// chunk ends a block (or the key) form C = x^(8 k c) D through the log /
+// of max(1, ceil(len_i / B)).  The entries take two launches, and by_items
+// (sigkey.cuh) picks on the device what they do: the signature kernel signs all
+// keys' blocks and prefix_rest_kernel adds them up along each key (prefix_sums);
+// or the signature kernel returns at once and prefix_rest_kernel does it all, one
+// thread per key (prefix_by_thread) or, for B = 16 (an entry after every chunk),
+// one warp per key (prefix_by_warp): 512 key bytes per step, lane l taking the
+// key's 16-byte chunk c = 32 s + l (realigned to the key's first byte from two
+// aligned chunks, the word part of the realignment warp-uniform).  The chunk's
+// value T_c = sum_j q_j x^(k j) is a Horner step from zero (gf16.cuh).  With C(c) =
+// sum_{c' <= c} x^(8 k c') T_c' the prefix through chunk c, the warp carries D(c) =
+// x^(-8 k c) C(c), which obeys D(c) = x^(-8 k) D(c-1) + T_c: an inclusive scan over
+// the lanes whose level s multiplies by the constant x^(-8 k 2^s) (tables in
+// shared memory), with the previous step's last D entering at lane 0.  Only the
+// lanes whose chunk ends a block (or the key) form C = x^(8 k c) D through the log /
 // antilog tables and store it.
 #pragma once
 #include <cstdint>
 
 namespace algsig {
 
-constexpr int kPThreads = 256;          // threads per block of the prefix kernels
+constexpr int kPThreads = 256;          // threads per block of the offset kernels
+constexpr int kPRestThreads = 1024;     // and of prefix_rest_kernel
 constexpr int kPLevels = 5;             // scan levels over 32 lanes
 constexpr int kPConst = 4 * kPLevels;   // tables x^(-8 k 2^s), k = 1..4, s = 0..4, at (k-1)*kPLevels+s
 // multiply-by-constant tables of the prefix scan (layout of rounds.cuh's), set up once per device
 __device__ uint16_t g_pconst[kPConst * 512];
+
+// the warp's number in prefix_rest_kernel: neighbouring ones on different SMs, so that few keys use them all
+__device__ __forceinline__ uint64_t prefix_warp() { return (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
+// wait until the kernel launched before has ended, where this one was allowed to start earlier
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // component-wise multiply of a packed value by x^(-8 k 2^s)
 __device__ __forceinline__ uint64_t mul_pscan(const uint16_t* ptab, uint64_t v, int s) {
@@ -251,14 +260,9 @@ __device__ __forceinline__ void prefix_load(const uint8_t* __restrict__ arena, u
 // sequence of (key, step) items, and the chunks of the next item (and the
 // offsets of the next key) are loaded before the current item is computed, so
 // the memory latency of a step overlaps the arithmetic of the one before.
-__global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __restrict__ arena,
-                                                           const uint64_t* __restrict__ off, uint64_t n,
-                                                           uint32_t block_bytes,
-                                                           const uint64_t* __restrict__ pref_off,
-                                                           uint64_t* __restrict__ out) {
-  if (by_items(off, n, block_bytes)) return;
-  extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ uint4 emask[17];
+__device__ __forceinline__ void prefix_by_warp(uint8_t* smem, uint4* emask, const uint8_t* __restrict__ arena,
+                                               const uint64_t* __restrict__ off, uint64_t n, uint32_t block_bytes,
+                                               const uint64_t* __restrict__ pref_off, uint64_t* __restrict__ out) {
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* ptab = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);
   for (int i = threadIdx.x; i < kPConst * 512 / 2; i += blockDim.x)
@@ -273,8 +277,8 @@ __global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __rest
   bp.dr = 32u % bp.cpb;
   bp.q0 = lane / bp.cpb;
   bp.r0 = lane % bp.cpb;
-  const uint64_t nwarps = (uint64_t)gridDim.x * (kPThreads / 32);
-  uint64_t i = (uint64_t)blockIdx.x * (kPThreads / 32) + (threadIdx.x >> 5);
+  const uint64_t nwarps = (uint64_t)gridDim.x * (kPRestThreads / 32);
+  uint64_t i = prefix_warp();
   if (i >= n) return;                                // warp-uniform
   // current key and its first step's chunks; the next key's offsets
   uint64_t s0 = off[i], len = off[i + 1] - s0, po = pref_off[i];
@@ -320,8 +324,6 @@ __global__ void __launch_bounds__(kPThreads) prefix_kernel(const uint8_t* __rest
   }
 }
 
-constexpr int kPThreadThreads = 1024;       // threads per block of prefix_thread_kernel
-
 // Cumulative signatures, one thread per key.  The thread runs the backward
 // Horner rule over the key's realigned chunks; since B is a
 // multiple of 16 every block boundary b_j = lo + (j+1) B falls at offset lo of
@@ -331,14 +333,9 @@ constexpr int kPThreadThreads = 1024;       // threads per block of prefix_threa
 //     C_j = S + x^(8 k c_j - k lo/2) acc'_j
 // (prefix = whole key minus suffix, the suffix moved to its place), formed
 // through the log / antilog tables, once per stored entry.
-__global__ void __launch_bounds__(kPThreadThreads) prefix_thread_kernel(const uint8_t* __restrict__ arena,
-                                                                    const uint64_t* __restrict__ off, uint64_t n,
-                                                                    uint32_t block_bytes,
-                                                                    const uint64_t* __restrict__ pref_off,
-                                                                    uint64_t* __restrict__ out) {
-  if (by_items(off, n, block_bytes)) return;
-  extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ uint4 emask[17];
+__device__ __forceinline__ void prefix_by_thread(uint8_t* smem, uint4* emask, const uint8_t* __restrict__ arena,
+                                                 const uint64_t* __restrict__ off, uint64_t n, uint32_t block_bytes,
+                                                 const uint64_t* __restrict__ pref_off, uint64_t* __restrict__ out) {
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* inv32 = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);
   for (int i = threadIdx.x; i < 256; i += blockDim.x)
@@ -347,8 +344,8 @@ __global__ void __launch_bounds__(kPThreadThreads) prefix_thread_kernel(const ui
   init_red_tables(red, red + kRedWords);                     // ends with __syncthreads()
   const RedCursor rc = red_cursor(red);
   const uint64_t cpb = block_bytes / 16u;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+  const uint64_t stride = (uint64_t)gridDim.x * kPRestThreads;
+  for (uint64_t i = 32 * prefix_warp() + (threadIdx.x & 31u); i < n; i += stride) {
     const uint64_t s0 = off[i], len = off[i + 1] - s0;
     uint64_t* o = out + pref_off[i];
     if (len == 0) {
@@ -404,21 +401,17 @@ __global__ void __launch_bounds__(kPThreadThreads) prefix_thread_kernel(const ui
 // up to 32 lines, 500k keys of 200-2000 bytes at B = 256 took 50 us, 23 now
 // (whole call 290 -> 265 us; at B = 64 720 -> 565; three keys of 1.4 MB on average
 // at B = 256 780 -> 605).
-constexpr int kPScanThreads = 1024;
 constexpr uint32_t kPScanLow = 16, kPScanHigh = 32;   // factors l and q: 0..15 and 0..31
 constexpr uint32_t kPScanTables = (kPScanLow - 1 + kPScanHigh - 1) * 8;
 constexpr size_t kSmemPScan = (size_t)kPScanTables * 512;
-__global__ void __launch_bounds__(kPScanThreads, 1) prefix_scan_kernel(const uint64_t* __restrict__ off, uint64_t n,
-                                                                    uint32_t block_bytes,
-                                                                    const uint64_t* __restrict__ pref_off,
-                                                                    uint64_t* __restrict__ out) {
-  if (!by_items(off, n, block_bytes) || pref_off[n] == n) return;   // no key of two blocks: nothing to add
-  extern __shared__ __align__(128) uint8_t smem[];
+__device__ __forceinline__ void prefix_sums(uint8_t* smem, const uint64_t* __restrict__ off, uint64_t n,
+                                            uint32_t block_bytes, const uint64_t* __restrict__ pref_off,
+                                            uint64_t* __restrict__ out) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t eb = (block_bytes / 2u) % kOrder;     // exponent from one block to the next
   // table t = 8 f + 2 (k - 1) + h, f a factor (l - 1, then 15 + q - 1): its products with a byte at bits
   // 8 h..8 h + 7; a lane makes the entries 8 lane..8 lane + 7 from the products with single bits
-  for (uint32_t t = threadIdx.x >> 5; t < kPScanTables; t += kPScanThreads / 32) {
+  for (uint32_t t = threadIdx.x >> 5; t < kPScanTables; t += kPRestThreads / 32) {
     const uint32_t f = t >> 3, i = f < kPScanLow - 1 ? f + 1 : kPScanLow * (f - (kPScanLow - 2));
     const uint32_t e0 = (uint32_t)((uint64_t)i * (((t >> 1) & 3u) + 1) * eb % kOrder) + 8u * (t & 1u);
     uint32_t bit = 0;                                  // lanes 0..7: x^(k i eb) x^(8 h + lane)
@@ -435,6 +428,7 @@ __global__ void __launch_bounds__(kPScanThreads, 1) prefix_scan_kernel(const uin
     reinterpret_cast<uint4*>(smem)[t * 32u + lane] = make_uint4(w0, w0 ^ p1, w0 ^ p2, w0 ^ p1 ^ p2);
   }
   __syncthreads();
+  grid_dependency_wait();                              // the blocks' signatures
   auto times = [&](uint64_t v, uint32_t f) -> uint64_t {
     const uint16_t* tab = reinterpret_cast<const uint16_t*>(smem) + f * 2048u;
     const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
@@ -453,8 +447,8 @@ __global__ void __launch_bounds__(kPScanThreads, 1) prefix_scan_kernel(const uin
     return shift_chunk_value((uint32_t)v & 0xFFFFu, (uint32_t)(v >> 16) & 0xFFFFu, (uint32_t)(v >> 32) & 0xFFFFu,
                              (uint32_t)(v >> 48), (uint32_t)(i % kOrder * eb % kOrder));
   };
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {   // warp-uniform
+  const uint64_t stride = (uint64_t)gridDim.x * kPRestThreads;
+  for (uint64_t i0 = 32 * prefix_warp(); i0 < n; i0 += stride) {   // warp-uniform
     const uint64_t i = i0 + lane;
     uint64_t p0 = 0, c = 0;
     if (i < n) {
@@ -497,8 +491,32 @@ __global__ void __launch_bounds__(kPScanThreads, 1) prefix_scan_kernel(const uin
   }
 }
 
-constexpr size_t kSmemPThread = (size_t)kRedBytes + 512 * 4 + 512 * 2;
-
-constexpr size_t kSmemPrefix = (size_t)kRedBytes + 512 * 4 + (size_t)kPConst * 512 * 2;
+// The second of the two launches of cumulative signatures, for whichever by_items
+// picks: the sums of the blocks' signatures, or all of the work.  It may start
+// while the signature kernel still runs, or has only begun to return (a
+// programmatic dependent launch): the sums wait for that kernel once their tables
+// are made, the others need nothing of it and only end after it.  One block of 1024
+// threads per SM for all three: the sums' tables take the shared memory, the other
+// two most registers.  Neighbouring warps are on different SMs, so that few keys
+// use them all.  (With three kernels one after the other, two of which returned at
+// once, 1000 keys of 32-100 bytes at blocks of 64 took 22.0 us a call, 11.0 now; 1000
+// of 200-2000 bytes at 256 24.4 and 17.1; 500k of 200-2000 bytes at 256 247 and 240.)
+static_assert((size_t)kRedBytes + 512 * 4 + (size_t)kPConst * 512 * 2 <= kSmemPScan, "prefix_by_warp's tables");
+__global__ void __launch_bounds__(kPRestThreads, 1) prefix_rest_kernel(const uint8_t* __restrict__ arena,
+                                                                    const uint64_t* __restrict__ off, uint64_t n,
+                                                                    uint32_t block_bytes,
+                                                                    const uint64_t* __restrict__ pref_off,
+                                                                    uint64_t* __restrict__ out) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ uint4 emask[17];
+  if (by_items(off, n, block_bytes)) {
+    if (pref_off[n] != n) prefix_sums(smem, off, n, block_bytes, pref_off, out);   // (else no key has two blocks)
+  } else if (block_bytes < 32) {
+    prefix_by_warp(smem, emask, arena, off, n, block_bytes, pref_off, out);
+  } else {
+    prefix_by_thread(smem, emask, arena, off, n, block_bytes, pref_off, out);
+  }
+  grid_dependency_wait();
+}
 
 }  // namespace algsig

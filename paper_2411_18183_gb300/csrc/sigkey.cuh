@@ -826,6 +826,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   constexpr bool BATCH = OF == LKOf::kBatchRows, ITEMS = OF == LKOf::kItems, CAPPED = OF == LKOf::kPrefixes;
   const uint64_t cap_len = CAPPED ? cap : ~0ull;
   if constexpr (ITEMS) {
+    asm volatile("griddepcontrol.launch_dependents;");   // prefix_rest_kernel, which waits where it has to
     if (!by_items(off, n, items.block)) return;
   }
   extern __shared__ __align__(128) uint8_t smem[];

@@ -1267,7 +1267,7 @@ static as_status ensure_device(DeviceState** out) {
     for (int i = 0; i < kSideStreams; ++i)
       if ((e = cudaStreamCreateWithFlags(&d.side[i], cudaStreamNonBlocking)) != cudaSuccess)
         return cuda_fail(e, "side stream");
-    if ((e = cudaFuncSetAttribute(prefix_rest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPScan)) !=
+    if ((e = cudaFuncSetAttribute(prefix_rest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPRest)) !=
         cudaSuccess)
       return cuda_fail(e, "kernel attribute");
     if ((e = cudaFuncSetAttribute(bl_hash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBHash)) !=
@@ -1580,7 +1580,7 @@ as_status as_sig_prefixes(const uint8_t* d_arena, const uint64_t* d_off, uint64_
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(want < (uint64_t)d->sms ? want : (uint64_t)d->sms));
   cfg.blockDim = dim3(kPRestThreads);
-  cfg.dynamicSmemBytes = kSmemPScan;
+  cfg.dynamicSmemBytes = kSmemPRest;
   cfg.stream = (cudaStream_t)stream;
   cfg.attrs = &early;
   cfg.numAttrs = 1;

@@ -393,26 +393,26 @@ __device__ __forceinline__ void prefix_by_thread(uint8_t* smem, uint4* emask, co
 // The cumulative signatures from those of the keys' blocks (the signature
 // kernel over items): C_j = sum_{i <= j} x^(k i B / 2) sig(block i), in place,
 // one thread per key; a key of more than 32 blocks is scanned by the warp.
-// The factor of block i = 16 q + l is applied as x^(k l B / 2) and x^(16 k q B / 2),
-// each by two tables of 256 entries (low and high byte) in shared memory that
-// every block makes for itself, for l < 16 and q < 32; the keys of more than 512
-// blocks go through the log / antilog tables.  What bounds it is the gathers:
-// through the log / antilog tables, eight per entry from 128 KB tables in L1, each
-// up to 32 lines, 500k keys of 200-2000 bytes at B = 256 took 50 us, 23 now
-// (whole call 290 -> 265 us; at B = 64 720 -> 565; three keys of 1.4 MB on average
-// at B = 256 780 -> 605).
-constexpr uint32_t kPScanLow = 16, kPScanHigh = 32;   // factors l and q: 0..15 and 0..31
-constexpr uint32_t kPScanTables = (kPScanLow - 1 + kPScanHigh - 1) * 8;
+// The factor x^(k i B / 2) of block i is applied digit by digit of i, three of
+// base 8, each by two tables of 256 entries (low and high byte) in shared memory
+// that every block makes for itself; the keys of more than 512 blocks go through the
+// log / antilog tables.  What bounds it is the gathers: through the log / antilog
+// tables, eight per entry from 128 KB tables in L1, each up to 32 lines, 500k keys
+// of 200-2000 bytes at B = 256 took 50 us, 23 with tables.  Two digits, of 16 and
+// 32, took 188 KB: the kernel's other two ways, which share its shared memory, were
+// then left with so little L1 that relations of short keys took up to 1.5 times as
+// long (500k keys of 160 bytes at B = 32 back to back 155 us, 93 with 86 KB).
+constexpr uint32_t kPScanTables = 3 * 7 * 8, kPScanBlocks = 512;
 constexpr size_t kSmemPScan = (size_t)kPScanTables * 512;
 __device__ __forceinline__ void prefix_sums(uint8_t* smem, const uint64_t* __restrict__ off, uint64_t n,
                                             uint32_t block_bytes, const uint64_t* __restrict__ pref_off,
                                             uint64_t* __restrict__ out) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t eb = (block_bytes / 2u) % kOrder;     // exponent from one block to the next
-  // table t = 8 f + 2 (k - 1) + h, f a factor (l - 1, then 15 + q - 1): its products with a byte at bits
+  // table t = 8 f + 2 (k - 1) + h, f a factor (block c 8^d: 7 d + c - 1): its products with a byte at bits
   // 8 h..8 h + 7; a lane makes the entries 8 lane..8 lane + 7 from the products with single bits
   for (uint32_t t = threadIdx.x >> 5; t < kPScanTables; t += kPRestThreads / 32) {
-    const uint32_t f = t >> 3, i = f < kPScanLow - 1 ? f + 1 : kPScanLow * (f - (kPScanLow - 2));
+    const uint32_t f = t >> 3, i = (f % 7 + 1) << (3 * (f / 7));
     const uint32_t e0 = (uint32_t)((uint64_t)i * (((t >> 1) & 3u) + 1) * eb % kOrder) + 8u * (t & 1u);
     uint32_t bit = 0;                                  // lanes 0..7: x^(k i eb) x^(8 h + lane)
     if (lane < 8u) bit = __ldg(&g_alog[(e0 + lane) % kOrder]);
@@ -438,9 +438,10 @@ __device__ __forceinline__ void prefix_sums(uint8_t* smem, const uint64_t* __res
     const uint32_t s4 = tab[1536u + (hi >> 16 & 0xFFu)] ^ tab[1792u + (hi >> 24)];
     return (uint64_t)(s1 | s2 << 16) | (uint64_t)(s3 | s4 << 16) << 32;
   };
-  auto moved = [&](uint64_t v, uint32_t i) -> uint64_t {     // block i's value in its place, i < 512
-    if (i & (kPScanLow - 1)) v = times(v, (i & (kPScanLow - 1)) - 1);
-    if (i / kPScanLow) v = times(v, kPScanLow - 2 + i / kPScanLow);
+  auto moved = [&](uint64_t v, uint32_t i) -> uint64_t {     // block i's value in its place, i < kPScanBlocks
+    if (i & 7u) v = times(v, (i & 7u) - 1);
+    if (i >> 3 & 7u) v = times(v, 7u + (i >> 3 & 7u) - 1);
+    if (i >> 6) v = times(v, 14u + (i >> 6) - 1);
     return v;
   };
   auto moved_far = [&](uint64_t v, uint64_t i) {
@@ -477,7 +478,7 @@ __device__ __forceinline__ void prefix_sums(uint8_t* smem, const uint64_t* __res
         const uint64_t j = b + lane;
         uint64_t v = next;
         next = j + 32 < cl ? out[pl + j + 32] : 0ull;
-        v = cl <= kPScanLow * kPScanHigh ? moved(v, (uint32_t)j) : moved_far(v, j);
+        v = cl <= kPScanBlocks ? moved(v, (uint32_t)j) : moved_far(v, j);
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
           const uint64_t t = __shfl_up_sync(0xFFFFFFFFu, v, d);
@@ -501,7 +502,8 @@ __device__ __forceinline__ void prefix_sums(uint8_t* smem, const uint64_t* __res
 // use them all.  (With three kernels one after the other, two of which returned at
 // once, 1000 keys of 32-100 bytes at blocks of 64 took 22.0 us a call, 11.0 now; 1000
 // of 200-2000 bytes at 256 24.4 and 17.1; 500k of 200-2000 bytes at 256 247 and 240.)
-static_assert((size_t)kRedBytes + 512 * 4 + (size_t)kPConst * 512 * 2 <= kSmemPScan, "prefix_by_warp's tables");
+constexpr size_t kSmemPWarp = (size_t)kRedBytes + 512 * 4 + (size_t)kPConst * 512 * 2;
+constexpr size_t kSmemPRest = kSmemPScan > kSmemPWarp ? kSmemPScan : kSmemPWarp;
 __global__ void __launch_bounds__(kPRestThreads, 1) prefix_rest_kernel(const uint8_t* __restrict__ arena,
                                                                     const uint64_t* __restrict__ off, uint64_t n,
                                                                     uint32_t block_bytes,

@@ -679,7 +679,7 @@ struct LKItems {
 // Whether a relation's cumulative signatures are computed by items (or by the
 // kernels of prefix.cuh, one key per thread or warp): a question of the mean key
 // length, which only the device knows, so both kernels are launched and one
-// returns at once.  An item costs the finish of a signature whatever its length,
+// and either kernel finds out.  An item costs the finish of a signature whatever its length,
 // a thread of its own follows a key at 90 instructions per 16 bytes and with
 // 16-byte loads.  us, items against the others, 500k keys of 200-2000 bytes (2M
 // of 32-128): blocks of 16 2043 / 1410 (735 / 1602), 32 1173 / 1295 (430 / 318),
@@ -826,8 +826,8 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   constexpr bool BATCH = OF == LKOf::kBatchRows, ITEMS = OF == LKOf::kItems, CAPPED = OF == LKOf::kPrefixes;
   const uint64_t cap_len = CAPPED ? cap : ~0ull;
   if constexpr (ITEMS) {
-    asm volatile("griddepcontrol.launch_dependents;");   // prefix_rest_kernel, which waits where it has to
     if (!by_items(off, n, items.block)) return;
+    asm volatile("griddepcontrol.launch_dependents;");   // prefix_rest_kernel, which waits where it has to
   }
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int kStages = kLKDepth / kLKStep;

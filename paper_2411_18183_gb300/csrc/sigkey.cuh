@@ -676,17 +676,36 @@ struct LKItems {
   uint32_t block = 0;
 };
 
-// Whether a relation's cumulative signatures are computed by items (or by the
-// kernels of prefix.cuh, one key per thread or warp): a question of the mean key
-// length, which only the device knows, so both kernels are launched and one
-// and either kernel finds out.  An item costs the finish of a signature whatever its length,
-// a thread of its own follows a key at 90 instructions per 16 bytes and with
-// 16-byte loads.  us, items against the others, 500k keys of 200-2000 bytes (2M
-// of 32-128): blocks of 16 2043 / 1410 (735 / 1602), 32 1173 / 1295 (430 / 318),
-// 64 724 / 956 (271 / 249), 256 299 / 669 (222 / 192), 4096 206 / 489.
+// Whether a relation's cumulative signatures are computed by items (or one key
+// per thread or warp, prefix.cuh): a question of the keys' lengths, which only the
+// device knows.  An item costs the finish of a signature whatever its length; a
+// thread of its own follows a key at 90 instructions per 16 bytes, and a warp's 32
+// take as long as their longest.  So what counts is the longest of neighbouring
+// keys: the mean of that over four places of eight keys each, the same for every
+// warp of both kernels.  (By the mean length alone, from 128 bytes on, equal keys
+// of 130-200 bytes took up to 1.4 times as long as with a thread each, and mixed
+// ones of which a tenth are long half the speed they could have.)
+// us, items / a thread per key, 500k keys at blocks of 32, 64, 256:
+//   equal, 130 bytes    113 / 91     74 / 59     40 / 34
+//   equal, 190 bytes    138 / 133    78 / 77     44 / 46
+//   65-195 bytes        110 / 107    69 / 78     39 / 43
+//   130-390 bytes       201 / 239   115 / 167    66 / 107
+//   48, a tenth 528     101 / 176    62 / 129    47 / 99
+// With one key or less per thread of the device the threads' latency is all that
+// counts (60k equal keys of 190 bytes 28 / 25, 21 / 18, 12 / 13; of 400 bytes 46 / 44,
+// 30 / 30, 21 / 21), but for so few that they do not fill it either.
+// A warp per key (blocks of 16): 500k of 190 bytes 260 / 299, of 260 404 / 350; 16k of
+// 96 bytes 19 / 17, 60k 27 / 40.
 __device__ __forceinline__ bool by_items(const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
-  const uint64_t bytes = __ldg(off + n) - __ldg(off);
-  return block < 32u ? bytes < 192u * n : bytes >= (block < 64u ? 256u : 128u) * n;
+  if (block < 32u) return n > 20000u && __ldg(off + n) - __ldg(off) < 192u * n;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t first = n / 8 * (2 * (lane >> 3) + 1), i = min(first / 8 * 8 + (lane & 7u), n - 1);
+  const uint64_t len = __ldg(off + i + 1) - __ldg(off + i);
+  uint32_t longest = (uint32_t)min(len, (uint64_t)0x10000000u);
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) longest = max(longest, __shfl_xor_sync(kFull, longest, d));
+  longest = __reduce_add_sync(kFull, longest >> 3) >> 2;         // each place's eight times
+  return longest >= (n >= (1u << 15) && n <= 5u << 15 ? 280u : 180u);
 }
 
 // A warp's items [lo, hi), whole groups of 32 but at the end, and a key at or

@@ -17,7 +17,8 @@
 // block leaves a factor x^(k a), taken off in the logarithm.
 //
 // 1M keys of 200-2000 bytes (1.1 GB): 1676 us with one thread per key and four
-// bytes per table step, 215 us in this form (5.1 TB/s).
+// bytes per table step, 215 us in this form (5.1 TB/s).  Relations of short keys
+// still take a thread per key (by_thread).
 #pragma once
 #include <cstdint>
 
@@ -54,12 +55,74 @@ __device__ __forceinline__ uint32_t red8_16(uint32_t u, const Cursor& c) {
   return u ^ c.load(tab_index(u, c.off16, kSel8));
 }
 
+// Horner's rule on four bytes (b0 lowest) for all four components: a_k x^(4k) +
+// b3 x^(3k) + b2 x^(2k) + b1 x^k + b0, at most 8 + 4 k bits before the reduction
+template <class Cursor>
+__device__ __forceinline__ void gf8_word(uint32_t w, uint32_t (&a)[4], const Cursor& rc) {
+  const uint32_t b0 = w & 0xFFu, b1 = (w >> 8) & 0xFFu, b2 = (w >> 16) & 0xFFu, b3 = w >> 24;
+  a[0] = red8_16((a[0] << 4) ^ (b3 << 3) ^ (b2 << 2) ^ (b1 << 1) ^ b0, rc);
+  a[1] = red8_16((a[1] << 8) ^ (b3 << 6) ^ (b2 << 4) ^ (b1 << 2) ^ b0, rc);
+  a[2] = red8_24((a[2] << 12) ^ (b3 << 9) ^ (b2 << 6) ^ (b1 << 3) ^ b0, rc);
+  a[3] = red8_24((a[3] << 16) ^ (b3 << 12) ^ (b2 << 8) ^ (b1 << 4) ^ b0, rc);
+}
+
 struct Net8 {
+  // Short keys, of which the signature kernel's work per key is more than a thread's work per byte: us, one key
+  // per thread / staged, 4M keys of 16, 32, 48, 64 bytes 68 / 155, 97 / 155, 129 / 157, 161 / 157; half to one
+  // and a half times 32, 40, 48 bytes 156 / 160, 177 / 160, 203 / 161.  Up to a key or so per thread of the device
+  // both are bound by the launch.
+  static constexpr uint64_t kThreadFrom = 100000;
+  static constexpr uint32_t kThreadBelow = 50;
   static constexpr int kPhases = 6;       // the rings of 24 and 16 words close together
   static constexpr int kShort = 0;
   static constexpr size_t kTabBytes = kLog8Bytes;
   __device__ __forceinline__ static const uint2* red_image() { return g_red8; }
   __device__ __forceinline__ static const uint4* tab_image() { return g_log8; }
+  // One key per thread: Horner's rule over the words of its bytes (realigned to its first one) from the last
+  // to the first, 16 bytes of memory at a time.  The next key's last 16 bytes and the offsets of the one
+  // after it are on their way meanwhile.  mt: lk_fill_masks' rows.
+  template <class Cursor>
+  __device__ __forceinline__ static void by_thread(const uint8_t* __restrict__ arena, const uint64_t* __restrict__ off,
+                                                   uint64_t n, uint64_t* __restrict__ out, const uint4* mt,
+                                                   const Cursor& rc) {
+    struct Key {
+      uint64_t s, e;
+    };
+    auto key = [&](uint64_t i) { return i < n ? Key{__ldg(off + i), __ldg(off + i + 1)} : Key{0, 0}; };
+    auto chunk = [&](uint64_t at) { return __ldg(reinterpret_cast<const uint4*>(arena + at)); };
+    auto last = [&](const Key& k) { return k.e > k.s ? chunk((k.e - 1) & ~15ull) : make_uint4(0, 0, 0, 0); };
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    Key k = key(i), k1 = key(i + stride);
+    uint4 w = last(k);
+    for (; i < n; i += stride) {
+      const Key k2 = key(i + 2 * stride);
+      const uint4 w1 = last(k1);
+      uint32_t a[4] = {0, 0, 0, 0};
+      if (k.e > k.s) {
+        const uint32_t sh = 8u * ((uint32_t)k.s & 3u), w0 = ((uint32_t)k.s & 15u) >> 2;
+        const uint4 m = mt[(((uint32_t)k.e - 1u) & 15u) + 1u];
+        w.x &= m.x; w.y &= m.y; w.z &= m.z; w.w &= m.w;
+        uint32_t above = 0;                            // the first word of the chunk above
+        for (uint64_t at = (k.e - 1) & ~15ull;; at -= 16) {
+          const bool first = at <= k.s;
+          const uint4 below = first ? w : chunk(at - 16);
+          const uint32_t from = first ? w0 : 0u;       // the first chunk's words from the key's first byte on
+          gf8_word(__funnelshift_r(w.w, above, sh), a, rc);
+          if (from <= 2u) gf8_word(__funnelshift_r(w.z, w.w, sh), a, rc);
+          if (from <= 1u) gf8_word(__funnelshift_r(w.y, w.z, sh), a, rc);
+          if (from == 0u) gf8_word(__funnelshift_r(w.x, w.y, sh), a, rc);
+          if (first) break;
+          above = w.x;
+          w = below;
+        }
+      }
+      out[i] = (uint64_t)(a[0] | (a[1] << 8) | (a[2] << 16) | (a[3] << 24));
+      k = k1;
+      k1 = k2;
+      w = w1;
+    }
+  }
   uint32_t p[24];                         // digits of the division by x^21 + x^10 + 1
   uint32_t q[16];                         // digits of the division by x^11 + x^5 + 1
   __device__ __forceinline__ void clear() {

@@ -223,6 +223,18 @@ __device__ __forceinline__ uint32_t xs3_component(const uint32_t (&c3)[16], cons
   return red32(acc, rc);
 }
 
+// The longest of eight neighbouring keys, the mean of that over four places of the
+// relation, to 8 bytes (whole warp): what a thread per key waits for.
+__device__ __forceinline__ uint32_t lk_longest_near(const uint64_t* __restrict__ off, uint64_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t first = n / 8 * (2 * (lane >> 3) + 1), i = min(first / 8 * 8 + (lane & 7u), n - 1);
+  const uint64_t len = __ldg(off + i + 1) - __ldg(off + i);
+  uint32_t longest = (uint32_t)min(len, (uint64_t)0x10000000u);
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) longest = max(longest, __shfl_xor_sync(kFull, longest, d));
+  return __reduce_add_sync(kFull, longest >> 3) >> 2;            // each place's eight times
+}
+
 // A lane's key in the current group.
 struct LKKey {
   uint64_t kq;          // key index
@@ -479,11 +491,13 @@ __device__ __forceinline__ void lk_short_blocks(uint32_t (&st)[kLKState], const 
 // What the kernel computes: signatures over GF(2^16) with two or four
 // components.  A net names its shared-memory tables and has the digit rings and
 // finish of the quotient form; kShort: groups of at most this many blocks take
-// the remainder form.
+// the remainder form; kThreadBelow: relations of more than kThreadFrom keys shorter
+// than this (lk_longest_near) are signed by Net::by_thread, one key per thread.
 template <int NCOMP>
 struct Net16 : QNet<NCOMP> {
   static constexpr int kComponents = NCOMP;
   static constexpr int kShort = kLKShort;
+  static constexpr uint32_t kThreadBelow = 0;         // (no way with a thread per key)
   static constexpr size_t kTabBytes = 4 * kInvEntries;
   __device__ __forceinline__ static const uint2* red_image() { return g_red16; }
   __device__ __forceinline__ static const uint4* tab_image() { return g_inv; }
@@ -681,8 +695,7 @@ struct LKItems {
 // device knows.  An item costs the finish of a signature whatever its length; a
 // thread of its own follows a key at 90 instructions per 16 bytes, and a warp's 32
 // take as long as their longest.  So what counts is the longest of neighbouring
-// keys: the mean of that over four places of eight keys each, the same for every
-// warp of both kernels.  (By the mean length alone, from 128 bytes on, equal keys
+// keys, the same for every warp of both kernels.  (By the mean length alone, from 128 bytes on, equal keys
 // of 130-200 bytes took up to 1.4 times as long as with a thread each, and mixed
 // ones of which a tenth are long half the speed they could have.)
 // us, items / a thread per key, 500k keys at blocks of 32, 64, 256:
@@ -698,14 +711,7 @@ struct LKItems {
 // 96 bytes 19 / 17, 60k 27 / 40.
 __device__ __forceinline__ bool by_items(const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
   if (block < 32u) return n > 20000u && __ldg(off + n) - __ldg(off) < 192u * n;
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t first = n / 8 * (2 * (lane >> 3) + 1), i = min(first / 8 * 8 + (lane & 7u), n - 1);
-  const uint64_t len = __ldg(off + i + 1) - __ldg(off + i);
-  uint32_t longest = (uint32_t)min(len, (uint64_t)0x10000000u);
-#pragma unroll
-  for (int d = 1; d < 8; d <<= 1) longest = max(longest, __shfl_xor_sync(kFull, longest, d));
-  longest = __reduce_add_sync(kFull, longest >> 3) >> 2;         // each place's eight times
-  return longest >= (n >= (1u << 15) && n <= 5u << 15 ? 280u : 180u);
+  return lk_longest_near(off, n) >= (n >= (1u << 15) && n <= 5u << 15 ? 280u : 180u);
 }
 
 // A warp's items [lo, hi), whole groups of 32 but at the end, and a key at or
@@ -886,6 +892,8 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     else
       lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
   }
+  bool by_thread = false;
+  if constexpr (Net::kThreadBelow > 0) by_thread = n > Net::kThreadFrom && lk_longest_near(off, n) < Net::kThreadBelow;
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, most, &wa) : 0u;
   if (wn && !ITEMS) lk_prefetch_window(W, off, wa, wa + wn);
@@ -901,8 +909,15 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     for (int j = 0; j < 4; ++j) line[j] = make_uint4(v, v, v, v);
   }
   __syncthreads();
-  if (k_lo >= k_hi) return;
   const LKCursor<AT400> rc(smem);
+  if constexpr (Net::kThreadBelow > 0) {
+    if (by_thread) {
+      cp_async_wait_all();
+      Net::by_thread(arena, off, n, sig_out, mt, rc);
+      return;
+    }
+  }
+  if (k_lo >= k_hi) return;
 
   uint8_t* stages = smem + lk_stage_base<kStages>((uint32_t)wib);
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(stages);

@@ -115,6 +115,11 @@ constexpr int kLKState = 40;                          // state registers of a ke
 // groups of at most this many blocks take lk_short_blocks (at most one step; 4M keys of 32-128 bytes:
 // 201, 199, 193 and 197 us with 0, 2, 3 and 4)
 constexpr int kLKShort = 3;
+// and windows whose keys all have at most as many are not sorted: a group's blocks beyond a key's own cost less
+// than the sort, whose counters few bins share (us, 4M keys, two components, sorted / not: empty 95 / 81, 0-6 bytes
+// 103 / 93, 12-36 108 / 99, equal ones of 64 104 / 89).  Asked of windows of kLKAsk bytes a key at most, and by the
+// block length of items.
+constexpr uint32_t kLKUnsorted = kLKShort, kLKAsk = 64;
 
 // Shared memory: 256-byte lines of two halves.  The lower halves of the first
 // 256 lines hold the reduction tables (16 copies of each entry).  A warp's
@@ -265,6 +270,13 @@ __device__ __forceinline__ uint32_t lk_blocks(uintptr_t abs, uint64_t len) {
   return nb < 0xFFFFFFFFull ? (uint32_t)nb : 0xFFFFFFFFu;
 }
 
+// the window's entries as they come
+__device__ __forceinline__ void lk_in_order(LKWarp& W) {
+  const uint32_t lane = threadIdx.x & 31u, e = 0x08080808u * lane;
+  reinterpret_cast<uint2*>(W.order)[lane] = make_uint2(0x03020100u + e, 0x07060504u + e);
+  __syncwarp();
+}
+
 // order the window's entries by block count: a counting sort over the block
 // counts (255 and more share the last bin; the order within a bin is
 // arbitrary), so that each group of 32 consecutive entries has keys of
@@ -272,13 +284,27 @@ __device__ __forceinline__ uint32_t lk_blocks(uintptr_t abs, uint64_t len) {
 // the bins' counts.  (Short keys are bound by shared-memory wavefronts, 76 % of
 // the peak for 4M keys of 32-128 bytes: with the bins moved eight words at a time
 // and lk_copy_setup's rows in different banks that call takes 181 us, 197 before.)
+template <bool ASK>
 __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_t wn, uintptr_t arena,
                                                uint64_t cap_len) {
   const uint32_t lane = threadIdx.x & 31u;
   if (wn <= 32) {                                    // one group: nothing to balance
-    W.order[lane] = (uint8_t)lane;
-    __syncwarp();
+    lk_in_order(W);
     return;
+  }
+  constexpr int kPer = kLKWin / 32;                   // entries per lane
+  auto blocks = [&](uint32_t i) -> uint32_t {
+    const uint64_t ks = W.woff[i];
+    return lk_blocks(arena + ks, min(W.woff[i + 1] - ks, cap_len));
+  };
+  if (ASK && min(W.woff[wn] - W.woff[0], cap_len * wn) <= kLKAsk * wn) {
+    uint32_t most = 0;
+#pragma unroll 1
+    for (uint32_t i = lane; i < wn; i += 32) most = max(most, blocks(i));
+    if (__reduce_max_sync(kFull, most) <= kLKUnsorted) {
+      lk_in_order(W);
+      return;
+    }
   }
   auto count = [&](uint32_t b) -> uint32_t& {
     return reinterpret_cast<uint32_t*>(rows + (b >> 5) * kLKPitch)[b & 31u];
@@ -286,7 +312,6 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
   uint4* mine = reinterpret_cast<uint4*>(&count(8 * lane));   // the lane's 8 consecutive bins
   mine[0] = mine[1] = make_uint4(0, 0, 0, 0);
   __syncwarp();
-  constexpr int kPer = kLKWin / 32;                   // entries per lane
   uint32_t bin[kPer], rank[kPer];
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
@@ -294,9 +319,7 @@ __device__ __forceinline__ void lk_sort_window(LKWarp& W, uint8_t* rows, uint32_
     bin[j] = 0;
     rank[j] = 0;
     if (i < wn) {
-      const uint64_t ks = W.woff[i], len = min(W.woff[i + 1] - ks, cap_len);
-      const uint32_t nb = lk_blocks(arena + ks, len);
-      bin[j] = nb < 255u ? nb : 255u;
+      bin[j] = min(blocks(i), 255u);
       rank[j] = atomicAdd(&count(bin[j]), 1u);
     }
   }
@@ -943,7 +966,10 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
         wn = kLKNarrowWin;
         ng = kLKNarrowWin / 32;
       }
-      lk_sort_window(W, stages, wn, reinterpret_cast<uintptr_t>(arena), cap_len);
+      if (ITEMS && items.block <= 32u * (kLKUnsorted - 1u))
+        lk_in_order(W);
+      else
+        lk_sort_window<!ITEMS>(W, stages, wn, reinterpret_cast<uintptr_t>(arena), cap_len);
     }
     const uint32_t G2 = lk_load_group(k2, W, wb, wn, g, arena, cap_len);
     if (++g == ng) {                                  // the window's offsets are free: fetch the next ones

@@ -85,7 +85,9 @@ class GraphBatch:
 class TuneCache:
     """Best (load factor, signature kernel shape) found by autotune, keyed by
     (GPU name, key-length class, size class) so that batches of the same shape
-    skip the timing.  Optionally persisted as JSON."""
+    skip the timing.  Optionally persisted as JSON, in which a shape is its warps
+    and depth: a shape's index says nothing to a library with other shapes, and an
+    entry whose shape the library does not have is timed anew."""
 
     LENGTH_CLASSES = (128, 1024, 8192)          # upper bounds of the key-length bands, then longer
 
@@ -97,9 +99,24 @@ class TuneCache:
             import os
             if os.path.exists(path):
                 with open(path) as f:
+                    shapes = self._shapes()
                     for k, v in json.load(f).items():
-                        # an entry is [load_factor, shape]; a bare number is a load factor at shape 0
-                        self.table[k] = (float(v[0]), int(v[1])) if isinstance(v, list) else (float(v), 0)
+                        # an entry is [load_factor, shape, [warps, depth] of the shape]; a bare number is a load
+                        # factor at shape 0, the default of every library
+                        if not isinstance(v, list):
+                            self.table[k] = (float(v), 0)
+                        elif len(v) == 3 and shapes and v[2] in shapes:
+                            self.table[k] = (float(v[0]), shapes.index(v[2]))
+                        elif len(v) == 3 and v[2] is None and shapes is None:
+                            self.table[k] = (float(v[0]), int(v[1]))
+
+    @staticmethod
+    def _shapes():
+        """The library's shapes as [warps, depth] lists, None where it is not built."""
+        try:
+            return [list(s) for s in sig_shapes()]
+        except (RuntimeError, OSError):
+            return None
 
     @classmethod
     def key(cls, device_name: str, mean_key_bytes: float, rows: int) -> str:
@@ -115,8 +132,10 @@ class TuneCache:
         self.table[key] = (float(load_factor), int(shape))
         if self.path:
             import json
+            shapes = self._shapes()
             with open(self.path, "w") as f:
-                json.dump({k: list(v) for k, v in self.table.items()}, f, indent=1, sort_keys=True)
+                json.dump({k: [lf, sh, shapes[sh] if shapes and sh < len(shapes) else None]
+                           for k, (lf, sh) in self.table.items()}, f, indent=1, sort_keys=True)
 
 
 def batch_shape_key(R: DeviceRelation, S: DeviceRelation, ranges) -> str:

@@ -535,8 +535,8 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
   if (tail) {
     const uint32_t off = (nfull - li) << 4;
     ts = ld16_stream(pS + off);
-    if ((nfull << 4) + 16u > sa + d) ta = ld16(pR + off);
-    if (16u < rem + d) tb = ld16(pR + off + 16);
+    if (r_low_partial(nfull, sa, d)) ta = ld16(pR + off);
+    if (r_high_partial(rem, d)) tb = ld16(pR + off + 16);
   }
   const uint32_t nmax = __reduce_max_sync(kFull, nfull);
   // one trip: the chunks from c0 on that the lanes have in flight
@@ -548,8 +548,8 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
       sv[u] = ra[u] = rb[u] = make_uint4(0, 0, 0, 0);
       if (ci < nfull) {
         sv[u] = ld16_stream(pS);
-        if (ci > 0u || sa + d < 16u) ra[u] = ld16(pR);
-        if (ci + 1u < nfull || rem + d > 0u) rb[u] = ld16(pR + 16);
+        if (r_low(ci, sa, d)) ra[u] = ld16(pR);
+        if (r_high(ci, nfull, rem, d)) rb[u] = ld16(pR + 16);
       }
       pS += 16u << lg;
       pR += 16u << lg;
@@ -676,7 +676,7 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
       const uint32_t d = (uint32_t)(reinterpret_cast<uintptr_t>(pR) - sa) & 15u;
       const uint64_t bS = reinterpret_cast<uint64_t>(pS - sa), bR = reinterpret_cast<uint64_t>(pR - sa - d);
       q[lane].a = make_uint4((uint32_t)bS, (uint32_t)(bS >> 32), (uint32_t)bR, (uint32_t)(bR >> 32));
-      q[lane].b = make_uint4(sa + l32, sa | (d << 8), row, tag);
+      q[lane].b = make_uint4(narrow_end(sa, l32), sa | (d << 8), row, tag);
     }
     __syncwarp();
   }

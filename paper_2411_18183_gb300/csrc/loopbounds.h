@@ -1,12 +1,13 @@
-// loopbounds.h -- loop bounds of the warp-wide byte comparison (the exact
-// verification of every candidate pair that makes the join exact) and of the
-// signature kernel's copies, shared by the device code and a host-compiled
-// check of the bounds.
+// loopbounds.h -- loop bounds of the byte comparisons (the exact verification of
+// every candidate pair that makes the join exact) and of the signature kernel's
+// copies, shared by the device code and host-compiled checks of the bounds.
 //
-// The comparison of two len-byte keys runs in 32-bit offsets from the aligned
-// 16-byte chunk that holds the S key's first byte (that byte at offset
-// sa < 16); the R key's bytes sit d < 16 bytes further.  One step compares
-// 1024 bytes, and every offset a step forms stays below
+// A comparison of two len-byte keys counts in 32 bits from the aligned 16-byte
+// chunk that holds the S key's first byte (that byte at offset sa < 16); the R
+// key's bytes sit d < 16 bytes further.  The probe's (compare_some) goes by chunks:
+// S chunk c against the R bytes [16 c + d, 16 c + d + 16), from the R chunks c and
+// c + 1.  The comparison join's (warp_equal) takes steps of 1024 bytes, and every
+// offset a step forms stays below
 //     steps * 1024 + d + 16  <=  sa + len + 1023 + 15 + 16,
 // which is below 2^32 for every len < kNarrowLen.  Longer keys are compared
 // in 64-bit offsets.  The loop is counted in steps, so it ends by
@@ -34,6 +35,16 @@ ALGSIG_HD uint32_t narrow_steps(uint32_t sa, uint32_t len) { return (uint32_t)((
 ALGSIG_HD uint64_t narrow_offset_end(uint32_t sa, uint32_t len, uint32_t d) {
   return (uint64_t)narrow_steps(sa, len) * 1024u + d + 16u;
 }
+
+// Chunks of the probe's comparison of keys of len < kNarrowLen bytes: the S key
+// ends at byte `end`, after nfull whole chunks and rem bytes of another.
+ALGSIG_HD uint32_t narrow_end(uint32_t sa, uint32_t len) { return sa + len; }
+// which of the two R chunks under whole S chunk c (below nfull), and under the
+// partial one (rem > 0), hold a byte of the R key
+ALGSIG_HD bool r_low(uint32_t c, uint32_t sa, uint32_t d) { return c > 0u || sa + d < 16u; }
+ALGSIG_HD bool r_high(uint32_t c, uint32_t nfull, uint32_t rem, uint32_t d) { return c + 1u < nfull || rem + d > 0u; }
+ALGSIG_HD bool r_low_partial(uint32_t nfull, uint32_t sa, uint32_t d) { return (nfull << 4) + 16u > sa + d; }
+ALGSIG_HD bool r_high_partial(uint32_t rem, uint32_t d) { return 16u < rem + d; }
 
 // Where a key of len > 0 bytes ends in the signature kernel's blocks of 32
 // bytes (four to a step, two 16-byte chunks each), its first byte being byte

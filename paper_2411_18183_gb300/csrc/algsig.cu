@@ -32,12 +32,10 @@ namespace algsig {
 // GF(2^16) logarithm / antilogarithm of x, set up once per device.
 __device__ uint16_t g_log[65536];
 __device__ uint16_t g_alog[65536];
-// constant-multiply tables of the tile combination (rounds.cuh), set up once per device
-__device__ uint16_t g_const[17 * 512];
+__device__ __align__(16) uint16_t g_inv32[512];   // multiplication by x^-32 (lo_correct_inv), set up once per device
 }  // namespace algsig
 
 #include "rounds.cuh"
-static_assert(algsig::kConstEntries == 17 * 512, "g_const holds the combination tables");
 #include "baseline.cuh"
 
 namespace algsig {
@@ -1168,27 +1166,19 @@ static as_status ensure_device(DeviceState** out) {
     h_log[0] = 0;
     if ((e = cudaMemcpyToSymbol(g_log, h_log, sizeof(h_log))) != cudaSuccess) return cuda_fail(e, "table setup");
     if ((e = cudaMemcpyToSymbol(g_alog, h_alog, sizeof(h_alog))) != cudaSuccess) return cuda_fail(e, "table setup");
-    // constant-multiply tables: c_k^(2^s) = x^(k kTile/2 2^s) at (k-1)*kScanLevels+s, then x^-32
-    static uint16_t h_const[kConstEntries];
     auto mul = [&](uint32_t a, uint32_t b) -> uint32_t {
       if (a == 0 || b == 0) return 0;
       return h_alog[((uint32_t)h_log[a] + (uint32_t)h_log[b]) % kOrder];
     };
-    for (int t = 0; t < kConstCount; t++) {
-      uint64_t ex;
-      if (t < 4 * kScanLevels) {
-        const int k = t / kScanLevels + 1, sh = t % kScanLevels;
-        ex = ((uint64_t)k * (kTile / 2) << sh) % kOrder;
-      } else {
-        ex = kOrder - 32;
-      }
-      const uint32_t C = h_alog[ex];
+    {  // multiplication by x^-32
+      uint16_t h_inv32[512];
+      const uint32_t C = h_alog[kOrder - 32];
       for (uint32_t b = 0; b < 256; b++) {
-        h_const[t * 512 + b] = (uint16_t)mul(b, C);
-        h_const[t * 512 + 256 + b] = (uint16_t)mul(mul(b, h_alog[8]), C);
+        h_inv32[b] = (uint16_t)mul(b, C);
+        h_inv32[256 + b] = (uint16_t)mul(mul(b, h_alog[8]), C);
       }
+      if ((e = cudaMemcpyToSymbol(g_inv32, h_inv32, sizeof(h_inv32))) != cudaSuccess) return cuda_fail(e, "table setup");
     }
-    if ((e = cudaMemcpyToSymbol(g_const, h_const, sizeof(h_const))) != cudaSuccess) return cuda_fail(e, "table setup");
     {  // the signature kernel's constant-multiply tables (quotient.cuh)
       static uint16_t h_inv[2 * kInvEntries];
       for (int t = 0; t < 2 * kInvTables; t++) {

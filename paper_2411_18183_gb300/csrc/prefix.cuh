@@ -36,7 +36,7 @@ constexpr int kPRestThreads = 1024;     // and of prefix_rest_kernel
 constexpr int kPLevels = 5;             // scan levels over 32 lanes
 constexpr int kPConst = 4 * kPLevels;   // tables x^(-8 k 2^s), k = 1..4, s = 0..4, at (k-1)*kPLevels+s
 // multiply-by-constant tables of the prefix scan (layout of rounds.cuh's), set up once per device
-__device__ uint16_t g_pconst[kPConst * 512];
+__device__ __align__(16) uint16_t g_pconst[kPConst * 512];
 
 // the warp's number in prefix_rest_kernel: neighbouring ones on different SMs, so that few keys use them all
 __device__ __forceinline__ uint64_t prefix_warp() { return (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
@@ -339,7 +339,7 @@ __device__ __forceinline__ void prefix_by_thread(uint8_t* smem, uint4* emask, co
   uint32_t* red = reinterpret_cast<uint32_t*>(smem);
   uint16_t* inv32 = reinterpret_cast<uint16_t*>(smem + kRedBytes + 512 * 4);
   for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    reinterpret_cast<uint32_t*>(inv32)[i] = reinterpret_cast<const uint32_t*>(g_const + 4 * kScanLevels * 512)[i];
+    reinterpret_cast<uint32_t*>(inv32)[i] = reinterpret_cast<const uint32_t*>(g_inv32)[i];
   fill_emask(emask);
   init_red_tables(red, red + kRedWords);                     // ends with __syncthreads()
   const RedCursor rc = red_cursor(red);

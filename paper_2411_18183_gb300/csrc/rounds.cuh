@@ -1,8 +1,8 @@
 // rounds.cuh -- warp-level helpers shared by the kernels: async copies, the
 // split of a relation's keys over warps in equal shares of key bytes (+ an
 // optional cost per key; a 32-ary search in the offsets by one warp), the
-// offsets a warp loads for a round of 32 keys, and the constant-multiply tables
-// of the cumulative signatures' tiles of kTile bytes.
+// offsets a warp loads for a round of 32 keys, and multiplication by constants
+// through tables of two byte-indexed halves.
 #pragma once
 #include <cstdint>
 
@@ -10,11 +10,6 @@
 
 namespace algsig {
 
-#ifndef ALGSIG_TILE_CHUNKS
-#define ALGSIG_TILE_CHUNKS 16
-#endif
-constexpr int kTileChunks = ALGSIG_TILE_CHUNKS;       // 16-byte chunks per tile
-constexpr int kTile = 16 * kTileChunks;               // bytes of realigned key per tile
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 
 // g_log / g_alog: GF(2^16) logarithm / antilogarithm of x, defined (and set
@@ -103,14 +98,6 @@ __device__ __forceinline__ PlanLoad plan_load(const uint64_t* __restrict__ off, 
   }
   return l;
 }
-
-// Constant-multiply tables (512 entries each, two byte-indexed halves), set up
-// once per device in g_const: c_k^(2^s) = x^(k kTile/2 2^s) for k = 1..4 and
-// s = 0..3 (the cumulative-signature scans), then x^-32.
-constexpr int kConstCount = 17;                       // 16 scan constants (s = 0..3) + x^-32
-constexpr int kScanLevels = 4;                         // c_k^(2^s) tables kept for s < kScanLevels
-constexpr int kConstEntries = kConstCount * 512;
-constexpr int kConstBytes = kConstEntries * 2;
 
 // multiply by the constant whose table starts at `tab`
 __device__ __forceinline__ uint32_t mulc(const uint16_t* tab, uint32_t v) {

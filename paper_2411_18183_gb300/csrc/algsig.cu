@@ -510,14 +510,15 @@ __device__ __forceinline__ uint4 chunk_diff(const uint4& sv, const uint4& ra, co
 // of a candidate's lanes takes the 16-byte S chunks i, i + 2^lg, ... and the two
 // aligned R chunks under each, kVAhead at a time; the last chunk, where it is
 // partial, is compared apart.  Only aligned chunks that hold a key byte are read.
-// A candidate of the whole warp's is left at its first 1 KB if that differs
-// (signatures collide where a caller gives its own, or two components), then every
-// 4 KB (PIECES, up to 10 KB not again) or every 1 KB; those of eight lanes, 1.5 KB
-// at most, are read to their ends.  (20k candidates of 32 KB that differ in their first
-// KB: 707 us read to the end, 60 now; 100k of 2 KB 105 and 75.  Equal keys of 2-8 KB
-// take 784 us read to the end, 781 with PIECES and 795 left every 1 KB; in the
-// kernel of the output modes PIECES spills, 310 against 290 us for 1-2 KB.)
-template <uint32_t lg, bool PIECES>
+// A candidate of the whole warp's is left after its first 1 KB if that differs
+// (signatures collide where a caller gives its own, or two components), later one
+// trip after the difference, the question being asked while the next chunks are
+// on their way; those of eight lanes, 1.5 KB at most, are read to their ends.  (20k
+// candidates of 32 KB that differ in their first KB: 723 us read to the end, 60 now;
+// 100k of 2 KB 101 and 74.  Equal keys of 2-8 KB 773 and 776 us, of 32 KB 723 and 736;
+// with the question after every trip 783 and 744, with whole pieces of 4 KB between
+// two questions 768 and 756.)
+template <uint32_t lg>
 __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint32_t todo,
                                                  const uint4* __restrict__ emask) {
   const uint32_t lane = threadIdx.x & 31u, li = lane & ((1u << lg) - 1u), c = r + (lane >> lg);
@@ -537,8 +538,9 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
     if (r_high_partial(rem, d)) tb = ld16(pR + off + 16);
   }
   const uint32_t nmax = __reduce_max_sync(kFull, nfull);
-  // one trip: the chunks from c0 on that the lanes have in flight
-  auto trip = [&](uint32_t c0) {
+  // one trip: the chunks from c0 on that the lanes have in flight; ask: false, and nothing compared, if one of
+  // the trips before has found a difference (asked while the chunks are on their way)
+  auto trip = [&](uint32_t c0, auto ask) -> bool {
     uint4 sv[kVAhead], ra[kVAhead], rb[kVAhead];
 #pragma unroll
     for (int u = 0; u < kVAhead; ++u) {
@@ -552,6 +554,7 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
       pS += 16u << lg;
       pR += 16u << lg;
     }
+    if (ask.value && __any_sync(kFull, diff != 0u)) return false;
 #pragma unroll
     for (int u = 0; u < kVAhead; ++u) {
       uint4 x = chunk_diff(sv[u], ra[u], rb[u], d);
@@ -561,30 +564,18 @@ __device__ __forceinline__ uint32_t compare_some(const Cand* q, uint32_t r, uint
       }
       diff |= (x.x | x.y) | (x.z | x.w);
     }
+    return true;
   };
   constexpr uint32_t kTrip = (uint32_t)kVAhead << lg;  // (all bounds below are warp-uniform)
   auto trips = [&](uint32_t c0, uint32_t end) {
-    for (; c0 < end; c0 += kTrip) trip(c0);
+    for (; c0 < end; c0 += kTrip) trip(c0, std::false_type());
   };
   if constexpr (lg < 5u) {
     trips(0u, nmax);
-  } else if constexpr (!PIECES) {
-    for (uint32_t c0 = 0; c0 < nmax; c0 += kTrip) {
-      trip(c0);
-      if (__any_sync(kFull, diff != 0u)) break;
-    }
   } else {
     trips(0u, min(kTrip, nmax));
     if (nmax > kTrip && !__any_sync(kFull, diff != 0u)) {
-      if (nmax <= 640u) {
-        trips(kTrip, nmax);
-      } else {
-        uint32_t c0 = kTrip;
-#pragma unroll 1
-        do {
-          trips(c0, min(c0 + 256u, nmax));
-          c0 += 256u;
-        } while (c0 < nmax && !__any_sync(kFull, diff != 0u));
+      for (uint32_t c0 = kTrip; c0 < nmax && trip(c0, std::true_type()); c0 += kTrip) {
       }
     }
   }
@@ -679,8 +670,8 @@ __device__ __forceinline__ bool queue_verify(Cand* q, uint64_t* ids, uint32_t nc
     __syncwarp();
   }
   uint32_t r = 0;
-  for (; r < few; r += 4u) bad |= compare_some<3, false>(q, r, todo, emask);
-  for (; r < nc; ++r) bad |= compare_some<5, BATCH || INNER>(q, r, todo, emask);
+  for (; r < few; r += 4u) bad |= compare_some<3>(q, r, todo, emask);
+  for (; r < nc; ++r) bad |= compare_some<5>(q, r, todo, emask);
   const bool eq = lane < nc && !((bad >> lane) & 1u);
   const uint32_t row = q[lane].b.z, tag = q[lane].b.w;   // (defined where eq)
   if (!BATCH && !INNER && eq && mode >= AS_JOIN_OUTER_R) atomicOr(P.matched + (row >> 5), 1u << (row & 31u));

@@ -73,51 +73,82 @@ struct Net8 {
   // both are bound by the launch.
   static constexpr uint64_t kThreadFrom = 100000;
   static constexpr uint32_t kThreadBelow = 50;
+  static constexpr uint64_t kThreadMost = 1024;
   static constexpr int kPhases = 6;       // the rings of 24 and 16 words close together
   static constexpr int kShort = 0;
   static constexpr size_t kTabBytes = kLog8Bytes;
   __device__ __forceinline__ static const uint2* red_image() { return g_red8; }
   __device__ __forceinline__ static const uint4* tab_image() { return g_log8; }
-  // One key per thread: Horner's rule over the words of its bytes (realigned to its first one) from the last
-  // to the first, 16 bytes of memory at a time.  The next key's last 16 bytes and the offsets of the one
-  // after it are on their way meanwhile.  mt: lk_fill_masks' rows.
+  // Bytes [s, e) of a key; empty where s >= e
+  struct Bytes {
+    uint64_t s, e;
+  };
+  __device__ __forceinline__ static uint4 chunk(const uint8_t* __restrict__ arena, uint64_t at) {
+    return __ldg(reinterpret_cast<const uint4*>(arena + at));
+  }
+  // the last 16-byte chunk of memory that holds one of them
+  __device__ __forceinline__ static uint4 last_chunk(const uint8_t* __restrict__ arena, const Bytes& k) {
+    return k.e > k.s ? chunk(arena, (k.e - 1) & ~15ull) : make_uint4(0, 0, 0, 0);
+  }
+  // Their signature's components by Horner's rule over words (realigned to byte s) from the last to the first,
+  // 16 bytes of memory at a time; w: their last chunk, mt: lk_fill_masks' rows
+  template <class Cursor>
+  __device__ __forceinline__ static void by_words(uint32_t (&a)[4], const uint8_t* __restrict__ arena, const Bytes& k,
+                                                  uint4 w, const uint4* mt, const Cursor& rc) {
+    a[0] = a[1] = a[2] = a[3] = 0;
+    if (k.e <= k.s) return;
+    const uint32_t sh = 8u * ((uint32_t)k.s & 3u), w0 = ((uint32_t)k.s & 15u) >> 2;
+    const uint4 m = mt[(((uint32_t)k.e - 1u) & 15u) + 1u];
+    w.x &= m.x; w.y &= m.y; w.z &= m.z; w.w &= m.w;
+    uint32_t above = 0;                                // the first word of the chunk above
+    for (uint64_t at = (k.e - 1) & ~15ull;; at -= 16) {
+      const bool first = at <= k.s;
+      const uint4 below = first ? w : chunk(arena, at - 16);
+      const uint32_t from = first ? w0 : 0u;           // the first chunk's words from byte s on
+      gf8_word(__funnelshift_r(w.w, above, sh), a, rc);
+      if (from <= 2u) gf8_word(__funnelshift_r(w.z, w.w, sh), a, rc);
+      if (from <= 1u) gf8_word(__funnelshift_r(w.y, w.z, sh), a, rc);
+      if (from == 0u) gf8_word(__funnelshift_r(w.x, w.y, sh), a, rc);
+      if (first) break;
+      above = w.x;
+      w = below;
+    }
+  }
+  // One key per thread.  The next key's last chunk and the offsets of the one after it are on their way
+  // meanwhile.  A key of more than kThreadMost bytes, of which the relation's four places showed none, is cut
+  // into 32 pieces for the warp: piece p is worth x^(k p) times its own signature, p its first byte's place.
   template <class Cursor>
   __device__ __forceinline__ static void by_thread(const uint8_t* __restrict__ arena, const uint64_t* __restrict__ off,
                                                    uint64_t n, uint64_t* __restrict__ out, const uint4* mt,
-                                                   const Cursor& rc) {
-    struct Key {
-      uint64_t s, e;
-    };
-    auto key = [&](uint64_t i) { return i < n ? Key{__ldg(off + i), __ldg(off + i + 1)} : Key{0, 0}; };
-    auto chunk = [&](uint64_t at) { return __ldg(reinterpret_cast<const uint4*>(arena + at)); };
-    auto last = [&](const Key& k) { return k.e > k.s ? chunk((k.e - 1) & ~15ull) : make_uint4(0, 0, 0, 0); };
+                                                   const uint8_t* lg, const Cursor& rc) {
+    auto key = [&](uint64_t i) { return i < n ? Bytes{__ldg(off + i), __ldg(off + i + 1)} : Bytes{0, 0}; };
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    Key k = key(i), k1 = key(i + stride);
-    uint4 w = last(k);
-    for (; i < n; i += stride) {
-      const Key k2 = key(i + 2 * stride);
-      const uint4 w1 = last(k1);
-      uint32_t a[4] = {0, 0, 0, 0};
-      if (k.e > k.s) {
-        const uint32_t sh = 8u * ((uint32_t)k.s & 3u), w0 = ((uint32_t)k.s & 15u) >> 2;
-        const uint4 m = mt[(((uint32_t)k.e - 1u) & 15u) + 1u];
-        w.x &= m.x; w.y &= m.y; w.z &= m.z; w.w &= m.w;
-        uint32_t above = 0;                            // the first word of the chunk above
-        for (uint64_t at = (k.e - 1) & ~15ull;; at -= 16) {
-          const bool first = at <= k.s;
-          const uint4 below = first ? w : chunk(at - 16);
-          const uint32_t from = first ? w0 : 0u;       // the first chunk's words from the key's first byte on
-          gf8_word(__funnelshift_r(w.w, above, sh), a, rc);
-          if (from <= 2u) gf8_word(__funnelshift_r(w.z, w.w, sh), a, rc);
-          if (from <= 1u) gf8_word(__funnelshift_r(w.y, w.z, sh), a, rc);
-          if (from == 0u) gf8_word(__funnelshift_r(w.x, w.y, sh), a, rc);
-          if (first) break;
-          above = w.x;
-          w = below;
+    Bytes k = key(i), k1 = key(i + stride);
+    uint4 w = last_chunk(arena, k);
+    for (; __any_sync(0xFFFFFFFFu, i < n); i += stride) {
+      const Bytes k2 = key(i + 2 * stride);
+      const uint4 w1 = last_chunk(arena, k1);
+      const bool many = k.e - k.s > kThreadMost;
+      uint32_t a[4];
+      by_words(a, arena, many ? Bytes{0, 0} : k, w, mt, rc);
+      for (uint32_t left = __ballot_sync(0xFFFFFFFFu, many); left; left &= left - 1u) {
+        const int l = __ffs((int)left) - 1;
+        const uint64_t s = __shfl_sync(0xFFFFFFFFu, k.s, l), e = __shfl_sync(0xFFFFFFFFu, k.e, l);
+        const uint64_t each = ((e - s + 15) / 32 + 16) & ~15ull, from = (s & ~15ull) + (threadIdx.x & 31u) * each;
+        const Bytes piece{max(s, from), min(e, from + each)};
+        uint32_t b[4];
+        by_words(b, arena, piece, last_chunk(arena, piece), mt, rc);
+        const uint32_t at = (uint32_t)((piece.s - s) % kOrder8);
+        uint32_t v = times_xe(lg, b[0], at) | times_xe(lg, b[1], 2u * at % kOrder8) << 8 |
+                     times_xe(lg, b[2], 3u * at % kOrder8) << 16 | times_xe(lg, b[3], 4u * at % kOrder8) << 24;
+        v = __reduce_xor_sync(0xFFFFFFFFu, v);
+        if ((int)(threadIdx.x & 31u) == l) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) a[c] = (v >> (8 * c)) & 0xFFu;
         }
       }
-      out[i] = (uint64_t)(a[0] | (a[1] << 8) | (a[2] << 16) | (a[3] << 24));
+      if (i < n) out[i] = (uint64_t)(a[0] | (a[1] << 8) | (a[2] << 16) | (a[3] << 24));
       k = k1;
       k1 = k2;
       w = w1;

@@ -229,7 +229,8 @@ __device__ __forceinline__ uint32_t xs3_component(const uint32_t (&c3)[16], cons
 }
 
 // The longest of eight neighbouring keys, the mean of that over four places of the
-// relation, to 8 bytes (whole warp): what a thread per key waits for.
+// relation, to 8 bytes, or the mean of all keys if that is more (whole warp): what
+// a thread per key waits for.
 __device__ __forceinline__ uint32_t lk_longest_near(const uint64_t* __restrict__ off, uint64_t n) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t first = n / 8 * (2 * (lane >> 3) + 1), i = min(first / 8 * 8 + (lane & 7u), n - 1);
@@ -237,7 +238,8 @@ __device__ __forceinline__ uint32_t lk_longest_near(const uint64_t* __restrict__
   uint32_t longest = (uint32_t)min(len, (uint64_t)0x10000000u);
 #pragma unroll
   for (int d = 1; d < 8; d <<= 1) longest = max(longest, __shfl_xor_sync(kFull, longest, d));
-  return __reduce_add_sync(kFull, longest >> 3) >> 2;            // each place's eight times
+  const uint32_t mean = (uint32_t)min((__ldg(off + n) - __ldg(off)) / n, (uint64_t)0x10000000u);
+  return max(__reduce_add_sync(kFull, longest >> 3) >> 2, mean); // (each place's eight times)
 }
 
 // A lane's key in the current group.
@@ -936,7 +938,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   if constexpr (Net::kThreadBelow > 0) {
     if (by_thread) {
       cp_async_wait_all();
-      Net::by_thread(arena, off, n, sig_out, mt, rc);
+      Net::by_thread(arena, off, n, sig_out, mt, tab, rc);
       return;
     }
   }

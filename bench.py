@@ -912,7 +912,7 @@ def run_gpu(args):
 
 
 # revision of each kernel's code; profiles/traffic.json holds counters per revision
-KERNEL_REVS = {"sig_key_kernel": "v5", "build_kernel": "v8", "verify_kernel": "v19", "sig_key_kernel+build": "v3"}
+KERNEL_REVS = {"sig_key_kernel": "v6", "build_kernel": "v8", "verify_kernel": "v20", "sig_key_kernel+build": "v4"}
 KERNEL_NAMES = {"sig_R": "sig_key_kernel", "sig_S": "sig_key_kernel", "build": "build_kernel",
                 "verify": "verify_kernel", "sig_build_R": "sig_key_kernel+build"}
 

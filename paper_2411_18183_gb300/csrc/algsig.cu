@@ -460,8 +460,8 @@ struct CandQueue {
   uint64_t ids[kVDrain];     // the ids of the candidates being verified
   uint32_t matched[kVOpen];  // a bit per S row of the open groups: a candidate was verified
 };
-// Chunks of each lane in flight: with 4 blocks of 64 registers two fit without spills (large join, blocks x
-// chunks: 4 x 2 2.83 ms, 3 x 4 2.85, 3 x 3 2.96, 4 x 3 3.02, 4 x 1 3.11)
+// Chunks of each lane in flight: with 4 blocks of 64 registers two fit (the output modes' kernel spills 28
+// bytes; large join, blocks x chunks: 4 x 2 2.83 ms, 3 x 4 2.85, 3 x 3 2.96, 4 x 3 3.02, 4 x 1 3.11)
 constexpr int kVAhead = 2;
 // Longest key compared by eight lanes: the whole warp's 512 bytes in a row take fewer requests (400k
 // candidates of 2-8 KB: 821 us with eight lanes, 750 us with the warp, when first compared) and are left where the

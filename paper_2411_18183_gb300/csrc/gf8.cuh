@@ -68,7 +68,7 @@ __device__ __forceinline__ void gf8_word(uint32_t w, uint32_t (&a)[4], const Cur
 
 struct Net8 {
   // Short keys, of which the signature kernel's work per key is more than a thread's work per byte: us, one key
-  // per thread / staged, 4M keys of 16, 32, 48, 64 bytes 68 / 155, 97 / 155, 129 / 157, 161 / 157; half to one
+  // per thread / staged, 4M keys of 16, 32, 48, 64 bytes 69 / 155, 99 / 155, 131 / 157, 161 / 157; half to one
   // and a half times 32, 40, 48 bytes 156 / 160, 177 / 160, 203 / 161.  Up to a key or so per thread of the device
   // both are bound by the launch.
   static constexpr uint64_t kThreadFrom = 100000;

@@ -31,8 +31,9 @@
 // per key.
 //
 // Scheduling.  Each warp owns a range of keys with an equal share of the work
-// (key bytes + a fixed cost per key) and walks it in windows of kLKWin keys.  A
-// window's keys are sorted by length, and the warp computes them in groups of
+// (key bytes + a fixed cost per key; keys cut to a length come in bands, and keys'
+// blocks are shared by their bytes) and walks it in windows of kLKWin keys.  A
+// window's keys are sorted by length (unless all are short), and the warp computes them in groups of
 // 32 consecutive sorted keys, one key per lane, so the lanes of a group have
 // (nearly) the same amount of work.  Keys are taken in 32-byte blocks from the
 // last to the first; the lanes of a group whose keys are shorter start later,

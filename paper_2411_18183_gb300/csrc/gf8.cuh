@@ -115,7 +115,7 @@ struct Net8 {
     }
   }
   // One key per thread.  The next key's last chunk and the offsets of the one after it are on their way
-  // meanwhile.  A key of more than kThreadMost bytes, of which the relation's four places showed none, is cut
+  // meanwhile.  A key of more than kThreadMost bytes, of which the places looked at showed none, is cut
   // into 32 pieces for the warp: piece p is worth x^(k p) times its own signature, p its first byte's place.
   template <class Cursor>
   __device__ __forceinline__ static void by_thread(const uint8_t* __restrict__ arena, const uint64_t* __restrict__ off,

@@ -511,7 +511,8 @@ __global__ void __launch_bounds__(kPRestThreads, 1) prefix_rest_kernel(const uin
                                                                     uint64_t* __restrict__ out) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint4 emask[17];
-  if (by_items(off, n, block_bytes)) {
+  __shared__ LKLook look;
+  if (by_items(look, off, n, block_bytes)) {
     if (pref_off[n] != n) prefix_sums(smem, off, n, block_bytes, pref_off, out);   // (else no key has two blocks)
   } else if (block_bytes < 32) {
     prefix_by_warp(smem, emask, arena, off, n, block_bytes, pref_off, out);

@@ -129,6 +129,7 @@ constexpr uint32_t kLKUnsorted = kLKShort, kLKAsk = 64;
 // after them two warps side by side.  Then the constant-multiply tables, the
 // byte masks and the warps' windows.
 constexpr size_t kSmemLKMasks = 17 * 16;
+constexpr size_t kSmemLKLook = 48;                    // an LKLook (not static: dynamic shared memory starts at 0x400)
 constexpr uint32_t kLKStageBytes = 32 * kLKPitch;     // from one stage of a warp to the next
 __host__ __device__ constexpr size_t lk_line_bytes(int warps, int depth) {
   const int stages = depth / kLKStep, beside = 8 / stages;
@@ -136,7 +137,7 @@ __host__ __device__ constexpr size_t lk_line_bytes(int warps, int depth) {
 }
 template <class Net>
 __host__ __device__ constexpr size_t lk_smem_bytes(int warps, int depth) {
-  return lk_line_bytes(warps, depth) + Net::kTabBytes + kSmemLKMasks + (size_t)warps * sizeof(LKWarp);
+  return lk_line_bytes(warps, depth) + Net::kTabBytes + kSmemLKMasks + kSmemLKLook + (size_t)warps * sizeof(LKWarp);
 }
 // byte offset of a warp's first stage
 template <int kStages>
@@ -229,18 +230,35 @@ __device__ __forceinline__ uint32_t xs3_component(const uint32_t (&c3)[16], cons
   return red32(acc, rc);
 }
 
-// The longest of eight neighbouring keys, the mean of that over four places of the
-// relation, to 8 bytes, or the mean of all keys if that is more (whole warp): what
-// a thread per key waits for.
-__device__ __forceinline__ uint32_t lk_longest_near(const uint64_t* __restrict__ off, uint64_t n) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t first = n / 8 * (2 * (lane >> 3) + 1), i = min(first / 8 * 8 + (lane & 7u), n - 1);
-  const uint64_t len = __ldg(off + i + 1) - __ldg(off + i);
-  uint32_t longest = (uint32_t)min(len, (uint64_t)0x10000000u);
+// The longest of 32 neighbouring keys, the mean of that over eight places of the
+// relation, or the mean of all keys if that is more: what a thread per key waits
+// for.  lk_look, by the whole block, of nine warps or more, puts together in shared
+// memory what lk_seen gives after a barrier: a warp looks at a place.  (Of eight keys
+// at four places it missed the long ones of a mixed relation often enough: 500k
+// keys of 24 bytes, a tenth of 264, byte symbols 81 us by threads, 27 staged; with
+// every warp looking at all eight places a call took 1 us longer.)
+constexpr uint32_t kLKPlaces = 8;
+struct LKLook {
+  uint32_t longest[kLKPlaces], mean;
+};
+static_assert(sizeof(LKLook) <= kSmemLKLook, "the place for it");
+__device__ __forceinline__ void lk_look(LKLook& l, const uint64_t* __restrict__ off, uint64_t n) {
+  const uint32_t lane = threadIdx.x & 31u, p = threadIdx.x >> 5;
+  if (p > kLKPlaces) return;                          // warp-uniform
+  if (p == kLKPlaces) {
+    if (lane == 0) l.mean = (uint32_t)min((__ldg(off + n) - __ldg(off)) / n, (uint64_t)0x10000000u);
+    return;
+  }
+  const uint64_t i = min(n / (2 * kLKPlaces) * (2 * p + 1) / 32 * 32 + lane, n - 1);
+  const uint32_t len = (uint32_t)min(__ldg(off + i + 1) - __ldg(off + i), (uint64_t)0x10000000u);
+  const uint32_t longest = __reduce_max_sync(kFull, len);
+  if (lane == 0) l.longest[p] = longest;
+}
+__device__ __forceinline__ uint32_t lk_seen(const LKLook& l) {
+  uint32_t sum = 0;
 #pragma unroll
-  for (int d = 1; d < 8; d <<= 1) longest = max(longest, __shfl_xor_sync(kFull, longest, d));
-  const uint32_t mean = (uint32_t)min((__ldg(off + n) - __ldg(off)) / n, (uint64_t)0x10000000u);
-  return max(__reduce_add_sync(kFull, longest >> 3) >> 2, mean); // (each place's eight times)
+  for (uint32_t p = 0; p < kLKPlaces; ++p) sum += l.longest[p] / kLKPlaces;
+  return max(sum, l.mean);
 }
 
 // A lane's key in the current group.
@@ -518,7 +536,7 @@ __device__ __forceinline__ void lk_short_blocks(uint32_t (&st)[kLKState], const 
 // components.  A net names its shared-memory tables and has the digit rings and
 // finish of the quotient form; kShort: groups of at most this many blocks take
 // the remainder form; kThreadBelow: relations of more than kThreadFrom keys shorter
-// than this (lk_longest_near) are signed by Net::by_thread, one key per thread.
+// than this (lk_seen) are signed by Net::by_thread, one key per thread.
 template <int NCOMP>
 struct Net16 : QNet<NCOMP> {
   static constexpr int kComponents = NCOMP;
@@ -735,9 +753,11 @@ struct LKItems {
 // 30 / 30, 21 / 21), but for so few that they do not fill it either.
 // A warp per key (blocks of 16): 500k of 190 bytes 260 / 299, of 260 404 / 350; 16k of
 // 96 bytes 19 / 17, 60k 27 / 40.
-__device__ __forceinline__ bool by_items(const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
+__device__ __forceinline__ bool by_items(LKLook& look, const uint64_t* __restrict__ off, uint64_t n, uint32_t block) {
   if (block < 32u) return n > 20000u && __ldg(off + n) - __ldg(off) < 192u * n;
-  return lk_longest_near(off, n) >= (n >= (1u << 15) && n <= 5u << 15 ? 280u : 180u);
+  lk_look(look, off, n);
+  __syncthreads();
+  return lk_seen(look) >= (n >= (1u << 15) && n <= 5u << 15 ? 280u : 180u);
 }
 
 // A warp's items [lo, hi), whole groups of 32 but at the end, and a key at or
@@ -876,17 +896,18 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
                                                                 const LKSecond second = LKSecond()) {
   constexpr bool BATCH = OF == LKOf::kBatchRows, ITEMS = OF == LKOf::kItems, CAPPED = OF == LKOf::kPrefixes;
   const uint64_t cap_len = CAPPED ? cap : ~0ull;
-  if constexpr (ITEMS) {
-    if (!by_items(off, n, items.block)) return;
-    asm volatile("griddepcontrol.launch_dependents;");   // prefix_rest_kernel, which waits where it has to
-  }
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int kStages = kLKDepth / kLKStep;
   static_assert(kLKDepth % kLKStep == 0 && kStages >= 2 && (kStages == 3 || 8 % kStages == 0), "whole steps in flight");
   constexpr size_t kLines = lk_line_bytes(kLKWarps, kLKDepth);
   uint8_t* tab = smem + kLines;
   uint4* mt = reinterpret_cast<uint4*>(smem + kLines + Net::kTabBytes);
-  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kLines + Net::kTabBytes + kSmemLKMasks);
+  LKLook& look = *reinterpret_cast<LKLook*>(smem + kLines + Net::kTabBytes + kSmemLKMasks);
+  LKWarp* warps = reinterpret_cast<LKWarp*>(smem + kLines + Net::kTabBytes + kSmemLKMasks + kSmemLKLook);
+  if constexpr (ITEMS) {
+    if (!by_items(look, off, n, items.block)) return;
+    asm volatile("griddepcontrol.launch_dependents;");   // prefix_rest_kernel, which waits where it has to
+  }
   const int wib = threadIdx.x >> 5;
   const uint32_t lane = threadIdx.x & 31u;
   LKWarp& W = warps[wib];
@@ -918,8 +939,9 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
     else
       lk_warp_range<BATCH, kLKWarps>(J, nj, s_side, off, n, warp, nwarps, &k_lo, &k_hi);
   }
-  bool by_thread = false;
-  if constexpr (Net::kThreadBelow > 0) by_thread = n > Net::kThreadFrom && lk_longest_near(off, n) < Net::kThreadBelow;
+  if constexpr (Net::kThreadBelow > 0) {
+    if (n > Net::kThreadFrom) lk_look(look, off, n);
+  }
   uint64_t wb = k_lo, wa = 0;                       // the current window: first key, its row, key count
   uint32_t wn = k_lo < k_hi ? lk_window<BATCH>(J, nj, s_side, k_lo, k_hi, most, &wa) : 0u;
   if (wn && !ITEMS) lk_prefetch_window(W, off, wa, wa + wn);
@@ -937,7 +959,7 @@ __global__ void __launch_bounds__(32 * kLKWarps, 1) sig_key_kernel(const uint8_t
   __syncthreads();
   const LKCursor<AT400> rc(smem);
   if constexpr (Net::kThreadBelow > 0) {
-    if (by_thread) {
+    if (n > Net::kThreadFrom && lk_seen(look) < Net::kThreadBelow) {
       cp_async_wait_all();
       Net::by_thread(arena, off, n, sig_out, mt, tab, rc);
       return;
